@@ -446,9 +446,8 @@ int dd_sap_smooth(dd_op_t opp, const dd_sap_params *p, const void *b, void *x, i
   // them, e.g. when this allocation fails, every phase forms b - D x)
   cudaStream_t st = (cudaStream_t)stream;
   const Geom &g = op->lat->g;
-  const size_t fb = (size_t)g.V * spinor_site_bytes(op->fp.prec);
   void *aux = nullptr;
-  if (cudaMallocAsync(&aux, 2 * (size_t)nrhs * fb, st) != cudaSuccess) {
+  if (cudaMallocAsync(&aux, (size_t)nrhs * sap_work_bytes(g, op->fp.prec, p->x_is_zero), st) != cudaSuccess) {
     cudaGetLastError();
     aux = nullptr;
   }
@@ -480,7 +479,7 @@ int dd_sap_smooth_multi(int nops, const dd_op_t *ops, const int *nrhs, const dd_
       rp.out[rp.n] = (char *)x[k] + r * fb;
     }
     lats[k] = SapLattice{op->lat->g, op->fp, nrhs[k]};
-    aux_bytes += 2 * (size_t)nrhs[k] * fb;
+    aux_bytes += (size_t)nrhs[k] * sap_work_bytes(op->lat->g, op->fp.prec, p->x_is_zero);
   }
   // work fields of the incremental colour residual, stream-ordered
   cudaStream_t st = (cudaStream_t)stream;
@@ -489,13 +488,14 @@ int dd_sap_smooth_multi(int nops, const dd_op_t *ops, const int *nrhs, const dd_
     cudaGetLastError();
     aux = nullptr;
   }
-  AuxPtrs ax{};
+  SapWork ax;
   for (int k = 0, i = 0; aux && k < nops; k++) {
     const size_t fb = (size_t)lats[k].g.V * spinor_site_bytes(lats[k].f.prec);
     for (int r = 0; r < nrhs[k]; r++, i++) {
       ax.e[i] = aux;
       ax.r[i] = aux + fb;
-      aux += 2 * fb;
+      if (sap_r0_bytes(lats[k].g, lats[k].f.prec, p->x_is_zero)) ax.r0[i] = aux + 2 * fb;
+      aux += sap_work_bytes(lats[k].g, lats[k].f.prec, p->x_is_zero);
     }
   }
   int rc = launch_sap_lattices(lats, nops, *p, rp, st, ax.e[0] ? &ax : nullptr);

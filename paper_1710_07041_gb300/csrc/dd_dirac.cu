@@ -146,6 +146,42 @@ __global__ void __launch_bounds__(TPB, MINB) k_dirac(Geom g_in, const void *__re
   store_spinor<SO, C>(p.out[r], g, b, s, acc);
 }
 
+// r = b - D x, r as an FP32 field (the first iterate's residual of the
+// Schwarz smoother; the arithmetic of k_dirac, the result not rounded to the
+// storage of x and b)
+template <typename S, int SHAPE>
+__global__ void __launch_bounds__(128, 5) k_residual(Geom g_in, const void *__restrict__ links,
+                                                     const void *__restrict__ clov, const RhsPtrs px,
+                                                     const RhsPtrs pb) {
+  using C = typename Store<S>::comp_t;
+  const Geom g = block_shape<SHAPE>(g_in);
+  const int nrhs = px.n;
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= g.V * nrhs) return;
+  const long long site = t / nrhs;
+  const int r = (int)(t - site * nrhs);
+  const int b = (int)(site / g.Vb), s = (int)(site - (long long)b * g.Vb);
+  const Site st = decode(g, b, s);
+  Spinor<C> x, acc;
+  load_spinor<S, C>(px.in[r], g, b, s, x);
+  clover_apply_no_l1<S, C>(clov, g.Vb, b, s, x, acc);
+  dirac_dir<0, S, C>(g, st, links, px.in[r], acc);
+  dirac_dir<1, S, C>(g, st, links, px.in[r], acc);
+  dirac_dir<2, S, C>(g, st, links, px.in[r], acc);
+  dirac_dir<3, S, C>(g, st, links, px.in[r], acc);
+  load_spinor<S, C>(pb.in[r], g, b, s, x);
+#pragma unroll
+  for (int i = 0; i < 12; i++) acc.c[i] = {x.c[i].re - acc.c[i].re, x.c[i].im - acc.c[i].im};
+  store_spinor<float, C>(px.out[r], g, b, s, acc);
+}
+template <typename S>
+int residual_t(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, cudaStream_t st) {
+  const unsigned grid = (unsigned)((g.V * x.n + 127) / 128);
+  if (shape_of(g) == 1) k_residual<S, 1><<<grid, 128, 0, st>>>(g, f.links, f.clov, x, b);
+  else k_residual<S, 0><<<grid, 128, 0, st>>>(g, f.links, f.clov, x, b);
+  return launched("k_residual");
+}
+
 template <typename S, int TPB, int MINB, bool NL1, typename SO = S>
 int dirac_v(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st) {
   long long n = g.V * p.n;
@@ -219,6 +255,17 @@ int launch_dirac(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_
     case DD_F16N: return dirac_t<hn16>(g, f, p, st);
   }
   set_error("apply_D: precision %d not available", f.prec);
+  return DD_EINVAL;
+}
+
+int launch_residual(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, cudaStream_t st) {
+  switch (f.prec) {
+    case DD_F32: return residual_t<float>(g, f, x, b, st);
+    case DD_F16: return residual_t<__half>(g, f, x, b, st);
+    case DD_BF16: return residual_t<__nv_bfloat16>(g, f, x, b, st);
+    case DD_F16N: return residual_t<hn16>(g, f, x, b, st);
+  }
+  set_error("residual: precision %d not available", f.prec);
   return DD_EINVAL;
 }
 

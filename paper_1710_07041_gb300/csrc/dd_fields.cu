@@ -439,16 +439,33 @@ int launch_pack_links(const Geom &g, int prec, const double *canon, void *out, i
   return launched("k_pack_links");
 }
 
+// canonical FP64 links -> the packed kernel's tiles (OpFields::links_full
+// where paired_links holds): [b][36][site pair] {re, re, im, im} of -U/2, one
+// thread per entry of a pair of neighbouring sites (pairs fastest: whole
+// lines written)
+template <typename P> __global__ void k_pack_links_paired(Geom g, const double2 *__restrict__ canon, P *out) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= g.V * 18) return;
+  const long long bi = t / g.Vh;
+  const int j = (int)(t - bi * g.Vh), b = (int)(bi / 36), i = (int)(bi - 36LL * b);
+  const double2 va = canon[canonical_index(g, b, 2 * j) * 36 + i], vb = canon[canonical_index(g, b, 2 * j + 1) * 36 + i];
+  P *q = out + 2 * t;
+  q[0] = to_pair<P, double>(-0.5 * va.x, -0.5 * vb.x);
+  q[1] = to_pair<P, double>(-0.5 * va.y, -0.5 * vb.y);
+}
+
 int launch_pack_links_full(const Geom &g, int prec, const double *canon, void *out, cudaStream_t st) {
   const double2 *c = (const double2 *)canon;
+  auto pack = [&](auto *p) {
+    using P = std::remove_pointer_t<decltype(p)>;
+    if (paired_links(g, prec)) k_pack_links_paired<P><<<grid_for(g.V * 18), TPB, 0, st>>>(g, c, p);
+    else k_pack_links<P, 9, false><<<grid_for(g.V), TPB, 0, st>>>(g, c, p, nullptr);
+  };
   switch (prec) {
-    case DD_F64: k_pack_links<double2, 9, false><<<grid_for(g.V), TPB, 0, st>>>(g, c, (double2 *)out, nullptr); break;
-    case DD_F32: k_pack_links<float2, 9, false><<<grid_for(g.V), TPB, 0, st>>>(g, c, (float2 *)out, nullptr); break;
+    case DD_F32: pack((float2 *)out); break;
     case DD_F16:
-    case DD_F16N: k_pack_links<__half2, 9, false><<<grid_for(g.V), TPB, 0, st>>>(g, c, (__half2 *)out, nullptr); break;
-    case DD_BF16:
-      k_pack_links<__nv_bfloat162, 9, false><<<grid_for(g.V), TPB, 0, st>>>(g, c, (__nv_bfloat162 *)out, nullptr);
-      break;
+    case DD_F16N: pack((__half2 *)out); break;
+    case DD_BF16: pack((__nv_bfloat162 *)out); break;
     default: set_error("bad precision %d", prec); return DD_EINVAL;
   }
   return launched("k_pack_links");

@@ -563,6 +563,19 @@ __device__ __forceinline__ void load_link(const void *links, const Geom &g, int 
   if constexpr (LP == 6) su3_third_row(u);
 }
 
+// Entry i (0..35) of site s in a links tile of the packed layout (see
+// OpFields::links_full; n sites): the link times -1/2 of two neighbouring
+// sites interleaved {re, re, im, im}.
+__device__ __forceinline__ float real_of(float v) { return v; }
+__device__ __forceinline__ float real_of(__half v) { return __half2float(v); }
+__device__ __forceinline__ float real_of(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ double real_of(double v) { return v; }
+template <typename C, typename P> __device__ __forceinline__ cpx<C> paired_link_entry(const P *tile, int n, int i, int s) {
+  using R = std::remove_const_t<std::remove_reference_t<decltype(tile->x)>>;
+  const R *e = (const R *)tile + 2 * ((size_t)i * n + (s & ~1)) + (s & 1);
+  return {(C)-2 * (C)real_of(e[0]), (C)-2 * (C)real_of(e[2])};
+}
+
 template <typename C> __device__ __forceinline__ cpx<C> cmul(cpx<C> a, cpx<C> b) {
   return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
 }
@@ -793,6 +806,10 @@ struct Gauge {
   int refs;
 };
 
+// the Schwarz kernel of this block shape and storage works on packed site
+// pairs (dd_sap_pair.cuh) and reads links_full in their order
+inline bool paired_links(const Geom &g, int prec) { return shape_of(g) != 0 && prec != DD_F64; }
+
 // Operator fields in one storage precision.
 struct OpFields {
   int prec = -1;
@@ -800,7 +817,9 @@ struct OpFields {
   // [nblocks][36][Vb] pairs, every entry: the Schwarz kernel rebuilds no rows
   // (its block solve reads each link about ten times per phase from L1 or
   // shared memory, where the rebuild would cost more issue slots than the
-  // bytes it saves); the same array as `links` for FP64
+  // bytes it saves); the same array as `links` for FP64. Where paired_links
+  // holds: the links times -1/2 (exact), the reals of sites 2j and 2j + 1
+  // interleaved {re, re, im, im} (the packed kernel's operand order)
   void *links_full = nullptr;
   void *clov = nullptr;   // A, chunked tiles of 36 pairs x Vb sites per block (clover_slot)
   void *cinv = nullptr;   // A^-1 on even sites, chunked tiles of 36 pairs x Vh sites
@@ -847,8 +866,14 @@ RhsPtrs contiguous(const void *in, void *out, int nrhs, size_t field_bytes);
 // residual after its own latest solve (odd sites; the even-site residual of
 // an even-odd block solve is zero).
 struct AuxPtrs {
-  void *e[MAX_RHS];
-  void *r[MAX_RHS];
+  void *e[MAX_RHS] = {};
+  void *r[MAX_RHS] = {};
+};
+// What a smoother call is given: the work fields its kernels take, and FP32
+// fields for b - D x of a given first iterate (x_is_zero = 0; packed links
+// only, may be null: then every phase forms b - D x).
+struct SapWork : AuxPtrs {
+  void *r0[MAX_RHS] = {};
 };
 
 // --------------------------------------------------------- kernel launchers
@@ -868,6 +893,8 @@ int launch_build_clover(const Geom &g, const double *links_canon, double c_sw, d
 int launch_convert_clover(int prec, const double *in, void *out, size_t ntiles, int n, cudaStream_t st);
 int launch_dirac(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st);
 int launch_dirac(const Geom &g, const OpFields &f, const void *in, void *out, int nrhs, cudaStream_t st);
+// r = b - D x with r as FP32 fields: x.in = x, x.out = r, b.in = b (32- and 16-bit storage)
+int launch_residual(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, cudaStream_t st);
 // y = D x with double-float fields (f = op->fdf) and double-float inputs p.in
 // (FP64 fields split by launch_split_pairs), FP64 outputs p.out
 int launch_dirac_df(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st);
@@ -898,15 +925,22 @@ struct SapLattice {
   int nrhs;
 };
 int launch_sap_lattices(const SapLattice *lats, int nlat, const dd_sap_params &sp, const RhsPtrs &p,
-                        cudaStream_t st, const AuxPtrs *aux);
+                        cudaStream_t st, const SapWork *aux);
 
 // aux (may be null): work fields for the incremental colour residual, one
 // pair per right-hand side of p; without them every phase recomputes
 // r = b - D x from x
 int launch_sap(const Geom &g, const OpFields &f, const dd_sap_params &sp, const RhsPtrs &p, cudaStream_t st,
-               const AuxPtrs *aux = nullptr);
-// nrhs contiguous fields b, x; aux_base (may be null): 2 x nrhs contiguous
-// work fields (e of every right-hand side, then r)
+               const SapWork *aux = nullptr);
+// nrhs contiguous fields b, x; aux_base (may be null): sap_work_bytes per
+// right-hand side of contiguous work fields (e of every right-hand side, then
+// r, then r0 where there is one)
+inline size_t sap_r0_bytes(const Geom &g, int prec, int x_is_zero) {
+  return !x_is_zero && paired_links(g, prec) ? (size_t)g.V * spinor_site_bytes(DD_F32) : 0;
+}
+inline size_t sap_work_bytes(const Geom &g, int prec, int x_is_zero) {
+  return 2 * (size_t)g.V * spinor_site_bytes(prec) + sap_r0_bytes(g, prec, x_is_zero);
+}
 int launch_sap(const Geom &g, const OpFields &f, const dd_sap_params &sp, const void *b, void *x, int nrhs,
                cudaStream_t st, void *aux_base = nullptr);
 // DD_OK, or DD_ETIMEOUT if a bounded device wait has expired since the last

@@ -659,7 +659,7 @@ __global__ void k_add_scale(const float4 *a, const float4 *b, float4 *y, float s
 // ---------------------------------------------------------------- MgWork
 MgWork::~MgWork() {
   for (auto &kv : graphs) cudaGraphExecDestroy(kv.second.first);
-  void *p[] = {Vc, w, w2, cb, ce, xf, rf, tf, tin, tout, partial, pnorm, st};
+  void *p[] = {Vc, w, w2, cb, ce, xf, rf, tf, tin, tout, se, sr, partial, pnorm, st};
   for (void *q : p)
     if (q) cudaFree(q);
 }
@@ -675,6 +675,7 @@ int MgWork::init(const Mg *mg) {
             cudaMalloc(&ce, sizeof(float2) * nc) == cudaSuccess && cudaMalloc(&xf, f32) == cudaSuccess &&
             cudaMalloc(&rf, f32) == cudaSuccess && cudaMalloc(&tf, f32) == cudaSuccess &&
             cudaMalloc(&tin, fp) == cudaSuccess && cudaMalloc(&tout, fp) == cudaSuccess &&
+            cudaMalloc(&se, fp) == cudaSuccess && cudaMalloc(&sr, fp) == cudaSuccess &&
             cudaMalloc(&partial, sizeof(float2) * cg_chunks(nc) * 65) == cudaSuccess &&
             cudaMalloc(&pnorm, sizeof(float) * cg_partials(nc)) == cudaSuccess &&
             cudaMalloc(&st, sizeof(CgState)) == cudaSuccess;
@@ -688,7 +689,7 @@ int MgWork::init(const Mg *mg) {
 
 size_t MgWork::bytes(const Geom &g, int prec, int N, int kmax) {
   const size_t nc = (size_t)g.nblocks * 2 * N;
-  return sizeof(float2) * nc * (kmax + 5) + (size_t)g.V * 24 * (4 * 3 + 2 * real_bytes(prec)) +
+  return sizeof(float2) * nc * (kmax + 5) + (size_t)g.V * 24 * (4 * 3 + 4 * real_bytes(prec)) +
          sizeof(float2) * cg_chunks(nc) * 65 + sizeof(float) * cg_partials(nc) + sizeof(CgState);
 }
 
@@ -783,11 +784,16 @@ static int mg_enqueue(const Mg *mg, MgWork &W, const float *r, float *x, cudaStr
   if ((rc = mg_sub(r, W.tf, W.rf, nf, st))) return rc;   // r1 = r - D x
   dd_sap_params sp = mg->p.smoother;
   sp.x_is_zero = 1;
+  SapWork ax;   // the smoother's work fields (corrections, block residuals)
+  ax.e[0] = W.se;
+  ax.r[0] = W.sr;
+  const size_t fb = (size_t)g.V * spinor_site_bytes(op->prec);
+  auto smooth = [&](const void *b, void *x) { return launch_sap(g, op->fp, sp, contiguous(b, x, 1, fb), st, &ax); };
   if (op->prec == DD_F32) {
-    if ((rc = launch_sap(g, op->fp, sp, W.rf, W.tf, 1, st))) return rc;
+    if ((rc = smooth(W.rf, W.tf))) return rc;
   } else {
     if ((rc = launch_convert_field(g, DD_F32, W.rf, op->prec, W.tin, 1, 1.0, st))) return rc;
-    if ((rc = launch_sap(g, op->fp, sp, W.tin, W.tout, 1, st))) return rc;
+    if ((rc = smooth(W.tin, W.tout))) return rc;
     if ((rc = launch_convert_field(g, op->prec, W.tout, DD_F32, W.tf, 1, 1.0, st))) return rc;
   }
   return mg_add_scale(W.xf, W.tf, x, scale, nf, st);
@@ -887,7 +893,7 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
   const size_t fs = (size_t)g.V * 24;
   const int N = mg->N;
   double *canon = nullptr, *nrm = nullptr;
-  void *pin = nullptr, *pout = nullptr;
+  void *pin = nullptr, *pout = nullptr, *aux = nullptr;
   DD_CUDA(cudaMalloc(&canon, fs * 8));
   int rc = DD_OK;
   Blas bl;
@@ -900,7 +906,8 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
   }
   if (cudaMalloc(&nrm, sizeof(double)) != cudaSuccess) rc = DD_ENOMEM;
   if (cudaMalloc(&pin, fs * real_bytes(op->prec)) != cudaSuccess ||
-      cudaMalloc(&pout, fs * real_bytes(op->prec)) != cudaSuccess)
+      cudaMalloc(&pout, fs * real_bytes(op->prec)) != cudaSuccess ||
+      cudaMalloc(&aux, sap_work_bytes(g, op->prec, 1)) != cudaSuccess)
     rc = DD_ENOMEM;
   const double sigma = std::sqrt(24.0 * (double)g.V);
   for (int k = 0; k < N && rc == DD_OK; k++) {
@@ -912,7 +919,7 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
     for (int it = 0; it < mg->p.setup_iters && rc == DD_OK; it++) {
       dd_sap_params sp = mg->p.smoother;
       sp.x_is_zero = 1;
-      if ((rc = launch_sap(g, op->fp, sp, pin, pout, 1, st))) break;
+      if ((rc = launch_sap(g, op->fp, sp, pin, pout, 1, st, aux))) break;
       if ((rc = launch_unpack(g, op->prec, pout, canon, 1, 1.0, st))) break;
       if ((rc = bl.norm2(canon, fs / 2, nrm, st))) break;
       double n2 = 0;
@@ -928,6 +935,7 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
   cudaFree(nrm);
   cudaFree(pin);
   cudaFree(pout);
+  cudaFree(aux);
   if (rc) return rc;
   k_orthonormalise<<<2 * g.nblocks, MG_TPB, 0, st>>>(g, mg->V, fs, N);
   if ((rc = launched("k_orthonormalise"))) return rc;

@@ -148,7 +148,7 @@ extern "C" int dd_solve_noalloc(dd_op_t opp, const dd_solve_params *p, const dou
   double *x = cv.take<double>(f64), *b = cv.take<double>(f64), *w = cv.take<double>(f64);
   double *canon = cv.take<double>(f64);
   void *tin = cv.take<char>(fp), *tout = cv.take<char>(fp), *zt = cv.take<char>(fz);
-  AuxPtrs ax{};   // the smoother's work fields (corrections, block residuals)
+  SapWork ax;   // the smoother's work fields (corrections, block residuals)
   ax.e[0] = cv.take<char>(fp);
   ax.r[0] = cv.take<char>(fp);
   const size_t vstride = f64_al / 16;   // complex entries between basis vectors

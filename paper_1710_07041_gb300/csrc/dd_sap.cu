@@ -83,15 +83,15 @@ unsigned *sap_timeout_counter() {
 }
 
 int sap_run_f64(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp,
-                const AuxPtrs *ax, cudaStream_t st);
+                const SapWork *ax, cudaStream_t st);
 int sap_run_f32(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp,
-                const AuxPtrs *ax, cudaStream_t st);
+                const SapWork *ax, cudaStream_t st);
 int sap_run_f16(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp,
-                const AuxPtrs *ax, cudaStream_t st);
+                const SapWork *ax, cudaStream_t st);
 int sap_run_f16n(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp,
-                 const AuxPtrs *ax, cudaStream_t st);
+                 const SapWork *ax, cudaStream_t st);
 int sap_run_bf16(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp,
-                const AuxPtrs *ax, cudaStream_t st);
+                const SapWork *ax, cudaStream_t st);
 
 namespace {
 // Self-test of the staging handshake: one 16-byte bulk copy tracked by an
@@ -143,7 +143,7 @@ struct GraphCache {
 // never destroyed: no CUDA call runs at process exit
 static GraphCache &g_graphs = *new GraphCache;
 
-int sap_launch_as_graph(const std::string &key, int variant, int nkernels, const RhsPtrs &rp, const AuxPtrs *ax,
+int sap_launch_as_graph(const std::string &key, int variant, int nkernels, const RhsPtrs &rp, const SapWork *ax,
                         const std::function<int()> &enqueue, cudaStream_t st) {
   const char *env = getenv("DD_SAP_GRAPHS");
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -229,10 +229,12 @@ int launch_sap(const Geom &g, const OpFields &f, const dd_sap_params &p, const v
   const size_t fb = (size_t)g.V * spinor_site_bytes(f.prec);
   for (int r0 = 0; r0 < nrhs; r0 += MAX_RHS) {
     int n = nrhs - r0 < MAX_RHS ? nrhs - r0 : MAX_RHS;
-    AuxPtrs ax{};
+    SapWork ax;
     for (int i = 0; aux_base && i < n; i++) {
       ax.e[i] = (char *)aux_base + (size_t)(r0 + i) * fb;
       ax.r[i] = (char *)aux_base + (size_t)(nrhs + r0 + i) * fb;
+      if (const size_t rb = sap_r0_bytes(g, f.prec, p.x_is_zero))
+        ax.r0[i] = (char *)aux_base + 2 * (size_t)nrhs * fb + (size_t)(r0 + i) * rb;
     }
     int rc = launch_sap(g, f, p, contiguous((const char *)b + r0 * fb, (char *)x + r0 * fb, n, fb), st,
                         aux_base ? &ax : nullptr);
@@ -242,13 +244,13 @@ int launch_sap(const Geom &g, const OpFields &f, const dd_sap_params &p, const v
 }
 
 int launch_sap(const Geom &g, const OpFields &f, const dd_sap_params &p, const RhsPtrs &rp, cudaStream_t st,
-               const AuxPtrs *ax) {
+               const SapWork *ax) {
   const SapLattice L{g, f, rp.n};
   return launch_sap_lattices(&L, 1, p, rp, st, ax);
 }
 
 int launch_sap_lattices(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, cudaStream_t st,
-                        const AuxPtrs *ax) {
+                        const SapWork *ax) {
   NvtxRange range("dd:sap");
   if (nl < 1 || nl > MAX_SAP_GROUPS) {
     set_error("sap: 1..%d lattices per launch", MAX_SAP_GROUPS);

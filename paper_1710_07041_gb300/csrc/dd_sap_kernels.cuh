@@ -14,7 +14,7 @@ namespace dd {
 // device counter of expired bounded waits (resolved before any capture)
 unsigned *sap_timeout_counter();
 // run `enqueue` (the launches of one smoother application) as a cached CUDA graph
-int sap_launch_as_graph(const std::string &key, int variant, int nkernels, const RhsPtrs &rp, const AuxPtrs *ax,
+int sap_launch_as_graph(const std::string &key, int variant, int nkernels, const RhsPtrs &rp, const SapWork *ax,
                         const std::function<int()> &enqueue, cudaStream_t st);
 
 // Residual modes of one colour phase (bit set `mode` of k_sap_phase).
@@ -84,13 +84,12 @@ __device__ __noinline__ void wait_expired(unsigned *timeouts, unsigned mbar, uns
   }
 }
 
-// ---- tensor memory (TMEM) as a per-thread store of the block's clover
-// blocks (STAGE 3). TMEM has 128 lanes x 512 columns of 32 bits per SM; a
-// warp reaches only the 32 lanes of its sub-partition (warp % 4), so thread
-// t of the CTA owns lane t % 128 and a column range chosen by t / 128. Each
-// clover block a thread multiplies with is read by that thread alone, which
-// is the access TMEM allows. Allocation is per CTA (a power of two of at
-// least 32 columns); the launch keeps at most 512 / NCOLS CTAs of TMEM
+// ---- tensor memory (TMEM) as a per-thread store of the operands a thread
+// alone reads again and again (the packed kernel, dd_sap_pair.cuh). TMEM has
+// 128 lanes x 512 columns of 32 bits per SM; a warp reaches only the 32 lanes
+// of its sub-partition (warp % 4), so thread t of the CTA owns lane t % 128
+// and a column range chosen by t / 128. Allocation is per CTA (a power of two
+// of at least 32 columns); the launch keeps at most 512 / NCOLS CTAs of TMEM
 // kernels on an SM through their shared-memory size, so an allocation never
 // waits for columns.
 template <int NCOLS> __device__ __forceinline__ void tmem_alloc(unsigned dst_smem) {
@@ -108,76 +107,33 @@ __device__ __forceinline__ void tmem_sync() {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
-// the 36 reals of a clover block (m[0..17], real and imaginary parts in
-// turn) to columns taddr ... taddr + 35 of the thread's lane (warp-collective)
-__device__ __forceinline__ void tmem_st36(uint32_t taddr, const cpx<float> *m) {
-  const float *f = (const float *)m;
-  unsigned u[36];
-#pragma unroll
-  for (int i = 0; i < 36; i++) u[i] = __float_as_uint(f[i]);
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};\n" ::"r"(taddr),
-      "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]), "r"(u[8]), "r"(u[9]),
-      "r"(u[10]), "r"(u[11]), "r"(u[12]), "r"(u[13]), "r"(u[14]), "r"(u[15]), "r"(u[16]), "r"(u[17]), "r"(u[18]),
-      "r"(u[19]), "r"(u[20]), "r"(u[21]), "r"(u[22]), "r"(u[23]), "r"(u[24]), "r"(u[25]), "r"(u[26]), "r"(u[27]),
-      "r"(u[28]), "r"(u[29]), "r"(u[30]), "r"(u[31])
-      : "memory");
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(taddr + 32), "r"(u[32]),
-               "r"(u[33]), "r"(u[34]), "r"(u[35])
-               : "memory");
-}
 // the stores of this thread have landed (before the columns are read)
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-// the inverse of tmem_st36 (warp-collective). Both loads and their wait are
-// one asm statement: the destination registers are defined only after it.
-__device__ __forceinline__ void tmem_ld36(uint32_t taddr, cpx<float> *m) {
-  unsigned u[36];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%36];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%32, %33, %34, %35}, [%37];\n"
-      "tcgen05.wait::ld.sync.aligned;\n"
-      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]),
-        "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(u[16]),
-        "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), "=r"(u[24]),
-        "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31]), "=r"(u[32]),
-        "=r"(u[33]), "=r"(u[34]), "=r"(u[35])
-      : "r"(taddr), "r"(taddr + 32)
-      : "memory");
-  float *f = (float *)m;
-#pragma unroll
-  for (int i = 0; i < 36; i++) f[i] = __uint_as_float(u[i]);
-}
-
 // Strided view of one block's pair tile: pair-major (the links: element
 // (i, site) at p[i * stride + site]) or chunked (the clover: see
-// clover_block_chunked, stride = sites per chunk row).
-template <typename P> struct Tile {
+// clover_block_chunked, stride = sites per chunk row). PAIRED: a links tile
+// in the packed kernel's layout (OpFields::links_full of the 4^4 and 8 x 4^3
+// blocks in 32- and 16-bit storage).
+template <typename P, bool PAIRED = false> struct Tile {
   const P *p;
   int stride;
 };
 
 // link mu of tile site s (all nine entries: the kernel reads the full-link
 // field, OpFields::links_full)
-template <typename C, typename P>
-__device__ __forceinline__ void tile_link(const Tile<P> &t, int s, int mu, Link<C> &u) {
+template <typename C, typename P, bool PAIRED>
+__device__ __forceinline__ void tile_link(const Tile<P, PAIRED> &t, int s, int mu, Link<C> &u) {
   DD_CHECK_INDEX(s, t.stride);
 #pragma unroll
-  for (int i = 0; i < 9; i++) u.m[i] = from_pair<C, P>(t.p[(9 * mu + i) * t.stride + s]);
+  for (int i = 0; i < 9; i++) {
+    if constexpr (PAIRED) u.m[i] = paired_link_entry<C, P>(t.p, t.stride, 9 * mu + i, s);
+    else u.m[i] = from_pair<C, P>(t.p[(9 * mu + i) * t.stride + s]);
+  }
 }
 // chirality block h of site s of a chunked clover tile (shared or global memory)
 template <typename C, typename P>
 __device__ __forceinline__ void tile_block(const Tile<P> &t, int s, int h, cpx<C> *m) {
   clover_block_chunked<false, C, P>(t.p, (size_t)t.stride, s, h, m);
-}
-
-// chirality block h of tile site s: from the thread's TMEM columns at taddr
-// (STAGE 3, which stored exactly this block there) or from the tile
-template <int STAGE, typename C, typename P>
-__device__ __forceinline__ void clover_of(const Tile<P> &t, uint32_t taddr, int s, int h, cpx<C> *m) {
-  if constexpr (STAGE == 3) tmem_ld36(taddr, m);
-  else tile_block(t, s, h, m);
 }
 
 // shared-memory vector: [12][Vh] complex, one parity of the block
@@ -215,9 +171,9 @@ __device__ __forceinline__ uint2 inner_neighbours(const Geom &g, const Site &t, 
 // shared half-vector v (the other parity), links from tile L. nf/nbk: neighbour
 // indices (NONE: outside the block); off: tile offset of the other parity.
 // SW: acc holds its spin halves swapped.
-template <int MU, bool SW, typename C, typename P>
+template <int MU, bool SW, typename C, typename T>
 __device__ __forceinline__ void hop_inner_dir(int Vh, int s, unsigned nf, unsigned nbk, int off, const cpx<C> *v,
-                                              const Tile<P> &L, Spinor<C> &acc) {
+                                              const T &L, Spinor<C> &acc) {
   Link<C> u;
   Spinor<C> psi;
   if (nf != NONE) {
@@ -234,9 +190,9 @@ __device__ __forceinline__ void hop_inner_dir(int Vh, int s, unsigned nf, unsign
 
 // The thread's partial sum over its two directions, its own spin half h in
 // acc.c[0..5] and the partner's half in acc.c[6..11] (exchange's layout).
-template <typename C, typename P>
+template <typename C, typename T>
 __device__ __forceinline__ void hops_inner(int Vh, int s, int h, uint2 nbr, int off, const cpx<C> *v,
-                                           const Tile<P> &L, Spinor<C> &acc) {
+                                           const T &L, Spinor<C> &acc) {
 #pragma unroll
   for (int i = 0; i < 12; i++) acc.c[i] = {0, 0};
   if (h == 0) {
@@ -248,10 +204,25 @@ __device__ __forceinline__ void hops_inner(int Vh, int s, int h, uint2 nbr, int 
   }
 }
 
+// full link mu of site (b, s) from the global field
+template <typename S, bool PAIRED, typename C>
+__device__ __forceinline__ void load_full_link(const void *links, const Geom &g, int b, int s, int mu, Link<C> &u) {
+  if constexpr (PAIRED) {
+    using P = typename Store<S>::pair_t;
+    DD_CHECK_INDEX(b, g.nblocks);
+    DD_CHECK_INDEX(s, g.Vb);
+#pragma unroll
+    for (int i = 0; i < 9; i++)
+      u.m[i] = paired_link_entry<C, P>((const P *)links + (size_t)b * 36 * g.Vb, g.Vb, 9 * mu + i, s);
+  } else {
+    load_link<S, C, 9, false>(links, g, b, s, mu, u);
+  }
+}
+
 // acc += hops into site t from the global field x, directions {2h, 2h+1};
 // neighbours inside the block are skipped when self_zero (x known to be 0
 // there), neighbours outside when halo_zero. SW: acc's spin halves swapped.
-template <int MU, bool SW, typename S, typename C>
+template <int MU, bool SW, typename S, bool PAIRED, typename C>
 __device__ __forceinline__ void hop_global_dir(const Geom &g, const Site &t, const void *links, const void *x,
                                                bool self_zero, bool halo_zero, Spinor<C> &acc) {
   int nb, ns;
@@ -262,29 +233,29 @@ __device__ __forceinline__ void hop_global_dir(const Geom &g, const Site &t, con
   neighbour(g, t, MU, +1, &nb, &ns, &sg, &inside);
   if (inside ? !self_zero : !halo_zero) {
     load_spinor<S, C>(x, g, nb, ns, psi);
-    load_link<S, C, 9, false>(links, g, t.b, t.s, MU, u);
+    load_full_link<S, PAIRED>(links, g, t.b, t.s, MU, u);
     hop<MU, true, C, SW>(acc, u, psi, (C)(-0.5f * sg));
   }
   neighbour(g, t, MU, -1, &nb, &ns, &sg, &inside);
   if (inside ? !self_zero : !halo_zero) {
     load_spinor<S, C>(x, g, nb, ns, psi);
-    load_link<S, C, 9, false>(links, g, nb, ns, MU, u);
+    load_full_link<S, PAIRED>(links, g, nb, ns, MU, u);
     hop<MU, false, C, SW>(acc, u, psi, (C)(-0.5f * sg));
   }
 }
 
 // (own spin half in acc.c[0..5], the partner's in acc.c[6..11], as hops_inner)
-template <typename S, typename C>
+template <typename S, bool PAIRED, typename C>
 __device__ __forceinline__ void hops_global(const Geom &g, const Site &t, int h, const void *links, const void *x,
                                             bool self_zero, bool halo_zero, Spinor<C> &acc) {
 #pragma unroll
   for (int i = 0; i < 12; i++) acc.c[i] = {0, 0};
   if (h == 0) {
-    hop_global_dir<0, false, S, C>(g, t, links, x, self_zero, halo_zero, acc);
-    hop_global_dir<1, false, S, C>(g, t, links, x, self_zero, halo_zero, acc);
+    hop_global_dir<0, false, S, PAIRED>(g, t, links, x, self_zero, halo_zero, acc);
+    hop_global_dir<1, false, S, PAIRED>(g, t, links, x, self_zero, halo_zero, acc);
   } else {
-    hop_global_dir<2, true, S, C>(g, t, links, x, self_zero, halo_zero, acc);
-    hop_global_dir<3, true, S, C>(g, t, links, x, self_zero, halo_zero, acc);
+    hop_global_dir<2, true, S, PAIRED>(g, t, links, x, self_zero, halo_zero, acc);
+    hop_global_dir<3, true, S, PAIRED>(g, t, links, x, self_zero, halo_zero, acc);
   }
 }
 
@@ -612,18 +583,11 @@ template <typename S> struct SapSmem {
   using P = typename Store<S>::pair_t;
   static constexpr int LT = 36;   // pairs per site of the links tile (full links)
   static size_t vec_bytes(const Geom &g) { return (size_t)12 * g.Vh * sizeof(cpx<C>); }
-  // TMEM columns of a STAGE-3 CTA: 128 per group of 128 threads (its A_ee^-1
-  // block at +0, its A_oo block at +64)
-  static int tmem_cols(const Geom &g) { return g.Vb > 256 ? 512 : 256; }
-  // stage: 0 nothing staged, 1 links + A_oo + A_ee^-1, 2 links only, 3 links
-  // staged and the clover blocks in TMEM (at least 80 KB, or 150 KB with 512
-  // columns: of an SM's 228 KB, two 256-column CTAs fit, three do not, nor
-  // a 512-column CTA beside any other)
+  // stage: 0 nothing staged, 1 links + A_oo + A_ee^-1, 2 links only
   static size_t bytes(const Geom &g, int stage) {
-    size_t b = 3 * vec_bytes(g) + 96 * sizeof(C) + 16;   // + staging mbarrier, TMEM address
+    size_t b = 3 * vec_bytes(g) + 96 * sizeof(C) + 16;   // + staging mbarrier
     if (stage == 1) b += ((size_t)LT * g.Vb + (size_t)36 * 2 * g.Vh) * sizeof(P);
-    if (stage == 2 || stage == 3) b += (size_t)LT * g.Vb * sizeof(P);
-    if (stage == 3) b = std::max(b, (size_t)(tmem_cols(g) > 256 ? 150 : 80) * 1024);
+    if (stage == 2) b += (size_t)LT * g.Vb * sizeof(P);
     return b;
   }
 };
@@ -644,11 +608,10 @@ __device__ __forceinline__ int sap_block_of(const Geom &g, int colour, int bi) {
 
 // STAGE: 0 operator tiles read through L1/L2; 1 links, A_oo and A_ee^-1 staged
 // in shared memory; 2 links staged, the clover blocks (each read by one
-// thread only) through L1/L2, which halves the footprint. UNROLL (specialised
-// shapes only): the MR loop's even and odd half-steps as separate code.
+// thread only) through L1/L2, which halves the footprint.
 // MULTI: the launch covers several lattice groups (without it, group 0 only,
 // whose fields the compiler reads at constant offsets).
-template <typename S, int STAGE, int MINB, int NT, int SHAPE, bool UNROLL = false, bool MULTI = false>
+template <typename S, int STAGE, int MINB, int NT, int SHAPE, bool MULTI = false>
 __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const RhsPtrs rp, const AuxPtrs ax,
                                                    int colour, int self_zero, int halo_zero, int mode, int nmr,
                                                    int tile, unsigned *timeouts) {
@@ -657,9 +620,10 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
   constexpr int LT = SapSmem<S>::LT;   // pairs per site of the links tile
   // a specialised shape is launched with one thread per site: blockDim.x == NT
   static_assert(SHAPE == 0 || (SHAPE == 1 && NT == 256) || (SHAPE == 2 && NT == 512), "shape / threads");
-  // TMEM holds FP32 clover blocks, one thread per lane: specialised shapes only
-  static_assert(STAGE != 3 || (SHAPE != 0 && sizeof(C) == 4), "TMEM clover: FP32 arithmetic, fixed shape");
-  constexpr int TCOLS = NT > 256 ? 512 : 256;
+  // the 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage hold their links in
+  // the packed kernel's layout
+  constexpr bool PAIRED = SHAPE != 0 && sizeof(C) == 4;
+  static_assert(!PAIRED || STAGE == 0, "packed links are read from global memory here");
   extern __shared__ __align__(16) unsigned char smem[];
   // every group of a launch has the same block shape (checked on the host)
   const int Vh = block_shape<SHAPE>(G.grp[0].g).Vh, Vb = block_shape<SHAPE>(G.grp[0].g).Vb;
@@ -670,24 +634,13 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
   cpx<C> *xch = te + 12 * Vh;     // partial-sum exchange between thread halves
   C *red = (C *)(xch + 12 * Vh);
   uint64_t *mbar = (uint64_t *)(red + 96);   // staging barrier (16 bytes reserved)
-  uint32_t *tmem_at = (uint32_t *)(mbar + 1);  // TMEM base address (STAGE 3)
   unsigned char *tiles = (unsigned char *)(red + 96) + 16;
   unsigned phase = 0;                        // parity of the staging barrier's current phase
   if constexpr (STAGE != 0) {
     if (threadIdx.x == 0) mbar_init(mbar);
-    if constexpr (STAGE == 3) {
-      if (threadIdx.x < 32) tmem_alloc<TCOLS>(smem_u32(tmem_at));
-      tmem_sync();
-    } else {
-      __syncthreads();
-    }
+    __syncthreads();
   }
   const unsigned mbar_s = smem_u32(mbar);
-  // this thread's TMEM columns: lane threadIdx.x % 128 (the warp's
-  // sub-partition), 128 columns per group of 128 threads
-  uint32_t tm = 0;
-  if constexpr (STAGE == 3)
-    tm = *tmem_at + ((uint32_t)(32 * ((threadIdx.x / 32) % 4)) << 16) + (uint32_t)(threadIdx.x / 128) * 128u;
   bool quit = false;   // a staging wait expired: leave through the common exit
 
   // Work items: (lattice group, block of this colour, right-hand-side tile),
@@ -765,7 +718,8 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
   // and for STAGE 1 the odd half of every clover chunk row (36 / CP pieces of
   // Vh chunks) and the even-site inverse tile (contiguous). Every size is a
   // multiple of 16 bytes and every address 16-byte aligned.
-  Tile<P> Lt, Ao, Ai;
+  Tile<P, PAIRED> Lt;
+  Tile<P> Ao, Ai;
   if constexpr (STAGE == 1) {
     P *sl = (P *)tiles;
     P *sa = sl + (size_t)LT * Vb;
@@ -785,7 +739,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
     Lt = {sl, Vb};
     Ao = {sa, Vh};
     Ai = {si, Vh};
-  } else if constexpr (STAGE == 2 || STAGE == 3) {
+  } else if constexpr (STAGE == 2) {
     P *sl = (P *)tiles;
     if (threadIdx.x == 0) {
       const unsigned lb = (unsigned)LT * Vb * sizeof(P);
@@ -802,24 +756,12 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
     Ai = {(const P *)cinv + (size_t)b * 36 * Vh, Vh};
   }
 
-  if constexpr (STAGE == 3) {
-    // this thread's two clover blocks (A_ee^-1 of even site j, A_oo of odd
-    // site j, chirality h) into its TMEM columns; the previous item's reads
-    // of them completed (tmem_ld36 waits). Both blocks are loaded before the
-    // first store (one round trip to L2 per item, not two).
-    cpx<C> mi[18], mo[18];
-    tile_block(Ai, j, h, mi);
-    tile_block(Ao, j, h, mo);
-    tmem_st36(tm, mi);
-    tmem_st36(tm + 64, mo);
-    tmem_wait_st();
-  }
   const Site se = decode(g, b, j), so = decode(g, b, Vh + j);
   const uint2 nbr_e = inner_neighbours(g, se, h), nbr_o = inner_neighbours(g, so, h);
   // corrections travel between phases as face flux (32-bit arithmetic,
   // blocks whose flux fits a spinor field; the same for every phase of the
   // lattice), else as e itself
-  const bool flux = flux_layout<C>(g);
+  const bool flux = !PAIRED && flux_layout<C>(g);
   // the flux receiver multiplies by the staged links: wait for them first
   const bool early = flux && (mode & SAP_INCR) && (mode & SAP_HALO_E);
   // right-hand sides blockIdx.y * tile ... share the staged tiles
@@ -843,7 +785,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
         phase ^= 1u;
       }
     }
-    if constexpr (sizeof(C) == 4)
+    if constexpr (sizeof(C) == 4 && !PAIRED)
       if (early) flux_receive<S, C, P>(g, b, Lt, ax.e[r], rho);
 
     // ---- 2. block residual (halves h of the even and odd site): r = b - D x,
@@ -870,7 +812,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
   #pragma unroll 1
         for (int par = 0; par < 2; par++) {
           Spinor<C> part;
-          hops_global<S, C>(g, par ? so : se, h, links, ax.e[r], true, false, part);
+          hops_global<S, PAIRED>(g, par ? so : se, h, links, ax.e[r], true, false, part);
           cpx<C> hx[6];
           exchange(xch, Vh, j, h, part, hx);
   #pragma unroll
@@ -886,7 +828,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
       for (int par = 0; par < 2; par++) {
         const Site &t = par ? so : se;
         Spinor<C> part;
-        hops_global<S, C>(g, t, h, links, xf, self_zero, halo_zero, part);
+        hops_global<S, PAIRED>(g, t, h, links, xf, self_zero, halo_zero, part);
         cpx<C> hx[6], ax[6] = {}, m[18], xh[6];
         exchange(xch, Vh, j, h, part, hx);
         if (!self_zero) {
@@ -923,7 +865,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
     // te = A_ee^-1 D_eo rho, then p = A_oo rho - D_oe te and the MR update.
     // Last step: e_e = A_ee^-1 (r_e - D_eo e_o).
     cpx<C> m[18], tmp[6], rh[6], eo[6], ee[6];
-    clover_of<STAGE>(Ai, tm, j, h, m);
+    tile_block(Ai, j, h, m);
     herm6_mv(m, r_e, tmp);
   #pragma unroll
     for (int i = 0; i < 6; i++) {
@@ -945,67 +887,6 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
       }
       __syncthreads();
     }
-    if constexpr (UNROLL && SHAPE != 0) {
-    // steps 2k-1 (even) and 2k (odd) for k = 1..n_MR as separate code, then
-    // the last even step: no run-time parity selects, twice the hop code
-  #pragma unroll 1
-    for (int k = 1; k <= nmr + 1; k++) {
-      const bool last = k == nmr + 1;
-      {   // even: te = A_ee^-1 D_eo rho, or on the last step e_e = A_ee^-1 (r_e - D_eo e_o)
-        Spinor<C> part;
-        hops_inner(Vh, j, h, nbr_e, Vh, rho, Lt, part);
-        cpx<C> hv[6], u[6], mu[6];
-        exchange(xch, Vh, j, h, part, hv);
-  #pragma unroll
-        for (int i = 0; i < 6; i++) u[i] = last ? cpx<C>{r_e[i].re - hv[i].re, r_e[i].im - hv[i].im} : hv[i];
-        clover_of<STAGE>(Ai, tm, j, h, m);
-        herm6_mv(m, u, mu);
-        if (last) {
-  #pragma unroll
-          for (int i = 0; i < 6; i++) ee[i] = mu[i];
-        } else {
-  #pragma unroll
-          for (int i = 0; i < 6; i++) te[(6 * h + i) * Vh + j] = mu[i];
-        }
-        __syncthreads();
-      }
-      if (last) break;
-      {   // odd: p = A_oo rho - D_oe te and the MR update of e_o and rho
-        Spinor<C> part;
-        hops_inner(Vh, Vh + j, h, nbr_o, 0, te, Lt, part);
-        cpx<C> hv[6], mu[6], p[6];
-        exchange(xch, Vh, j, h, part, hv);
-        clover_of<STAGE>(Ao, tm + 64, j, h, m);
-        herm6_mv(m, rh, mu);
-        C pr_re = 0, pr_im = 0, pp = 0;
-  #pragma unroll
-        for (int i = 0; i < 6; i++) {
-          p[i] = {mu[i].re - hv[i].re, mu[i].im - hv[i].im};
-          pr_re += p[i].re * rh[i].re + p[i].im * rh[i].im;
-          pr_im += p[i].re * rh[i].im - p[i].im * rh[i].re;
-          pp += p[i].re * p[i].re + p[i].im * p[i].im;
-        }
-        block_sum3<SHAPE != 0 ? NT / 32 : 0>(pr_re, pr_im, pp, red);
-        C a_re = 0, a_im = 0;
-        if (pp > (C)0) {
-          a_re = pr_re / pp;
-          a_im = pr_im / pp;
-        }
-  #pragma unroll
-        for (int i = 0; i < 6; i++) {
-          eo[i].re += a_re * rh[i].re - a_im * rh[i].im;
-          eo[i].im += a_re * rh[i].im + a_im * rh[i].re;
-          rh[i].re -= a_re * p[i].re - a_im * p[i].im;
-          rh[i].im -= a_re * p[i].im + a_im * p[i].re;
-        }
-        // the even step after the last MR update reads e_o instead of rho
-        const bool last_odd = k == nmr;
-  #pragma unroll
-        for (int i = 0; i < 6; i++) rho[(6 * h + i) * Vh + j] = last_odd ? eo[i] : rh[i];
-        __syncthreads();
-      }
-    }
-    } else {
     const int last = 2 * nmr + 1;
   #pragma unroll 1
     for (int step = 1; step <= last; step++) {
@@ -1019,7 +900,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
   #pragma unroll
       for (int i = 0; i < 6; i++)
         u[i] = odd ? rh[i] : (step == last ? cpx<C>{r_e[i].re - hv[i].re, r_e[i].im - hv[i].im} : hv[i]);
-      clover_of<STAGE>(odd ? Ao : Ai, tm + (odd ? 64 : 0), j, h, m);
+      tile_block(odd ? Ao : Ai, j, h, m);
       herm6_mv(m, u, mu);
       if (odd) {
         cpx<C> p[6];
@@ -1057,7 +938,6 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
       }
       __syncthreads();
     }
-    }
 
     // ---- x += e: gather both halves through shared memory, then half 0
     // writes the even site j and half 1 the odd site j (and, when asked,
@@ -1093,21 +973,29 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
       }
       store_spinor<S, C>(xf, g, b, s, xs);
     }
-    if constexpr (sizeof(C) == 4)
+    if constexpr (sizeof(C) == 4 && !PAIRED)
       if ((mode & SAP_WRITE_E) && flux) flux_produce<S, C, P>(g, b, se.bc, Lt, te, xch, ax.e[r]);
     __syncthreads();   // shared vectors are reused by the next right-hand side
   }
   if (quit) break;
   }  // work items
-  if constexpr (STAGE == 3) {
-    // every thread's TMEM reads are complete; the allocating warp frees
-    tmem_sync();
-    if (threadIdx.x < 32) tmem_dealloc<TCOLS>(*tmem_at);
-  }
 }
 
-template <typename S, int STAGE, int MINB, int NT, int SHAPE, bool UNROLL = false, bool MULTI = false>
-int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const AuxPtrs *ax, int tile,
+// the launch's group table: work items (block of a colour, tile of right-hand
+// sides) of every lattice in turn
+inline SapGroups sap_groups(const SapLattice *L, int nl, int tile) {
+  SapGroups G{};
+  G.n = nl;
+  for (int k = 0, rhs0 = 0; k < nl; k++) {
+    G.grp[k] = SapGroup{L[k].g, L[k].f.links_full, L[k].f.clov, L[k].f.cinv, rhs0, L[k].nrhs, G.nitems};
+    G.nitems += L[k].g.nblocks / 2 * ((L[k].nrhs + tile - 1) / tile);
+    rhs0 += L[k].nrhs;
+  }
+  return G;
+}
+
+template <typename S, int STAGE, int MINB, int NT, int SHAPE, bool MULTI = false>
+int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
           bool persistent, cudaStream_t st) {
   if (nl > 1 && !MULTI) {
     set_error("sap: this launch variant covers one lattice");
@@ -1115,7 +1003,7 @@ int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
   }
   const Geom &g = L[0].g;   // every lattice of the launch has this block shape
   size_t smem = SapSmem<S>::bytes(g, STAGE);
-  auto kern = k_sap_phase<S, STAGE, MINB, NT, SHAPE, UNROLL, MULTI>;
+  auto kern = k_sap_phase<S, STAGE, MINB, NT, SHAPE, MULTI>;
   // raise the kernel's dynamic shared-memory limit once (never during a capture)
   static std::mutex mu;
   static int raised = 0;
@@ -1126,15 +1014,8 @@ int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
       raised = 227 * 1024;
     }
   }
-  SapGroups G{};
-  G.n = nl;
-  int nitems = 0;
-  for (int k = 0, rhs0 = 0; k < nl; k++) {
-    G.grp[k] = SapGroup{L[k].g, L[k].f.links_full, L[k].f.clov, L[k].f.cinv, rhs0, L[k].nrhs, nitems};
-    nitems += L[k].g.nblocks / 2 * ((L[k].nrhs + tile - 1) / tile);
-    rhs0 += L[k].nrhs;
-  }
-  G.nitems = nitems;
+  const SapGroups G = sap_groups(L, nl, tile);
+  const int nitems = G.nitems;
   int grid = nitems;
   if (persistent) {
     int dev = 0, sms = 0, occ = 0;
@@ -1163,161 +1044,11 @@ int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
         if (!(sw == p.sweeps - 1 && colour == 1)) mode |= SAP_WRITE_E;
         if (sw + 1 < p.sweeps) mode |= SAP_WRITE_R;
       }
-      kern<<<grid, g.Vb, smem, st>>>(G, rp, ax ? *ax : none, colour, self_zero, halo_zero, mode, p.mr_steps, tile,
+      kern<<<grid, g.Vb, smem, st>>>(G, rp, ax ? (const AuxPtrs &)*ax : none, colour, self_zero, halo_zero, mode, p.mr_steps, tile,
                                      sap_timeout_counter());
       DD_LAUNCHED();
     }
   return DD_OK;
-}
-
-// the kernel specialised for the lattice's block shape when there is one
-template <typename S, int STAGE, int MINB, int NT = 256>
-int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const AuxPtrs *ax, int tile,
-          bool persistent, cudaStream_t st) {
-  constexpr int SH = NT == 256 ? 1 : 2;   // the shape this thread count fits
-  if (shape_of(L[0].g) == SH)
-    return nl > 1 ? sap_k<S, STAGE, MINB, NT, SH, false, true>(L, nl, p, rp, ax, tile, persistent, st)
-                  : sap_k<S, STAGE, MINB, NT, SH>(L, nl, p, rp, ax, tile, persistent, st);
-  if constexpr (STAGE == 3) {   // TMEM clover: specialised shapes only
-    set_error("sap: the TMEM clover layout exists for the specialised block shapes only");
-    return (int)DD_EINVAL;
-  } else {
-    return nl > 1 ? sap_k<S, STAGE, MINB, NT, 0, false, true>(L, nl, p, rp, ax, tile, persistent, st)
-                  : sap_k<S, STAGE, MINB, NT, 0>(L, nl, p, rp, ax, tile, persistent, st);
-  }
-}
-// the MR loop unrolled by parity (specialised shape only)
-template <typename S, int STAGE, int MINB, int NT = 256>
-int sap_u(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const AuxPtrs *ax, int tile,
-          bool persistent, cudaStream_t st) {
-  constexpr int SH = NT == 256 ? 1 : 2;
-  if (shape_of(L[0].g) != SH) {
-    set_error("sap: the unrolled MR loop exists for the specialised block shapes only");
-    return DD_EINVAL;
-  }
-  return sap_k<S, STAGE, MINB, NT, SH, true>(L, nl, p, rp, ax, tile, persistent, st);
-}
-
-template <typename S> constexpr bool sixteen_bit() {
-  return Store<S>::prec == DD_F16 || Store<S>::prec == DD_BF16 || Store<S>::prec == DD_F16N;
-}
-
-// Launch variants: tiles staged in shared memory with one CTA per SM; tiles
-// staged with two CTAs per SM (fits when the storage is 16-bit); only the
-// links staged, with two CTAs per SM (when the full staging does not fit
-// twice); tiles read through L1/L2 with two CTAs per SM; for 16-bit storage
-// on the 4^4 shape with one right-hand side, the two-CTA layouts again with
-// the MR loop unrolled by parity; for 32- and 16-bit storage on the
-// specialised shapes, the links staged and the clover blocks in TMEM.
-// Variants that do not fit are skipped. With several right-hand sides a CTA also solves `tile` of them with one
-// staging of its block's operator (rhs_tile; 0 lets the autotuner choose).
-template <typename S>
-int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const AuxPtrs *ax,
-                 cudaStream_t st) {
-  const Geom &g = L[0].g;
-  const size_t limit = 227 * 1024, half = 113 * 1024;
-  const bool stage1 = SapSmem<S>::bytes(g, 1) <= limit;
-  const bool stage2 = SapSmem<S>::bytes(g, 1) <= half;
-  const bool links2 = !stage2 && SapSmem<S>::bytes(g, 2) <= half;
-  const bool nost2 = SapSmem<S>::bytes(g, 0) <= half;
-  if (!stage1 && SapSmem<S>::bytes(g, 0) > limit) {
-    set_error("sap: block of %d sites needs more shared memory than available", g.Vb);
-    return DD_EINVAL;
-  }
-  // links staged and the clover blocks in TMEM (32- and 16-bit storage on
-  // the specialised shapes)
-  constexpr bool tmem_ok = Store<S>::prec != DD_F64;
-  const int sh = shape_of(g);
-  int layouts[8], nlay = 0;
-  if (g.Vb > 256) {
-    // 512-site blocks (e.g. 8 x 4^3): 512 threads, one CTA per SM
-    layouts[nlay++] = stage1 ? 3 : 4;
-    if (tmem_ok && sh == 2 && SapSmem<S>::bytes(g, 3) <= limit) layouts[nlay++] = 9;
-  } else {
-    if (stage1) layouts[nlay++] = 0;
-    if (stage2) layouts[nlay++] = 1;
-    if (links2) layouts[nlay++] = 5;
-    if (nost2 || !stage1) layouts[nlay++] = 2;
-    // 16-bit storage on the 4^4 shape with one right-hand side: the two-CTA
-    // layouts also with the MR loop unrolled by parity (measured faster
-    // there, slower in multi-source tiles and for FP32)
-    if (sixteen_bit<S>() && shape_of(g) == 1 && rp.n == 1) {
-      if (stage2) layouts[nlay++] = 6;
-      if (nost2 || !stage1) layouts[nlay++] = 7;
-    }
-    if (tmem_ok && sh == 1 && SapSmem<S>::bytes(g, 3) <= half) layouts[nlay++] = 8;
-  }
-  int tiles[6], nt = 0;
-  if (p.rhs_tile > 0) {
-    tiles[nt++] = p.rhs_tile < rp.n ? p.rhs_tile : rp.n;
-  } else {
-    const int cand[5] = {1, 2, 4, 8, 12};
-    for (int c : cand)
-      if (c <= rp.n) tiles[nt++] = c;
-  }
-  // variant k: layout k % nlay, RHS tile (k / nlay) % nt, persistent grid if k >= nlay * nt
-  auto run = [&](int k) {
-    const int layout = layouts[k % nlay], tile = tiles[(k / nlay) % nt];
-    const bool pers = k >= nlay * nt;
-    switch (layout) {
-      case 1: return sap_t<S, 1, 2>(L, nl, p, rp, ax, tile, pers, st);
-      case 2: return sap_t<S, 0, 2>(L, nl, p, rp, ax, tile, pers, st);
-      case 3: return sap_t<S, 1, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
-      case 4: return sap_t<S, 0, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
-      case 5: return sap_t<S, 2, 2>(L, nl, p, rp, ax, tile, pers, st);
-      case 8:
-      case 9:
-        if constexpr (tmem_ok) {
-          if (layout == 8) return sap_t<S, 3, 2>(L, nl, p, rp, ax, tile, pers, st);
-          return sap_t<S, 3, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
-        }
-        return (int)DD_EINVAL;
-      case 6:
-      case 7:
-        if constexpr (sixteen_bit<S>()) {
-          if (layout == 6) return sap_u<S, 1, 2>(L, nl, p, rp, ax, tile, pers, st);
-          return sap_u<S, 0, 2>(L, nl, p, rp, ax, tile, pers, st);
-        }
-        return (int)DD_EINVAL;
-      default: return sap_t<S, 1, 1>(L, nl, p, rp, ax, tile, pers, st);
-    }
-  };
-  int k = 0;
-  // the tuner's key: lattice, precision, right-hand-side count, smoother
-  // parameters and boundary; a launch over several lattices is tuned once
-  // per block shape, precision and total right-hand-side count (a served
-  // stream meets ever new mixes of lattices, each would otherwise be tuned)
-  std::string key;
-  if (nl == 1) {
-    key = tune_key("sap", g, L[0].f.prec, rp.n) + "|" + std::to_string(p.sweeps) + "," +
-          std::to_string(p.mr_steps) + "," + std::to_string(p.rhs_tile) + "," + std::to_string(g.antiperiodic);
-  } else {
-    Geom gb = g;   // the block shape only
-    for (int mu = 0; mu < 4; mu++) gb.L[mu] = 0;
-    key = tune_key("sap-lattices", gb, L[0].f.prec, rp.n) + "|" + std::to_string(p.sweeps) + "," +
-          std::to_string(p.mr_steps) + "," + std::to_string(p.rhs_tile);
-  }
-  // the graph cache's key adds every lattice's extents, boundary and right-hand sides
-  std::string shape;
-  for (int k = 0; k < nl; k++)
-    shape += "|" + std::to_string(L[k].g.L[0]) + "," + std::to_string(L[k].g.L[1]) + "," +
-             std::to_string(L[k].g.L[2]) + "," + std::to_string(L[k].g.L[3]) + "," + std::to_string(L[k].nrhs) + "," +
-             std::to_string(L[k].g.antiperiodic);
-  // a graph may only replay where a fresh capture records the same arguments:
-  // every lattice's field pointers are part of its key
-  std::string fields;
-  for (int k = 0; k < nl; k++)
-    fields += std::to_string((uintptr_t)L[k].f.links_full) + "," + std::to_string((uintptr_t)L[k].f.clov) + "," +
-              std::to_string((uintptr_t)L[k].f.cinv) + ";";
-  // x is pure output when x_is_zero, so trial runs leave the same result
-  if (p.x_is_zero) {
-    int rc = tuned_variant(key, 2 * nlay * nt, run, st, &k);
-    if (rc) return rc;
-  } else {
-    int c = tune_lookup(key);
-    k = c >= 0 ? c : 0;
-  }
-  return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps, rp, ax, [&] { return run(k); }, st);
 }
 
 }  // namespace

@@ -1,0 +1,191 @@
+// Host side of the Schwarz smoother for one storage precision: launch
+// variants, tuning, graph key (included by dd_sap_<prec>.cu).
+#pragma once
+#include "dd_sap_pair.cuh"
+
+namespace dd {
+namespace {
+
+// the kernel specialised for the lattice's block shape when there is one (in
+// 32- and 16-bit storage only without staging: the form without work fields)
+template <typename S, int STAGE, int MINB, int NT = 256>
+int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
+          bool persistent, cudaStream_t st) {
+  constexpr int SH = NT == 256 ? 1 : 2;   // the shape this thread count fits
+  if (shape_of(L[0].g) == SH) {
+    if constexpr (STAGE == 0 || Store<S>::prec == DD_F64)
+      return nl > 1 ? sap_k<S, STAGE, MINB, NT, SH, true>(L, nl, p, rp, ax, tile, persistent, st)
+                    : sap_k<S, STAGE, MINB, NT, SH>(L, nl, p, rp, ax, tile, persistent, st);
+    set_error("sap: no staged layout for this block shape");
+    return DD_EINVAL;
+  }
+  return nl > 1 ? sap_k<S, STAGE, MINB, NT, 0, true>(L, nl, p, rp, ax, tile, persistent, st)
+                : sap_k<S, STAGE, MINB, NT, 0>(L, nl, p, rp, ax, tile, persistent, st);
+}
+
+// One smoother application in the packed kernel (dd_sap_pair.cuh). From a
+// given x the first sweep works on the residual b - D x, formed once as an
+// FP32 field by the operator's kernel; after that, as from x = 0, every phase
+// takes its residual from the stored one and the neighbours' flux.
+template <typename S, int SHAPE, bool MULTI>
+int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork &ax, int tile,
+               cudaStream_t st) {
+  using PG = PairGeom<SHAPE>;
+  auto kern = k_sap_pair<S, SHAPE, MULTI>;
+  static std::once_flag once;   // raise the kernel's shared-memory limit (never during a capture)
+  static cudaError_t limit = cudaSuccess;
+  std::call_once(once, [&] {
+    limit = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG::SMEM);
+  });
+  DD_CUDA(limit);
+  const SapGroups G = sap_groups(L, nl, tile);
+  // Each CTA requests into L2 the operator of the block that a quarter of the
+  // resident CTAs ahead of it starts on (a block's start then waits for L2
+  // instead of HBM: 0.412 -> 0.405 ms per FP32 phase at 64x32^3; half of the
+  // resident CTAs ahead: 0.428, all of them: 0.445, the requests then push
+  // one another out of L2)
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int ahead = sms * (SHAPE == 1 ? 2 : 1) / 4;
+  RhsPtrs first = rp;   // the first sweep's right-hand sides
+  if (!p.x_is_zero) {
+    RhsPtrs x, b;
+    for (int k = 0, r = 0; k < nl; k++) {
+      x.n = b.n = L[k].nrhs;
+      for (int i = 0; i < L[k].nrhs; i++, r++) {
+        x.in[i] = rp.out[r];
+        x.out[i] = ax.r0[r];
+        b.in[i] = rp.in[r];
+        b.out[i] = nullptr;
+        first.in[r] = ax.r0[r];
+      }
+      if (int rc = launch_residual(L[k].g, L[k].f, x, b, st)) return rc;
+    }
+  }
+  for (int sw = 0; sw < p.sweeps; sw++)
+    for (int colour = 0; colour < 2; colour++) {
+      int mode = sw ? SAP_HALO_E : SAP_FROM_B | (colour ? SAP_HALO_E : 0) | (p.x_is_zero ? 0 : SAP_B32);
+      if (!(sw == p.sweeps - 1 && colour == 1)) mode |= SAP_WRITE_E;   // read by the next phase
+      if (sw + 1 < p.sweeps) mode |= SAP_WRITE_R;                      // by this colour's next one
+      kern<<<G.nitems, PG::NT, PG::SMEM, st>>>(G, sw ? rp : first, ax, colour, p.x_is_zero && sw == 0, mode,
+                                               p.mr_steps, tile, ahead, sap_timeout_counter());
+      DD_LAUNCHED();
+    }
+  return DD_OK;
+}
+
+// Launch variants. The 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage run
+// in the packed kernel, whatever the lattice size and right-hand-side count;
+// only a call without work fields (or DD_SAP_INCR=0) takes the unstaged
+// general kernel there. The other blocks and FP64 run in the general kernel:
+// tiles staged in shared memory with one CTA per SM; tiles staged with two
+// CTAs per SM (fits when the storage is 16-bit); only the links staged, with
+// two CTAs per SM (when the full staging does not fit twice); tiles read
+// through L1/L2 with two CTAs per SM. Variants that do not fit are skipped.
+// With several right-hand sides a CTA also solves `tile` of them with one
+// staging of its block's operator (rhs_tile; 0 lets the autotuner choose).
+template <typename S>
+int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax,
+                 cudaStream_t st) {
+  const Geom &g = L[0].g;
+  const bool paired = paired_links(g, L[0].f.prec);
+  if (paired && ax && !p.x_is_zero && !ax->r0[0]) ax = nullptr;
+  const bool pair = paired && ax;
+  const size_t limit = 227 * 1024, half = 113 * 1024;
+  const bool stage1 = SapSmem<S>::bytes(g, 1) <= limit;
+  const bool stage2 = SapSmem<S>::bytes(g, 1) <= half;
+  const bool links2 = !stage2 && SapSmem<S>::bytes(g, 2) <= half;
+  const bool nost2 = SapSmem<S>::bytes(g, 0) <= half;
+  if (!stage1 && SapSmem<S>::bytes(g, 0) > limit) {
+    set_error("sap: block of %d sites needs more shared memory than available", g.Vb);
+    return DD_EINVAL;
+  }
+  int layouts[4], nlay = 0;
+  if (paired) {
+    layouts[nlay++] = g.Vb > 256 ? 4 : 2;
+  } else if (g.Vb > 256) {
+    // 512-site blocks (e.g. 8 x 4^3): 512 threads, one CTA per SM
+    layouts[nlay++] = stage1 ? 3 : 4;
+  } else {
+    if (stage1) layouts[nlay++] = 0;
+    if (stage2) layouts[nlay++] = 1;
+    if (links2) layouts[nlay++] = 5;
+    if (nost2 || !stage1) layouts[nlay++] = 2;
+  }
+  int tiles[6], nt = 0;
+  if (p.rhs_tile > 0) {
+    tiles[nt++] = p.rhs_tile < rp.n ? p.rhs_tile : rp.n;
+  } else {
+    const int cand[5] = {1, 2, 4, 8, 12};
+    for (int c : cand)
+      if (c <= rp.n) tiles[nt++] = c;
+  }
+  // variant k: layout k % nlay, RHS tile (k / nlay) % nt, persistent grid if
+  // k >= nlay * nt; packed kernel: RHS tile k
+  auto run = [&](int k) {
+    if constexpr (Store<S>::prec != DD_F64) {
+      if (pair) {
+        if (shape_of(g) == 1)
+          return nl > 1 ? sap_pair_k<S, 1, true>(L, nl, p, rp, *ax, tiles[k], st)
+                        : sap_pair_k<S, 1, false>(L, nl, p, rp, *ax, tiles[k], st);
+        return nl > 1 ? sap_pair_k<S, 2, true>(L, nl, p, rp, *ax, tiles[k], st)
+                      : sap_pair_k<S, 2, false>(L, nl, p, rp, *ax, tiles[k], st);
+      }
+    }
+    const int layout = layouts[k % nlay], tile = tiles[(k / nlay) % nt];
+    const bool pers = k >= nlay * nt;
+    switch (layout) {
+      case 1: return sap_t<S, 1, 2>(L, nl, p, rp, ax, tile, pers, st);
+      case 2: return sap_t<S, 0, 2>(L, nl, p, rp, ax, tile, pers, st);
+      case 3: return sap_t<S, 1, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
+      case 4: return sap_t<S, 0, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
+      case 5: return sap_t<S, 2, 2>(L, nl, p, rp, ax, tile, pers, st);
+      default: return sap_t<S, 1, 1>(L, nl, p, rp, ax, tile, pers, st);
+    }
+  };
+  const int nvar = pair ? nt : 2 * nlay * nt;
+  int k = 0;
+  // the tuner's key: lattice, precision, right-hand-side count, smoother
+  // parameters and boundary; a launch over several lattices is tuned once
+  // per block shape, precision and total right-hand-side count (a served
+  // stream meets ever new mixes of lattices, each would otherwise be tuned)
+  const std::string kind = pair ? "sap-pair" : "sap";
+  std::string key;
+  if (nl == 1) {
+    key = tune_key(kind.c_str(), g, L[0].f.prec, rp.n) + "|" + std::to_string(p.sweeps) + "," +
+          std::to_string(p.mr_steps) + "," + std::to_string(p.rhs_tile) + "," + std::to_string(g.antiperiodic);
+  } else {
+    Geom gb = g;   // the block shape only
+    for (int mu = 0; mu < 4; mu++) gb.L[mu] = 0;
+    key = tune_key((kind + "-lattices").c_str(), gb, L[0].f.prec, rp.n) + "|" + std::to_string(p.sweeps) + "," +
+          std::to_string(p.mr_steps) + "," + std::to_string(p.rhs_tile);
+  }
+  // the graph cache's key adds every lattice's extents, boundary and right-hand sides
+  std::string shape;
+  for (int k = 0; k < nl; k++)
+    shape += "|" + std::to_string(L[k].g.L[0]) + "," + std::to_string(L[k].g.L[1]) + "," +
+             std::to_string(L[k].g.L[2]) + "," + std::to_string(L[k].g.L[3]) + "," + std::to_string(L[k].nrhs) + "," +
+             std::to_string(L[k].g.antiperiodic);
+  // a graph may only replay where a fresh capture records the same arguments:
+  // every lattice's field pointers are part of its key
+  std::string fields = p.x_is_zero ? "z" : "x";
+  for (int k = 0; k < nl; k++)
+    fields += std::to_string((uintptr_t)L[k].f.links_full) + "," + std::to_string((uintptr_t)L[k].f.clov) + "," +
+              std::to_string((uintptr_t)L[k].f.cinv) + "," + std::to_string((uintptr_t)L[k].f.links) + ";";
+  if (!p.x_is_zero && pair)
+    for (int r = 0; r < rp.n; r++) fields += std::to_string((uintptr_t)ax->r0[r]) + ",";
+  // x is pure output when x_is_zero, so trial runs leave the same result
+  if (p.x_is_zero) {
+    int rc = tuned_variant(key, nvar, run, st, &k);
+    if (rc) return rc;
+  } else {
+    int c = tune_lookup(key);
+    k = c >= 0 && c < nvar ? c : 0;
+  }
+  return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps + (p.x_is_zero || !pair ? 0 : nl), rp, ax,
+                             [&] { return run(k); }, st);
+}
+
+}  // namespace
+}  // namespace dd

@@ -430,7 +430,7 @@ int BatchSolver::arnoldi_step(std::vector<Slot *> &A) {
   } else {
     const bool direct = op_->prec == zprec_ && A.size() == 1;
     RhsPtrs sp_ptrs;
-    AuxPtrs ax;
+    SapWork ax;
     SapLattice lats[MAX_SAP_GROUPS];
     int nlat = 0;
     sp_ptrs.n = 0;
