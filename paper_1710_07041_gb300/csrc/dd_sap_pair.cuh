@@ -84,9 +84,10 @@ template <int SHAPE> struct PairGeom {
   static constexpr int BT = SHAPE == 2 ? 8 : 4;
   static constexpr int ROWS = 16 * BT, NT = 2 * ROWS, VH = 2 * ROWS, VB = 4 * ROWS;
   static constexpr int TCOLS = 2 * NT;   // TMEM columns (256 per 128 threads)
-  // shared memory: links, two vectors, reduction scratch, barrier, TMEM address
+  // shared memory: links, two vectors (first: the incoming flux), reduction
+  // scratch, two barriers, TMEM address
   static constexpr int LINKS = 36 * 2 * ROWS, VEC = 12 * ROWS;   // in quads
-  static constexpr size_t SMEM = (size_t)(LINKS + 2 * VEC) * 16 + 3 * 8 * 4 + 16;
+  static constexpr size_t SMEM = (size_t)(LINKS + 2 * VEC) * 16 + 3 * 8 * 4 + 32;
 };
 
 // ---- tensor memory: N words of this thread's lane from column taddr
@@ -685,14 +686,17 @@ __device__ __forceinline__ void half_st(void *field, const Geom &g, int b, int s
 template <typename S, bool RES> struct QuadStore {
   static constexpr bool f32 = Store<S>::prec == DD_F32 || (RES && Store<S>::prec == DD_F16N);
   static constexpr int bytes = f32 ? 16 : 8;
+  using raw = std::conditional_t<f32, float4, uint2>;   // as loaded, converted where it is used
 };
-template <typename S, bool RES> __device__ __forceinline__ quad quad_ld(const void *p, size_t i) {
+template <typename S, bool RES>
+__device__ __forceinline__ typename QuadStore<S, RES>::raw quad_raw(const void *p, size_t i) {
+  return ((const typename QuadStore<S, RES>::raw *)p)[i];
+}
+template <typename S, bool RES> __device__ __forceinline__ quad quad_of(typename QuadStore<S, RES>::raw v) {
   if constexpr (QuadStore<S, RES>::f32) {
-    const float4 v = ((const float4 *)p)[i];
     return quad{pk(v.x, v.y), pk(v.z, v.w)};
   } else {
     using P = typename Store<S>::pair_t;
-    const uint2 v = ((const uint2 *)p)[i];
     const P *h = (const P *)&v;
     const cpx<float> a = from_pair<float, P>(h[0]), b = from_pair<float, P>(h[1]);
     return quad{pk(a.re, a.im), pk(b.re, b.im)};
@@ -727,20 +731,17 @@ template <int SHAPE> struct Flux {
   }
   static constexpr int total = off(8);
   static_assert(total <= 12 * PG::VB, "the flux fits a spinor field");
+  static_assert(total * 8 <= 2 * PG::VEC * 16, "and the shared vectors");
 };
 template <int SHAPE, int MU> __device__ __forceinline__ int face_row(const PairThread &T) {
   if constexpr (MU == 1) return T.z + 4 * T.t;
   if constexpr (MU == 2) return T.y + 4 * T.t;
   return T.y + 4 * T.z;
 }
-template <typename P> __device__ __forceinline__ cpx<float> pair_at(const void *p, size_t i) {
-  return from_pair<float, P>(((const P *)p)[i]);
-}
-
-// incoming flux of the y, z or t face the row lies on, added to the even
-// (acc[0]) and odd (acc[1]) pair's partial sums
+// incoming flux of the y, z or t face the row lies on, added to the partial
+// sums of the row's pair of parity p
 template <typename S, int SHAPE, int MU>
-__device__ __forceinline__ void flux_in(const PairThread &T, const char *H, const quad *L, PairAcc *acc) {
+__device__ __forceinline__ void flux_in(const PairThread &T, const char *H, const quad *L, int p, PairAcc &acc) {
   using PG = PairGeom<SHAPE>;
   constexpr int R = PG::ROWS, ST = 2 * R, FR = Flux<SHAPE>::FR(MU), PB = sizeof(typename Store<S>::pair_t);
   constexpr int last = MU == 3 ? PG::BT - 1 : 3;
@@ -749,42 +750,38 @@ __device__ __forceinline__ void flux_in(const PairThread &T, const char *H, cons
   if (!up && x != 0) return;
   const char *F = H + (size_t)(up ? Flux<SHAPE>::off(2 * MU) : Flux<SHAPE>::off(2 * MU + 1)) * PB;
   const int fr = face_row<SHAPE, MU>(T);
+  u64 v[6], hv[6];
 #pragma unroll
-  for (int p = 0; p < 2; p++) {
-    u64 v[6], hv[6];
+  for (int c = 0; c < 3; c++) {
+    const quad w = quad_of<S, false>(quad_raw<S, false>(F, ((3 * T.h + c) * 2 + p) * FR + fr));
+    v[2 * c] = w.x;
+    v[2 * c + 1] = w.y;
+  }
+  if (up) {
+    su3_pair<false>(L + 9 * MU * ST + p * R + T.r, ST, v, hv);
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
-      const quad w = quad_ld<S, false>(F, ((3 * T.h + c) * 2 + p) * FR + fr);
-      v[2 * c] = w.x;
-      v[2 * c + 1] = w.y;
-    }
-    if (up) {
-      su3_pair<false>(L + 9 * MU * ST + p * R + T.r, ST, v, hv);
-#pragma unroll
-      for (int i = 0; i < 6; i++) v[i] = hv[i];
-    }
-    acc_add(acc[p].u, v);
-    // the signs of hops_pair: forward hops across the upper face
-    if constexpr (MU == 1) acc_s(acc[p].b, up ? T.sh : T.nsh, v);
-    if constexpr (MU == 2) acc_si(acc[p].a, up ? T.nsh : T.sh, up ? T.sh : T.nsh, v);
-    if constexpr (MU == 3) {
-      if (up) acc_sub(acc[p].a, v);
-      else acc_add(acc[p].a, v);
-    }
+    for (int i = 0; i < 6; i++) v[i] = hv[i];
+  }
+  acc_add(acc.u, v);
+  // the signs of hops_pair: forward hops across the upper face
+  if constexpr (MU == 1) acc_s(acc.b, up ? T.sh : T.nsh, v);
+  if constexpr (MU == 2) acc_si(acc.a, up ? T.nsh : T.sh, up ? T.sh : T.nsh, v);
+  if constexpr (MU == 3) {
+    if (up) acc_sub(acc.a, v);
+    else acc_add(acc.a, v);
   }
 }
 // the x faces: site x = 0 is element A of the row's pair of parity q, site
-// x = 3 element B of the other one
+// x = 3 element B of the other one, whose hop l / hv starts the sums
 template <typename S, int SHAPE>
-__device__ __forceinline__ void flux_in_x(const PairThread &T, const char *H, const quad *L, PairAcc *acc) {
+__device__ __forceinline__ void flux_x(const PairThread &T, const char *H, const quad *L, float *l, float *hv) {
   using P = typename Store<S>::pair_t;
-  using PG = PairGeom<SHAPE>;
-  constexpr int R = PG::ROWS, ST = 2 * R;
-  const char *F0 = H + (size_t)Flux<SHAPE>::off(0) * sizeof(P), *F1 = H + (size_t)Flux<SHAPE>::off(1) * sizeof(P);
-  float c[6], hv[6], w[18], l[6];
+  constexpr int R = PairGeom<SHAPE>::ROWS, ST = 2 * R;
+  float c[6], w[18];
 #pragma unroll
   for (int k = 0; k < 3; k++) {
-    const cpx<float> v = pair_at<P>(F0, (3 * T.h + k) * R + T.r), u = pair_at<P>(F1, (3 * T.h + k) * R + T.r);
+    const P *F = (const P *)H + (3 * T.h + k) * R + T.r;
+    const cpx<float> v = from_pair<float, P>(F[Flux<SHAPE>::off(0)]), u = from_pair<float, P>(F[Flux<SHAPE>::off(1)]);
     c[2 * k] = v.re;
     c[2 * k + 1] = v.im;
     l[2 * k] = u.re;
@@ -798,20 +795,29 @@ __device__ __forceinline__ void flux_in_x(const PairThread &T, const char *H, co
     w[2 * i + 1] = hi(u.y);
   }
   su3_one(w, c, hv);
+}
+// d: chirality half h of the incoming hops into the row's pair of parity p
+template <typename S, int SHAPE>
+__device__ __forceinline__ void flux_sum(const PairThread &T, const char *H, const quad *L, int p,
+                                         const float *l, const float *hv, u64 *d) {
+  PairAcc acc;
+  const bool at0 = T.q == p;   // this parity holds x = 0 (else x = 3)
 #pragma unroll
-  for (int p = 0; p < 2; p++) {
-    const bool at0 = T.q == p;   // this parity holds x = 0 (else x = 3)
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      const float re = at0 ? l[2 * k] : hv[2 * k], im = at0 ? l[2 * k + 1] : hv[2 * k + 1];
-      const u64 vr = at0 ? pk(re, 0.f) : pk(0.f, re), vi = at0 ? pk(im, 0.f) : pk(0.f, im);
-      acc[p].u[2 * k] = add2(acc[p].u[2 * k], vr);
-      acc[p].u[2 * k + 1] = add2(acc[p].u[2 * k + 1], vi);
-      // lower face (backward hop): b += i hv; upper (forward): b -= i hv
-      acc[p].b[2 * k] = at0 ? sub2(acc[p].b[2 * k], vi) : add2(acc[p].b[2 * k], vi);
-      acc[p].b[2 * k + 1] = at0 ? add2(acc[p].b[2 * k + 1], vr) : sub2(acc[p].b[2 * k + 1], vr);
-    }
+  for (int k = 0; k < 3; k++) {
+    const float re = at0 ? l[2 * k] : hv[2 * k], im = at0 ? l[2 * k + 1] : hv[2 * k + 1];
+    const u64 vr = at0 ? pk(re, 0.f) : pk(0.f, re), vi = at0 ? pk(im, 0.f) : pk(0.f, im);
+    acc.u[2 * k] = vr;
+    acc.u[2 * k + 1] = vi;
+    // lower face (backward hop): b = i hv; upper (forward): b = -i hv
+    acc.b[2 * k] = at0 ? neg2(vi) : vi;
+    acc.b[2 * k + 1] = at0 ? vr : neg2(vr);
+    acc.a[2 * k] = acc.a[2 * k + 1] = 0ull;
   }
+  flux_in<S, SHAPE, 1>(T, H, L, p, acc);
+  flux_in<S, SHAPE, 2>(T, H, L, p, acc);
+  flux_in<S, SHAPE, 3>(T, H, L, p, acc);
+  __syncwarp();
+  to_chirality(T, acc, d);
 }
 
 // index of the neighbouring block in direction mu and whether the hop crosses
@@ -823,11 +829,12 @@ template <int MU> __device__ __forceinline__ int block_step(const Geom &g, int b
   sg = (MU == 3 && wrap && g.antiperiodic) ? -1.f : 1.f;
   return b + (v - bc[MU]) * g.bstride[MU];
 }
-// the hop of the correction (shared vectors ve, vo) across the y, z or t face
-// the row lies on, into the neighbouring block's entry
+// the hop of the correction (the row's pair of parity p: u spin h of the upper
+// components, d and e lower spins h and 1 - h) across the y, z or t face the
+// row lies on, into the neighbouring block's entry
 template <typename S, int SHAPE, int MU>
 __device__ __forceinline__ void flux_out(const PairThread &T, const Geom &g, int b, const int *bc, const quad *L,
-                                         const quad *V, char *H) {
+                                         int p, const u64 *u, const u64 *d, const u64 *e, char *H) {
   using PG = PairGeom<SHAPE>;
   constexpr int R = PG::ROWS, ST = 2 * R, FR = Flux<SHAPE>::FR(MU), PB = sizeof(typename Store<S>::pair_t);
   constexpr int last = MU == 3 ? PG::BT - 1 : 3;
@@ -838,43 +845,36 @@ __device__ __forceinline__ void flux_out(const PairThread &T, const Geom &g, int
   const int nb = block_step<MU>(g, b, bc, up, sg);
   char *F = H + ((size_t)nb * Flux<SHAPE>::total + (up ? Flux<SHAPE>::off(2 * MU + 1) : Flux<SHAPE>::off(2 * MU))) * PB;
   const int fr = face_row<SHAPE, MU>(T);
+  u64 chi[6], hv[6];
+  // across the upper face the receiver's backward hop, across the lower its forward one
+  if constexpr (MU == 1) proj_s(u, e, up ? T.nsh : T.sh, chi);
+  if constexpr (MU == 2) proj_si(u, d, up ? T.nsh : T.sh, up ? T.sh : T.nsh, chi);
+  if constexpr (MU == 3) {
 #pragma unroll
-  for (int p = 0; p < 2; p++) {
-    const quad *v = V + p * PG::VEC;
-    u64 u[6], d[6], chi[6], hv[6];
-    ld3(v + spin_at(R, T.h, T.r), R, u);
-    ld3(v + spin_at(R, MU == 1 ? 3 - T.h : 2 + T.h, T.r), R, d);
-    // across the upper face the receiver's backward hop, across the lower its forward one
-    if constexpr (MU == 1) proj_s(u, d, up ? T.nsh : T.sh, chi);
-    if constexpr (MU == 2) proj_si(u, d, up ? T.nsh : T.sh, up ? T.sh : T.nsh, chi);
-    if constexpr (MU == 3) {
-#pragma unroll
-      for (int i = 0; i < 6; i++) chi[i] = up ? add2(u[i], d[i]) : sub2(u[i], d[i]);
-    }
-    if (up) {
-      su3_pair<true>(L + 9 * MU * ST + p * R + T.r, ST, chi, hv);
-#pragma unroll
-      for (int i = 0; i < 6; i++) chi[i] = hv[i];
-    }
-    if constexpr (MU == 3) {
-#pragma unroll
-      for (int i = 0; i < 6; i++) chi[i] = mul2(pk(sg, sg), chi[i]);
-    }
-#pragma unroll
-    for (int c = 0; c < 3; c++)
-      quad_st<S, false>(F, ((3 * T.h + c) * 2 + 1 - p) * FR + fr, chi[2 * c], chi[2 * c + 1]);   // the receiver's parity
+    for (int i = 0; i < 6; i++) chi[i] = up ? add2(u[i], d[i]) : sub2(u[i], d[i]);
   }
+  if (up) {
+    su3_pair<true>(L + 9 * MU * ST + p * R + T.r, ST, chi, hv);
+#pragma unroll
+    for (int i = 0; i < 6; i++) chi[i] = hv[i];
+  }
+  if constexpr (MU == 3) {
+#pragma unroll
+    for (int i = 0; i < 6; i++) chi[i] = mul2(pk(sg, sg), chi[i]);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; c++)
+    quad_st<S, false>(F, ((3 * T.h + c) * 2 + 1 - p) * FR + fr, chi[2 * c], chi[2 * c + 1]);   // the receiver's parity
 }
 template <typename S, int SHAPE>
 __device__ __forceinline__ void flux_out_x(const PairThread &T, const Geom &g, int b, const int *bc, const quad *L,
                                            const quad *V, char *H) {
   using P = typename Store<S>::pair_t;
-  using PG = PairGeom<SHAPE>;
-  constexpr int R = PG::ROWS, ST = 2 * R;
+  constexpr int R = PairGeom<SHAPE>::ROWS, ST = 2 * R;
   float sg, c[6], o[6];
   u64 u[6], e[6];
   // x = 0 (element A of parity q): forward projection to the block below
-  const quad *v = V + T.q * PG::VEC;
+  const quad *v = V + T.q * PairGeom<SHAPE>::VEC;
   ld3(v + spin_at(R, T.h, T.r), R, u);
   ld3(v + spin_at(R, 3 - T.h, T.r), R, e);
   P *F = (P *)H + (size_t)block_step<0>(g, b, bc, false, sg) * Flux<SHAPE>::total + Flux<SHAPE>::off(0);
@@ -882,7 +882,7 @@ __device__ __forceinline__ void flux_out_x(const PairThread &T, const Geom &g, i
   for (int k = 0; k < 3; k++)
     F[(3 * T.h + k) * R + T.r] = to_pair<P, float>(lo(u[2 * k]) - lo(e[2 * k + 1]), lo(u[2 * k + 1]) + lo(e[2 * k]));
   // x = 3 (element B of the other parity): the backward hop into the block above
-  v = V + (1 - T.q) * PG::VEC;
+  v = V + (1 - T.q) * PairGeom<SHAPE>::VEC;
   ld3(v + spin_at(R, T.h, T.r), R, u);
   ld3(v + spin_at(R, 3 - T.h, T.r), R, e);
 #pragma unroll
@@ -920,8 +920,9 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
   quad *L = (quad *)smem, *V = L + PG::LINKS;   // links; vectors: even sites, odd sites
   float *red = (float *)(V + 2 * PG::VEC);
   uint64_t *mbar = (uint64_t *)(red + 24);
-  uint32_t *tmem_at = (uint32_t *)(mbar + 1);
-  const unsigned mbar_s = smem_u32(mbar);
+  uint64_t *fbar = mbar + 1;   // the incoming flux
+  uint32_t *tmem_at = (uint32_t *)(mbar + 2);
+  const unsigned mbar_s = smem_u32(mbar), fbar_s = smem_u32(fbar);
 
   PairThread T;
   {
@@ -948,13 +949,33 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
   constexpr unsigned RQ = QuadStore<S, true>::bytes, RB = 6 * NT * RQ;   // stored residual of a block
   constexpr unsigned FB = Flux<SHAPE>::total * sizeof(P);
 
+  // this thread's clover blocks: chirality h of the even and the odd pair, both
+  // sites' chunks (neighbours in memory) in one 32-byte load
+  uint32_t m0[72], m1[72];
+  clover_pair<P>(cinv + (size_t)b * 36 * PG::VH, PG::VH, 2 * T.r, T.h, m0);
+  // (the odd half of each chunk row)
+  clover_pair<P>(clov + (size_t)b * 36 * PG::VB + (size_t)PG::VH * CP, PG::VB, 2 * T.r, T.h, m1);
+  // The incoming flux of right-hand side r, contiguous, into the place of the
+  // vectors (its reader's prologue then has no trip to L2 in it: read face by
+  // face from global memory it took 8200 clocks of a block's 57500 at
+  // 64x32^3; issued by thread 0)
+  auto flux_issue = [&](int r) {
+    fence_proxy_async();
+    mbar_arrive_expect(fbar, FB);
+    bulk_g2s(V, (const char *)ax.e[r] + (size_t)b * FB, FB, fbar);
+  };
+  // one thread of each warp asks for what comes later
   if (threadIdx.x == 0) {
+    mbar_init(mbar);
+    mbar_init(fbar);
+    fence_proxy_async();
     if constexpr (Store<S>::prec == DD_F32) {
-      mbar_init(mbar);
-      fence_proxy_async();
       mbar_arrive_expect(mbar, LBYTES);
       bulk_g2s(L, (const char *)links + (size_t)b * LBYTES, LBYTES, mbar);
     }
+    if (mode & SAP_HALO_E) flux_issue(rhs0 + rt * tile);
+  }
+  if (threadIdx.x == 64) {
     // the operator tiles of the CTA that starts about when this one ends,
     // requested into L2
     if (const int ni = item + ahead; ahead && ni < G.nitems) {
@@ -967,21 +988,17 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
       const P *nc = (const P *)G.grp[nk].clov + nb * 36 * PG::VB;
       for (int c = 0; c < 36 / CP; c++) prefetch_l2(nc + ((size_t)c * PG::VB + PG::VH) * CP, PG::VH * 16u);
     }
+  }
+  if (threadIdx.x == 32) {
     // fields read later in the block's life, requested into L2
     for (int q = 0; q < tile; q++) {
       const int r = rhs0 + rt * tile + q;
       if (rt * tile + q >= nrhs) break;
       if (!self_zero) prefetch_l2((const char *)rp.out[r] + (size_t)b * PG::VB * SB, PG::VB * SB);
       if (!(mode & SAP_FROM_B)) prefetch_l2((const char *)ax.r[r] + (size_t)b * RB, RB);
-      if (mode & SAP_HALO_E) prefetch_l2((const char *)ax.e[r] + (size_t)b * FB, FB);
+      if ((mode & SAP_HALO_E) && q) prefetch_l2((const char *)ax.e[r] + (size_t)b * FB, FB);
     }
   }
-  // this thread's clover blocks: chirality h of the even and the odd pair, both
-  // sites' chunks (neighbours in memory) in one 32-byte load
-  uint32_t m0[72], m1[72];
-  clover_pair<P>(cinv + (size_t)b * 36 * PG::VH, PG::VH, 2 * T.r, T.h, m0);
-  // (the odd half of each chunk row)
-  clover_pair<P>(clov + (size_t)b * 36 * PG::VB + (size_t)PG::VH * CP, PG::VB, 2 * T.r, T.h, m1);
   if (threadIdx.x < 32) tmem_alloc<PG::TCOLS>(smem_u32(tmem_at));
   tmem_sync();
   // lane threadIdx.x % 128 of the warp's sub-partition, 256 columns per 128 threads
@@ -1000,6 +1017,7 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
     const bool ok = mbar_wait(mbar_s, 0);
     if (__syncthreads_or(!ok)) {   // the staging wait expired: leave as a whole
       wait_expired(timeouts, mbar_s, 0);
+      if (threadIdx.x == 0 && (mode & SAP_HALO_E)) mbar_wait(fbar_s, 0);   // its other copy in flight
       quit = true;
     }
   } else {
@@ -1069,8 +1087,9 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
     for (int rr = 0; rr < tile; rr++) {
       if (rt * tile + rr >= nrhs) break;
       const int r = rhs0 + rt * tile + rr;
+      // ---- the block residual: b or the stored one (zero on even sites after
+      // the first sweep), minus the incoming flux
       u64 r_e[12], r_o[12];
-      // ---- the block residual: b or the stored one, minus the incoming flux
       if (mode & SAP_FROM_B) {
         cpx<float> A[6], B[6];
         auto take = [&](int s, u64 *o) {
@@ -1088,31 +1107,32 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
         const char *res = (const char *)ax.r[r] + (size_t)b * RB;
 #pragma unroll
         for (int i = 0; i < 6; i++) {
-          const quad v = quad_ld<S, true>(res, i * NT + threadIdx.x);
+          const quad v = quad_of<S, true>(quad_raw<S, true>(res, i * NT + threadIdx.x));
           r_o[2 * i] = v.x;
           r_o[2 * i + 1] = v.y;
           r_e[2 * i] = r_e[2 * i + 1] = 0ull;
         }
       }
       if (mode & SAP_HALO_E) {
-        PairAcc acc[2];
+        // (the same for a warp, whose halves exchange below)
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(fbar_s, rr & 1));
+        if (ok) {
+          const char *H = (const char *)V;
+          float l[6], hx[6];
+          u64 d[12];
+          flux_x<S, SHAPE>(T, H, L, l, hx);
+          flux_sum<S, SHAPE>(T, H, L, 0, l, hx, d);
 #pragma unroll
-        for (int p = 0; p < 2; p++)
+          for (int i = 0; i < 12; i++) r_e[i] = sub2(r_e[i], d[i]);
+          flux_sum<S, SHAPE>(T, H, L, 1, l, hx, d);
 #pragma unroll
-          for (int i = 0; i < 6; i++) acc[p].u[i] = acc[p].a[i] = acc[p].b[i] = 0ull;
-        const char *H = (const char *)ax.e[r] + (size_t)b * FB;
-        flux_in_x<S, SHAPE>(T, H, L, acc);
-        flux_in<S, SHAPE, 1>(T, H, L, acc);
-        flux_in<S, SHAPE, 2>(T, H, L, acc);
-        flux_in<S, SHAPE, 3>(T, H, L, acc);
-        __syncwarp();
-        u64 d[12];
-        to_chirality(T, acc[0], d);
-#pragma unroll
-        for (int i = 0; i < 12; i++) r_e[i] = sub2(r_e[i], d[i]);
-        to_chirality(T, acc[1], d);
-#pragma unroll
-        for (int i = 0; i < 12; i++) r_o[i] = sub2(r_o[i], d[i]);
+          for (int i = 0; i < 12; i++) r_o[i] = sub2(r_o[i], d[i]);
+        }
+        // the flux has been read by all (or a wait expired: leave as a whole)
+        if (__syncthreads_or(!ok)) {
+          wait_expired(timeouts, fbar_s, rr & 1);
+          break;
+        }
       }
       // ---- Schur right-hand side, MR steps, reconstruction: half-steps on
       // the even (p = 0) and odd (p = 1) sites in turn, one body of code.
@@ -1198,37 +1218,54 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
           st6(T, V, R, te);
         }
       }
-      // ---- x += e, the residual for the block's next phase
+      // ---- the residual for the block's next phase, the flux of e, x += e (x
+      // is read ahead of the flux, whose arithmetic covers the wait)
+      // (every thread is past its last hops at the sum's barrier; without MR steps there was none)
+      if (nmr == 0) __syncthreads();
+      st6(T, V, R, ee);
+      st6(T, V + PG::VEC, R, eo);
+      cpx<float> xe[2][6], xo[2][6];
+      if (!self_zero) {
+        half_ld<S>(rp.out[r], g, b, 2 * T.r, T.h, xe[0], xe[1]);
+        half_ld<S>(rp.out[r], g, b, PG::VH + 2 * T.r, T.h, xo[0], xo[1]);
+      }
       if (mode & SAP_WRITE_R) {
         char *res = (char *)ax.r[r] + (size_t)b * RB;
 #pragma unroll
         for (int i = 0; i < 6; i++) quad_st<S, true>(res, i * NT + threadIdx.x, rh[2 * i], rh[2 * i + 1]);
       }
-      auto update = [&](int s, const u64 *e) {
-        cpx<float> A[6], B[6];
-        if (!self_zero) half_ld<S>(rp.out[r], g, b, s, T.h, A, B);
-#pragma unroll
-        for (int i = 0; i < 6; i++) {
-          const cpx<float> a = {lo(e[2 * i]), lo(e[2 * i + 1])}, c = {hi(e[2 * i]), hi(e[2 * i + 1])};
-          A[i] = self_zero ? a : cpx<float>{A[i].re + a.re, A[i].im + a.im};
-          B[i] = self_zero ? c : cpx<float>{B[i].re + c.re, B[i].im + c.im};
-        }
-        half_st<S>(rp.out[r], g, b, s, T.h, A, B);
-      };
-      update(2 * T.r, ee);
-      update(PG::VH + 2 * T.r, eo);
       if (mode & SAP_WRITE_E) {
-        __syncthreads();   // the last step's reads of the vectors are done
-        st6(T, V, R, ee);
-        st6(T, V + PG::VEC, R, eo);
         __syncthreads();
         char *H = (char *)ax.e[r];
         flux_out_x<S, SHAPE>(T, g, b, bc, L, V, H);
-        flux_out<S, SHAPE, 1>(T, g, b, bc, L, V, H);
-        flux_out<S, SHAPE, 2>(T, g, b, bc, L, V, H);
-        flux_out<S, SHAPE, 3>(T, g, b, bc, L, V, H);
+#pragma unroll
+        for (int p = 0; p < 2; p++) {
+          const quad *v = V + p * PG::VEC;
+          u64 u[6], d[6], e[6];
+          ld3(v + spin_at(R, T.h, T.r), R, u);
+          ld3(v + spin_at(R, 2 + T.h, T.r), R, d);
+          ld3(v + spin_at(R, 3 - T.h, T.r), R, e);
+          flux_out<S, SHAPE, 1>(T, g, b, bc, L, p, u, d, e, H);
+          flux_out<S, SHAPE, 2>(T, g, b, bc, L, p, u, d, e, H);
+          flux_out<S, SHAPE, 3>(T, g, b, bc, L, p, u, d, e, H);
+        }
+        __syncwarp();
       }
+      auto update = [&](int s, const quad *v, cpx<float>(*x)[6]) {
+        u64 e[12];   // this thread's part of the correction
+        ld6(T, v, R, e);
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+          const cpx<float> a = {lo(e[2 * i]), lo(e[2 * i + 1])}, c = {hi(e[2 * i]), hi(e[2 * i + 1])};
+          x[0][i] = self_zero ? a : cpx<float>{x[0][i].re + a.re, x[0][i].im + a.im};
+          x[1][i] = self_zero ? c : cpx<float>{x[1][i].re + c.re, x[1][i].im + c.im};
+        }
+        half_st<S>(rp.out[r], g, b, s, T.h, x[0], x[1]);
+      };
+      update(2 * T.r, V, xe);
+      update(PG::VH + 2 * T.r, V + PG::VEC, xo);
       __syncthreads();   // the shared vectors are reused by the next right-hand side
+      if (threadIdx.x == 0 && (mode & SAP_HALO_E) && rr + 1 < tile && rt * tile + rr + 1 < nrhs) flux_issue(r + 1);
     }
   }
   // every thread's TMEM accesses are complete; the allocating warp frees
