@@ -738,10 +738,11 @@ template <int SHAPE, int MU> __device__ __forceinline__ int face_row(const PairT
   if constexpr (MU == 2) return T.y + 4 * T.t;
   return T.y + 4 * T.z;
 }
-// incoming flux of the y, z or t face the row lies on, added to the partial
-// sums of the row's pair of parity p
+// incoming flux of the y, z or t face the row lies on, added to the even
+// (acc[0]) and odd (acc[1]) pair's partial sums (the two side by side: their
+// chains of dependent instructions overlap)
 template <typename S, int SHAPE, int MU>
-__device__ __forceinline__ void flux_in(const PairThread &T, const char *H, const quad *L, int p, PairAcc &acc) {
+__device__ __forceinline__ void flux_in(const PairThread &T, const char *H, const quad *L, PairAcc *acc) {
   using PG = PairGeom<SHAPE>;
   constexpr int R = PG::ROWS, ST = 2 * R, FR = Flux<SHAPE>::FR(MU), PB = sizeof(typename Store<S>::pair_t);
   constexpr int last = MU == 3 ? PG::BT - 1 : 3;
@@ -750,25 +751,33 @@ __device__ __forceinline__ void flux_in(const PairThread &T, const char *H, cons
   if (!up && x != 0) return;
   const char *F = H + (size_t)(up ? Flux<SHAPE>::off(2 * MU) : Flux<SHAPE>::off(2 * MU + 1)) * PB;
   const int fr = face_row<SHAPE, MU>(T);
-  u64 v[6], hv[6];
+  u64 v[2][6], hv[2][6];
 #pragma unroll
-  for (int c = 0; c < 3; c++) {
-    const quad w = quad_of<S, false>(quad_raw<S, false>(F, ((3 * T.h + c) * 2 + p) * FR + fr));
-    v[2 * c] = w.x;
-    v[2 * c + 1] = w.y;
-  }
+  for (int p = 0; p < 2; p++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      const quad w = quad_of<S, false>(quad_raw<S, false>(F, ((3 * T.h + c) * 2 + p) * FR + fr));
+      v[p][2 * c] = w.x;
+      v[p][2 * c + 1] = w.y;
+    }
   if (up) {
-    su3_pair<false>(L + 9 * MU * ST + p * R + T.r, ST, v, hv);
 #pragma unroll
-    for (int i = 0; i < 6; i++) v[i] = hv[i];
+    for (int p = 0; p < 2; p++) su3_pair<false>(L + 9 * MU * ST + p * R + T.r, ST, v[p], hv[p]);
+#pragma unroll
+    for (int p = 0; p < 2; p++)
+#pragma unroll
+      for (int i = 0; i < 6; i++) v[p][i] = hv[p][i];
   }
-  acc_add(acc.u, v);
-  // the signs of hops_pair: forward hops across the upper face
-  if constexpr (MU == 1) acc_s(acc.b, up ? T.sh : T.nsh, v);
-  if constexpr (MU == 2) acc_si(acc.a, up ? T.nsh : T.sh, up ? T.sh : T.nsh, v);
-  if constexpr (MU == 3) {
-    if (up) acc_sub(acc.a, v);
-    else acc_add(acc.a, v);
+#pragma unroll
+  for (int p = 0; p < 2; p++) {
+    acc_add(acc[p].u, v[p]);
+    // the signs of hops_pair: forward hops across the upper face
+    if constexpr (MU == 1) acc_s(acc[p].b, up ? T.sh : T.nsh, v[p]);
+    if constexpr (MU == 2) acc_si(acc[p].a, up ? T.nsh : T.sh, up ? T.sh : T.nsh, v[p]);
+    if constexpr (MU == 3) {
+      if (up) acc_sub(acc[p].a, v[p]);
+      else acc_add(acc[p].a, v[p]);
+    }
   }
 }
 // the x faces: site x = 0 is element A of the row's pair of parity q, site
@@ -796,28 +805,33 @@ __device__ __forceinline__ void flux_x(const PairThread &T, const char *H, const
   }
   su3_one(w, c, hv);
 }
-// d: chirality half h of the incoming hops into the row's pair of parity p
+// chirality half h of the incoming hops into the row's even and odd pair
 template <typename S, int SHAPE>
-__device__ __forceinline__ void flux_sum(const PairThread &T, const char *H, const quad *L, int p,
-                                         const float *l, const float *hv, u64 *d) {
-  PairAcc acc;
-  const bool at0 = T.q == p;   // this parity holds x = 0 (else x = 3)
+__device__ __forceinline__ void flux_sum(const PairThread &T, const char *H, const quad *L, u64 *de, u64 *dd) {
+  PairAcc acc[2];
+  float l[6], hv[6];
+  flux_x<S, SHAPE>(T, H, L, l, hv);
 #pragma unroll
-  for (int k = 0; k < 3; k++) {
-    const float re = at0 ? l[2 * k] : hv[2 * k], im = at0 ? l[2 * k + 1] : hv[2 * k + 1];
-    const u64 vr = at0 ? pk(re, 0.f) : pk(0.f, re), vi = at0 ? pk(im, 0.f) : pk(0.f, im);
-    acc.u[2 * k] = vr;
-    acc.u[2 * k + 1] = vi;
-    // lower face (backward hop): b = i hv; upper (forward): b = -i hv
-    acc.b[2 * k] = at0 ? neg2(vi) : vi;
-    acc.b[2 * k + 1] = at0 ? vr : neg2(vr);
-    acc.a[2 * k] = acc.a[2 * k + 1] = 0ull;
+  for (int p = 0; p < 2; p++) {
+    const bool at0 = T.q == p;   // this parity holds x = 0 (else x = 3)
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const float re = at0 ? l[2 * k] : hv[2 * k], im = at0 ? l[2 * k + 1] : hv[2 * k + 1];
+      const u64 vr = at0 ? pk(re, 0.f) : pk(0.f, re), vi = at0 ? pk(im, 0.f) : pk(0.f, im);
+      acc[p].u[2 * k] = vr;
+      acc[p].u[2 * k + 1] = vi;
+      // lower face (backward hop): b = i hv; upper (forward): b = -i hv
+      acc[p].b[2 * k] = at0 ? neg2(vi) : vi;
+      acc[p].b[2 * k + 1] = at0 ? vr : neg2(vr);
+      acc[p].a[2 * k] = acc[p].a[2 * k + 1] = 0ull;
+    }
   }
-  flux_in<S, SHAPE, 1>(T, H, L, p, acc);
-  flux_in<S, SHAPE, 2>(T, H, L, p, acc);
-  flux_in<S, SHAPE, 3>(T, H, L, p, acc);
+  flux_in<S, SHAPE, 1>(T, H, L, acc);
+  flux_in<S, SHAPE, 2>(T, H, L, acc);
+  flux_in<S, SHAPE, 3>(T, H, L, acc);
   __syncwarp();
-  to_chirality(T, acc, d);
+  to_chirality(T, acc[0], de);
+  to_chirality(T, acc[1], dd);
 }
 
 // index of the neighbouring block in direction mu and whether the hop crosses
@@ -906,6 +920,11 @@ __device__ __forceinline__ void flux_out_x(const PairThread &T, const Geom &g, i
   for (int k = 0; k < 3; k++) F[(3 * T.h + k) * R + T.r] = to_pair<P, float>(o[2 * k], o[2 * k + 1]);
 }
 
+// Programmatic launch: this grid lets the next one of the stream start before
+// it ends; the next one waits for it (complete, its writes visible) in grid_wait.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // One colour phase. Work items (lattice group, block of the colour, tile of
 // right-hand sides), one per CTA. mode: SAP_INCR is implied.
 template <typename S, int SHAPE, bool MULTI>
@@ -964,6 +983,9 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
     mbar_arrive_expect(fbar, FB);
     bulk_g2s(V, (const char *)ax.e[r] + (size_t)b * FB, FB, fbar);
   };
+  // The next phase's CTAs may start as soon as every CTA of this one has: up to
+  // grid_wait they touch the operator only, which no phase writes.
+  grid_launch_dependents();
   // one thread of each warp asks for what comes later
   if (threadIdx.x == 0) {
     mbar_init(mbar);
@@ -973,7 +995,10 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
       mbar_arrive_expect(mbar, LBYTES);
       bulk_g2s(L, (const char *)links + (size_t)b * LBYTES, LBYTES, mbar);
     }
-    if (mode & SAP_HALO_E) flux_issue(rhs0 + rt * tile);
+    if (mode & SAP_HALO_E) {
+      grid_wait();
+      flux_issue(rhs0 + rt * tile);
+    }
   }
   if (threadIdx.x == 64) {
     // the operator tiles of the CTA that starts about when this one ends,
@@ -990,7 +1015,8 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
     }
   }
   if (threadIdx.x == 32) {
-    // fields read later in the block's life, requested into L2
+    // fields read later in the block's life, requested into L2 once written
+    grid_wait();
     for (int q = 0; q < tile; q++) {
       const int r = rhs0 + rt * tile + q;
       if (rt * tile + q >= nrhs) break;
@@ -1083,6 +1109,7 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
     }
     int bc[4];
     block_coords(g, b, bc);
+    grid_wait();   // the phases before have written x, the residuals and the flux
 #pragma unroll 1
     for (int rr = 0; rr < tile; rr++) {
       if (rt * tile + rr >= nrhs) break;
@@ -1118,15 +1145,13 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
         const bool ok = __all_sync(0xffffffffu, mbar_wait(fbar_s, rr & 1));
         if (ok) {
           const char *H = (const char *)V;
-          float l[6], hx[6];
-          u64 d[12];
-          flux_x<S, SHAPE>(T, H, L, l, hx);
-          flux_sum<S, SHAPE>(T, H, L, 0, l, hx, d);
+          u64 d[2][12];
+          flux_sum<S, SHAPE>(T, H, L, d[0], d[1]);
 #pragma unroll
-          for (int i = 0; i < 12; i++) r_e[i] = sub2(r_e[i], d[i]);
-          flux_sum<S, SHAPE>(T, H, L, 1, l, hx, d);
-#pragma unroll
-          for (int i = 0; i < 12; i++) r_o[i] = sub2(r_o[i], d[i]);
+          for (int i = 0; i < 12; i++) {
+            r_e[i] = sub2(r_e[i], d[0][i]);
+            r_o[i] = sub2(r_o[i], d[1][i]);
+          }
         }
         // the flux has been read by all (or a wait expired: leave as a whole)
         if (__syncthreads_or(!ok)) {

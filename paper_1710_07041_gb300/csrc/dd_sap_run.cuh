@@ -68,8 +68,22 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
       int mode = sw ? SAP_HALO_E : SAP_FROM_B | (colour ? SAP_HALO_E : 0) | (p.x_is_zero ? 0 : SAP_B32);
       if (!(sw == p.sweeps - 1 && colour == 1)) mode |= SAP_WRITE_E;   // read by the next phase
       if (sw + 1 < p.sweeps) mode |= SAP_WRITE_R;                      // by this colour's next one
-      kern<<<G.nitems, PG::NT, PG::SMEM, st>>>(G, sw ? rp : first, ax, colour, p.x_is_zero && sw == 0, mode,
-                                               p.mr_steps, tile, ahead, sap_timeout_counter());
+      // programmatic launch: a phase's CTAs stage their operator tiles while
+      // the phase before drains, and wait for it (griddepcontrol.wait) before
+      // they read what it wrote
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)G.nitems);
+      cfg.blockDim = dim3(PG::NT);
+      cfg.dynamicSmemBytes = PG::SMEM;
+      cfg.stream = st;
+      cudaLaunchAttribute at = {};
+      at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at.val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      DD_CUDA(cudaLaunchKernelEx(&cfg, kern, G, sw ? rp : first, (const AuxPtrs &)ax, colour,
+                                 (int)(p.x_is_zero && sw == 0), mode, (int)p.mr_steps, tile, ahead,
+                                 sap_timeout_counter()));
       DD_LAUNCHED();
     }
   return DD_OK;
