@@ -994,6 +994,32 @@ inline SapGroups sap_groups(const SapLattice *L, int nl, int tile) {
   return G;
 }
 
+// what is known to be zero in colour phase `colour` of sweep sw, and its
+// residual mode (incr: work fields given)
+struct SapPhase {
+  int self_zero, halo_zero, mode;
+};
+inline SapPhase sap_phase(const dd_sap_params &p, int sw, int colour, bool incr) {
+  // with x = 0 on entry: the first phase sees x = 0 everywhere, the
+  // second still has x = 0 on its own (colour-1) blocks
+  SapPhase f;
+  f.self_zero = (p.x_is_zero && sw == 0) ? 1 : 0;
+  f.halo_zero = (p.x_is_zero && sw == 0 && colour == 0) ? 1 : 0;
+  f.mode = 0;
+  if (incr) {
+    // a block's residual: b on its first solve when x = 0 there (minus the
+    // neighbours' corrections from colour 0 when it is colour 1), the
+    // stored residual from the second sweep on; from a given x the first
+    // sweep forms b - D x. Corrections are read by the next phase,
+    // residuals by the same colour in the next sweep.
+    if (p.x_is_zero && sw == 0) f.mode = SAP_INCR | SAP_FROM_B | (colour ? SAP_HALO_E : 0);
+    else if (sw > 0) f.mode = SAP_INCR | SAP_HALO_E;
+    if (!(sw == p.sweeps - 1 && colour == 1)) f.mode |= SAP_WRITE_E;
+    if (sw + 1 < p.sweeps) f.mode |= SAP_WRITE_R;
+  }
+  return f;
+}
+
 template <typename S, int STAGE, int MINB, int NT, int SHAPE, bool MULTI = false>
 int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
           bool persistent, cudaStream_t st) {
@@ -1028,24 +1054,9 @@ int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
   const AuxPtrs none{};
   for (int sw = 0; sw < p.sweeps; sw++)
     for (int colour = 0; colour < 2; colour++) {
-      // with x = 0 on entry: the first phase sees x = 0 everywhere, the
-      // second still has x = 0 on its own (colour-1) blocks
-      int self_zero = (p.x_is_zero && sw == 0) ? 1 : 0;
-      int halo_zero = (p.x_is_zero && sw == 0 && colour == 0) ? 1 : 0;
-      int mode = 0;
-      if (ax) {
-        // a block's residual: b on its first solve when x = 0 there (minus the
-        // neighbours' corrections from colour 0 when it is colour 1), the
-        // stored residual from the second sweep on; from a given x the first
-        // sweep forms b - D x. Corrections are read by the next phase,
-        // residuals by the same colour in the next sweep.
-        if (p.x_is_zero && sw == 0) mode = SAP_INCR | SAP_FROM_B | (colour ? SAP_HALO_E : 0);
-        else if (sw > 0) mode = SAP_INCR | SAP_HALO_E;
-        if (!(sw == p.sweeps - 1 && colour == 1)) mode |= SAP_WRITE_E;
-        if (sw + 1 < p.sweeps) mode |= SAP_WRITE_R;
-      }
-      kern<<<grid, g.Vb, smem, st>>>(G, rp, ax ? (const AuxPtrs &)*ax : none, colour, self_zero, halo_zero, mode, p.mr_steps, tile,
-                                     sap_timeout_counter());
+      const SapPhase f = sap_phase(p, sw, colour, ax != nullptr);
+      kern<<<grid, g.Vb, smem, st>>>(G, rp, ax ? (const AuxPtrs &)*ax : none, colour, f.self_zero, f.halo_zero, f.mode,
+                                     p.mr_steps, tile, sap_timeout_counter());
       DD_LAUNCHED();
     }
   return DD_OK;

@@ -1,6 +1,7 @@
 // Host side of the Schwarz smoother for one storage precision: launch
 // variants, tuning, graph key (included by dd_sap_<prec>.cu).
 #pragma once
+#include "dd_sap_fine.cuh"
 #include "dd_sap_pair.cuh"
 
 namespace dd {
@@ -89,10 +90,27 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
   return DD_OK;
 }
 
+// one smoother application in the FP64 small-block kernel (dd_sap_fine.cuh)
+template <bool MULTI>
+int sap_fine_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
+               cudaStream_t st) {
+  const SapGroups G = sap_groups(L, nl, tile);
+  const AuxPtrs none{};
+  for (int sw = 0; sw < p.sweeps; sw++)
+    for (int colour = 0; colour < 2; colour++) {
+      const SapPhase f = sap_phase(p, sw, colour, ax != nullptr);
+      k_sap_fine<MULTI><<<G.nitems, fine_threads(L[0].g), fine_smem(L[0].g), st>>>(
+          G, rp, ax ? (const AuxPtrs &)*ax : none, colour, f.self_zero, f.halo_zero, f.mode, p.mr_steps, tile);
+      DD_LAUNCHED();
+    }
+  return DD_OK;
+}
+
 // Launch variants. The 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage run
 // in the packed kernel, whatever the lattice size and right-hand-side count;
 // only a call without work fields (or DD_SAP_INCR=0) takes the unstaged
-// general kernel there. The other blocks and FP64 run in the general kernel:
+// general kernel there. FP64 blocks of 16 and 32 sites run in the small-block
+// kernel. Everything else runs in the general kernel:
 // tiles staged in shared memory with one CTA per SM; tiles staged with two
 // CTAs per SM (fits when the storage is 16-bit); only the links staged, with
 // two CTAs per SM (when the full staging does not fit twice); tiles read
@@ -105,7 +123,7 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
   const Geom &g = L[0].g;
   const bool paired = paired_links(g, L[0].f.prec);
   if (paired && ax && !p.x_is_zero && !ax->r0[0]) ax = nullptr;
-  const bool pair = paired && ax;
+  const bool pair = paired && ax, fine = Store<S>::prec == DD_F64 && fine_block(g);
   const size_t limit = 227 * 1024, half = 113 * 1024;
   const bool stage1 = SapSmem<S>::bytes(g, 1) <= limit;
   const bool stage2 = SapSmem<S>::bytes(g, 1) <= half;
@@ -136,7 +154,7 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
       if (c <= rp.n) tiles[nt++] = c;
   }
   // variant k: layout k % nlay, RHS tile (k / nlay) % nt, persistent grid if
-  // k >= nlay * nt; packed kernel: RHS tile k
+  // k >= nlay * nt; packed and small-block kernels: RHS tile k
   auto run = [&](int k) {
     if constexpr (Store<S>::prec != DD_F64) {
       if (pair) {
@@ -146,6 +164,11 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
         return nl > 1 ? sap_pair_k<S, 2, true>(L, nl, p, rp, *ax, tiles[k], st)
                       : sap_pair_k<S, 2, false>(L, nl, p, rp, *ax, tiles[k], st);
       }
+    }
+    if constexpr (Store<S>::prec == DD_F64) {
+      if (fine)
+        return nl > 1 ? sap_fine_k<true>(L, nl, p, rp, ax, tiles[k], st)
+                      : sap_fine_k<false>(L, nl, p, rp, ax, tiles[k], st);
     }
     const int layout = layouts[k % nlay], tile = tiles[(k / nlay) % nt];
     const bool pers = k >= nlay * nt;
@@ -158,13 +181,13 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
       default: return sap_t<S, 1, 1>(L, nl, p, rp, ax, tile, pers, st);
     }
   };
-  const int nvar = pair ? nt : 2 * nlay * nt;
+  const int nvar = pair || fine ? nt : 2 * nlay * nt;
   int k = 0;
   // the tuner's key: lattice, precision, right-hand-side count, smoother
   // parameters and boundary; a launch over several lattices is tuned once
   // per block shape, precision and total right-hand-side count (a served
   // stream meets ever new mixes of lattices, each would otherwise be tuned)
-  const std::string kind = pair ? "sap-pair" : "sap";
+  const std::string kind = pair ? "sap-pair" : fine ? "sap-fine" : "sap";
   std::string key;
   if (nl == 1) {
     key = tune_key(kind.c_str(), g, L[0].f.prec, rp.n) + "|" + std::to_string(p.sweeps) + "," +
