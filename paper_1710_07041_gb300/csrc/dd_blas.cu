@@ -86,13 +86,17 @@ __global__ void __launch_bounds__(RED_TPB) k_maxpy_norm(const double2 *__restric
   block_reduce<1>(acc, smem, partial + blockIdx.x);
 }
 
-// out[i] = sum_b partial[b][i]: one CTA per value i, fixed summation order
-// (thread t sums blocks t, t + 256, ..., then a fixed-shape tree)
-__global__ void __launch_bounds__(256) k_sum_partials(const double *partial, int nblk, int stride, int nv,
-                                                      double *out) {
+// Sums over the CTAs of a reduction, one CTA per value, fixed summation order
+// (thread t sums blocks t, t + 256, ..., then a fixed-shape tree): value i <
+// nh goes to h[i], value stride - 1 (the norm) to *last and, where inv is
+// given, its reciprocal to *inv - straight to where they are read, with no
+// copies behind the sum (three small copies per Arnoldi step and right-hand
+// side before).
+__global__ void __launch_bounds__(256) k_sum_partials(const double *partial, int nblk, int stride, int nh, double *h,
+                                                      double *last, double *inv) {
   __shared__ double red[256];
-  const int i = blockIdx.x;
-  if (i >= nv) return;
+  const bool norm = (int)blockIdx.x >= nh;
+  const int i = norm ? stride - 1 : blockIdx.x;
   double s = 0;
   for (int b = threadIdx.x; b < nblk; b += 256) s += partial[(size_t)b * stride + i];
   red[threadIdx.x] = s;
@@ -101,7 +105,14 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double *partial, int
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[i] = red[0];
+  if (threadIdx.x == 0) {
+    if (norm) {
+      *last = red[0];
+      if (inv) *inv = 1.0 / red[0];
+    } else {
+      h[i] = red[0];
+    }
+  }
 }
 
 __global__ void k_scale(double2 *y, const double2 *x, double a, size_t n) {
@@ -425,16 +436,14 @@ __global__ void __launch_bounds__(128) k_update_x_df(Geom g, double *x, const vo
 
 Blas::~Blas() {
   if (partial) cudaFree(partial);
-  if (result) cudaFree(result);
   if (hpin) cudaFreeHost(hpin);
 }
 
 int Blas::init(int sms) {
   nblk = sms > 0 ? 4 * sms : 608;
   partial = (double *)pool_dev_alloc(sizeof(double) * (size_t)nblk * (2 * 16 + 1));
-  result = (double *)pool_dev_alloc(sizeof(double) * 256);
   hpin = (double *)pool_host_alloc(sizeof(double) * 256);
-  if (!partial || !result || !hpin) {
+  if (!partial || !hpin) {
     set_error("blas: out of memory for reduction scratch");
     return DD_ENOMEM;
   }
@@ -443,9 +452,8 @@ int Blas::init(int sms) {
 
 void Blas::release_to_pool() {
   pool_dev_free(partial, sizeof(double) * (size_t)nblk * (2 * 16 + 1));
-  pool_dev_free(result, sizeof(double) * 256);
   pool_host_free(hpin, sizeof(double) * 256);
-  partial = result = hpin = nullptr;
+  partial = hpin = nullptr;
 }
 
 int Blas::mdot(const double *V, size_t ldv, int k, const double *w, size_t n, double *h_dev, double *wnorm2_dev,
@@ -461,11 +469,11 @@ int Blas::mdot(const double *V, size_t ldv, int k, const double *w, size_t n, do
       k_mdot<16><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, (const double2 *)w, n, partial);
     int stride = kk <= 4 ? 9 : 33;
     DD_LAUNCHED();
-    k_sum_partials<<<stride, 256, 0, st>>>(partial, nblk, stride, stride, result);
-    DD_LAUNCHED();
-    if (kk > 0) DD_CUDA(cudaMemcpyAsync(h_dev + 2 * i0, result, sizeof(double) * 2 * kk, cudaMemcpyDeviceToDevice, st));
-    if (wnorm2_dev && i0 == 0)
-      DD_CUDA(cudaMemcpyAsync(wnorm2_dev, result + (stride - 1), sizeof(double), cudaMemcpyDeviceToDevice, st));
+    double *wn = i0 == 0 ? wnorm2_dev : nullptr;
+    if (const int n_out = 2 * kk + (wn ? 1 : 0)) {
+      k_sum_partials<<<n_out, 256, 0, st>>>(partial, nblk, stride, 2 * kk, h_dev + 2 * i0, wn, nullptr);
+      DD_LAUNCHED();
+    }
     if (k == 0) break;
   }
   return DD_OK;
@@ -484,7 +492,7 @@ int Blas::maxpy_norm(const double *V, size_t ldv, int k, const double *h_dev, do
     DD_LAUNCHED();
   }
   if (k == 0) return norm2(w, n, norm2_dev, st);
-  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 1, norm2_dev);
+  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 0, nullptr, norm2_dev, nullptr);
   DD_LAUNCHED();
   return DD_OK;
 }
@@ -492,10 +500,8 @@ int Blas::maxpy_norm(const double *V, size_t ldv, int k, const double *h_dev, do
 int Blas::norm2(const double *w, size_t n, double *norm2_dev, cudaStream_t st) {
   k_mdot<4><<<nblk, RED_TPB, 0, st>>>((const double2 *)w, 0, 0, (const double2 *)w, n, partial);
   DD_LAUNCHED();
-  k_sum_partials<<<9, 256, 0, st>>>(partial, nblk, 9, 9, result);
-  DD_LAUNCHED();
-  DD_CUDA(cudaMemcpyAsync(norm2_dev, result + 8, sizeof(double), cudaMemcpyDeviceToDevice, st));
-  return DD_OK;
+  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 9, 0, nullptr, norm2_dev, nullptr);
+  return launched("k_sum_partials");
 }
 
 int Blas::scale(double *y, const double *x, double a, size_t n, cudaStream_t st) {
@@ -525,18 +531,18 @@ int Blas::df_mdot(const float *V, size_t ldv, int k, const float *w, size_t n, d
       k_df_mdot<8><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, (const float4 *)w, n, partial);
     int stride = kk <= 4 ? 9 : 17;
     DD_LAUNCHED();
-    k_sum_partials<<<stride, 256, 0, st>>>(partial, nblk, stride, stride, result);
-    DD_LAUNCHED();
-    if (kk > 0) DD_CUDA(cudaMemcpyAsync(h_dev + 2 * i0, result, sizeof(double) * 2 * kk, cudaMemcpyDeviceToDevice, st));
-    if (wnorm2_dev && i0 == 0)
-      DD_CUDA(cudaMemcpyAsync(wnorm2_dev, result + (stride - 1), sizeof(double), cudaMemcpyDeviceToDevice, st));
+    double *wn = i0 == 0 ? wnorm2_dev : nullptr;
+    if (const int n_out = 2 * kk + (wn ? 1 : 0)) {
+      k_sum_partials<<<n_out, 256, 0, st>>>(partial, nblk, stride, 2 * kk, h_dev + 2 * i0, wn, nullptr);
+      DD_LAUNCHED();
+    }
     if (k == 0) break;
   }
   return DD_OK;
 }
 
 int Blas::df_maxpy_norm(const float *V, size_t ldv, int k, const double *h_dev, float *w, size_t n, double *norm2_dev,
-                        cudaStream_t st, const float *w32, int lvb, const double *scl) {
+                        cudaStream_t st, const float *w32, int lvb, const double *scl, double *inv2_dev) {
   if (k == 0) return df_mdot(V, ldv, 0, w, n, nullptr, norm2_dev, st, w32, lvb);
   for (int i0 = 0; i0 < k; i0 += 8) {
     int kk = k - i0 < 8 ? k - i0 : 8;
@@ -556,7 +562,7 @@ int Blas::df_maxpy_norm(const float *V, size_t ldv, int k, const double *h_dev, 
       k_df_maxpy_norm<8><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, hi, (float4 *)w, n, partial, nullptr, 0, si);
     DD_LAUNCHED();
   }
-  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 1, norm2_dev);
+  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 0, nullptr, norm2_dev, inv2_dev);
   return launched("k_sum_partials");
 }
 

@@ -8,7 +8,6 @@ namespace dd {
 struct Blas {
   int nblk = 0;
   double *partial = nullptr;  // [nblk][33] per-block partial sums
-  double *result = nullptr;   // [256] reduced values
   double *hpin = nullptr;     // pinned host mirror
   ~Blas();
   int init(int sms);
@@ -32,9 +31,10 @@ struct Blas {
               cudaStream_t st, const float *w32 = nullptr, int lvb = 0);
   // scl (device, optional): the coefficients h_i are multiplied by scl[i]
   // before the update (for a basis stored as v_i = s_i V_i with h_i = <V_i, w>
-  // the caller passes s_i^2)
+  // the caller passes s_i^2); inv2_dev (device, optional) receives 1 / *norm2
   int df_maxpy_norm(const float *V, size_t ldv, int k, const double *h_dev, float *w, size_t n, double *norm2_dev,
-                    cudaStream_t st, const float *w32 = nullptr, int lvb = 0, const double *scl = nullptr);
+                    cudaStream_t st, const float *w32 = nullptr, int lvb = 0, const double *scl = nullptr,
+                    double *inv2_dev = nullptr);
   int set_double(double *dev, double v, cudaStream_t st);   // *dev = v, stream-ordered
   int df_scale(float *y, const float *x, double a, size_t n, cudaStream_t st);
   int f64_to_df(float *y, const double *x, double a, size_t n, cudaStream_t st);  // y = a x

@@ -140,7 +140,6 @@ extern "C" int dd_solve_noalloc(dd_op_t opp, const dd_solve_params *p, const dou
   Blas bl;
   bl.nblk = nblk;
   bl.partial = cv.take<double>(sizeof(double) * (size_t)nblk * 33);
-  bl.result = cv.take<double>(sizeof(double) * 256);
   double *hd = cv.take<double>(sizeof(double) * 136);
   double *yd = cv.take<double>(sizeof(double) * 2 * MAXM);
   double *Vb = cv.take<double>((size_t)(m + 1) * f64_al);
@@ -156,7 +155,7 @@ extern "C" int dd_solve_noalloc(dd_op_t opp, const dd_solve_params *p, const dou
   // the Blas object borrows scratch; detach it before it goes out of scope
   struct Detach {
     Blas &b;
-    ~Detach() { b.partial = b.result = nullptr; }
+    ~Detach() { b.partial = nullptr; }
   } detach{bl};
 
   const double sigma = std::sqrt(24.0 * (double)g.V);

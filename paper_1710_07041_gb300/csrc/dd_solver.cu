@@ -394,13 +394,15 @@ int BatchSolver::mdot(Slot *s, int kk, double *h, double *wn2, bool from32) {
   return blas_.mdot(s->Vb, n, kk, s->w, n, h, wn2, st_);
 }
 
+// (for a double-float basis also s->sdev[kk] = 1 / |w|^2, the next vector's
+// update coefficient)
 int BatchSolver::maxpy(Slot *s, int kk, const double *h, double *wn2, bool from32) {
   const Geom &g = s->op->lat->g;
   const size_t n = (size_t)g.V * 12;
   const int lvb = g.lbd[0] + g.lbd[1] + g.lbd[2] + g.lbd[3];
   if (df_)
     return blas_.df_maxpy_norm((const float *)s->Vb, n, kk, h, (float *)(s->Vb + 2 * n * kk), n, wn2, st_,
-                               from32 ? (const float *)s->zt : nullptr, lvb, s->sdev);
+                               from32 ? (const float *)s->zt : nullptr, lvb, s->sdev, s->sdev + kk);
   return blas_.maxpy_norm(s->Vb, n, kk, h, s->w, n, wn2, st_);
 }
 
@@ -537,13 +539,9 @@ int BatchSolver::arnoldi_step(std::vector<Slot *> &A) {
     const size_t n = (size_t)s.op->lat->g.V * 12;
     for (int q = 0; q <= j; q++) s.H[(size_t)q * m + j] = hcol[i][q];
     if (hn > 0) {
-      if (df_) {   // v_{j+1} = Vb_{j+1} / hn, kept as a scale
-        s.scl[j + 1] = 1.0 / hn;
-        rc = blas_.set_double(s.sdev + j + 1, 1.0 / (hn * hn), st_);
-      } else {
-        rc = blas_.scale(s.Vb + 2 * n * (j + 1), s.w, 1.0 / hn, n, st_);
-      }
-      if (rc) return rc;
+      // v_{j+1} = Vb_{j+1} / hn: kept as a scale (double-float; its square is on the device already)
+      if (df_) s.scl[j + 1] = 1.0 / hn;
+      else if ((rc = blas_.scale(s.Vb + 2 * n * (j + 1), s.w, 1.0 / hn, n, st_))) return rc;
     }
     for (int q = 0; q < j; q++) {
       cd a = s.H[(size_t)q * m + j], c2 = s.H[(size_t)(q + 1) * m + j];
