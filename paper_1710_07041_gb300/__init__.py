@@ -157,21 +157,32 @@ def _check(rc: int, what: str):
         raise DDError(rc, f"{what}: {lib().dd_last_error().decode()}")
 
 
-def _stream_ptr(stream):
+_torch = None
+
+
+def _stream_ptr(stream) -> int:
+    """The stream's address; None: torch's current stream (read as a raw
+    pointer, without building a Stream object: a smallest operator product is
+    a few microseconds)."""
     if stream is None:
-        import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        global _torch
+        if _torch is None:
+            import torch as _torch_module
+            _torch_module.cuda.current_stream()   # initialises CUDA
+            _torch = _torch_module
+        return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
-def _ptr(t) -> ctypes.c_void_p:
+def _ptr(t) -> int:
+    """Address of a contiguous array or tensor (ctypes converts it)."""
     if isinstance(t, np.ndarray):
         assert t.flags.c_contiguous
-        return ctypes.c_void_p(t.ctypes.data)
+        return t.ctypes.data
     assert t.is_contiguous()
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Handle:
@@ -320,8 +331,8 @@ def sap_smooth_multi(items, sweeps: int, mr_steps: int, x_is_zero: bool = True, 
     n = len(items)
     ops = (ctypes.c_void_p * n)(*[op.handle for op, _, _, _ in items])
     nrhs = (ctypes.c_int * n)(*[int(k) for _, _, _, k in items])
-    bs = (ctypes.c_void_p * n)(*[_ptr(b).value for _, b, _, _ in items])
-    xs = (ctypes.c_void_p * n)(*[_ptr(x).value for _, _, x, _ in items])
+    bs = (ctypes.c_void_p * n)(*[_ptr(b) for _, b, _, _ in items])
+    xs = (ctypes.c_void_p * n)(*[_ptr(x) for _, _, x, _ in items])
     p = SapParams(sweeps, mr_steps, int(bool(x_is_zero)), rhs_tile)
     _check(lib().dd_sap_smooth_multi(n, ops, nrhs, ctypes.byref(p), bs, xs, _stream_ptr(stream)),
            "dd_sap_smooth_multi")

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "dd_internal.cuh"
+#include "dd_pool.cuh"
 
 namespace dd {
 
@@ -446,11 +447,7 @@ int dd_sap_smooth(dd_op_t opp, const dd_sap_params *p, const void *b, void *x, i
   // them, e.g. when this allocation fails, every phase forms b - D x)
   cudaStream_t st = (cudaStream_t)stream;
   const Geom &g = op->lat->g;
-  void *aux = nullptr;
-  if (cudaMallocAsync(&aux, (size_t)nrhs * sap_work_bytes(g, op->fp.prec, p->x_is_zero), st) != cudaSuccess) {
-    cudaGetLastError();
-    aux = nullptr;
-  }
+  void *aux = pool_stream_alloc((size_t)nrhs * sap_work_bytes(g, op->fp.prec, p->x_is_zero), st);
   int rc = launch_sap(g, op->fp, *p, b, x, nrhs, st, aux);
   if (aux) cudaFreeAsync(aux, st);
   return rc;
@@ -483,11 +480,7 @@ int dd_sap_smooth_multi(int nops, const dd_op_t *ops, const int *nrhs, const dd_
   }
   // work fields of the incremental colour residual, stream-ordered
   cudaStream_t st = (cudaStream_t)stream;
-  char *aux = nullptr;
-  if (cudaMallocAsync((void **)&aux, aux_bytes, st) != cudaSuccess) {
-    cudaGetLastError();
-    aux = nullptr;
-  }
+  char *aux = (char *)pool_stream_alloc(aux_bytes, st);
   SapWork ax;
   for (int k = 0, i = 0; aux && k < nops; k++) {
     const size_t fb = (size_t)lats[k].g.V * spinor_site_bytes(lats[k].f.prec);

@@ -224,8 +224,12 @@ int dirac_t(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st)
     return v >= 4 ? shape(v - 4, std::true_type{}) : shape(v, std::false_type{});
   };
   int v = 0;
-  int rc = tuned_variant(tune_key("dirac", g, f.prec, p.n), DIRAC_VARIANTS, run, st, &v);
-  if (rc) return rc;
+  const TuneFast fast = tune_fast_key(1, g, f.prec, p.n);
+  if (!tune_fast_find(fast, &v)) {
+    const std::string key = tune_key("dirac", g, f.prec, p.n);
+    if (int rc = tuned_variant(key, DIRAC_VARIANTS, run, st, &v)) return rc;
+    if (!getenv("DD_TUNE_VARIANT") && tune_lookup(key) == v) tune_fast_store(fast, v);
+  }
   return run(v);
 }
 

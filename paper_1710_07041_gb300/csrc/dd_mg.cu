@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "dd_mg.cuh"
+#include "dd_pool.cuh"
 
 namespace dd {
 namespace {
@@ -659,31 +660,26 @@ __global__ void k_add_scale(const float4 *a, const float4 *b, float4 *y, float s
 // ---------------------------------------------------------------- MgWork
 MgWork::~MgWork() {
   for (auto &kv : graphs) cudaGraphExecDestroy(kv.second.first);
-  void *p[] = {Vc, w, w2, cb, ce, xf, rf, tf, tin, tout, se, sr, partial, pnorm, st};
-  for (void *q : p)
-    if (q) cudaFree(q);
+  for (auto &b : bufs) {
+    if (cache) pool_dev_free(*b.first, b.second);
+    else if (*b.first) cudaFree(*b.first);
+  }
 }
 
 int MgWork::init(const Mg *mg) {
   const Geom &g = mg->op->lat->g;
   nc = (size_t)g.nblocks * 2 * mg->N;
-  const size_t f32 = (size_t)g.V * 24 * 4, fp = (size_t)g.V * spinor_site_bytes(mg->op->prec);
+  const size_t f32 = (size_t)g.V * 24 * 4, fp = (size_t)g.V * spinor_site_bytes(mg->op->prec), cv = sizeof(float2) * nc;
   const int kmax = mg->p.coarse_max_iter;
-  bool ok = cudaMalloc(&Vc, sizeof(float2) * nc * (kmax + 1)) == cudaSuccess &&
-            cudaMalloc(&w, sizeof(float2) * nc) == cudaSuccess && cudaMalloc(&w2, sizeof(float2) * nc) == cudaSuccess &&
-            cudaMalloc(&cb, sizeof(float2) * nc) == cudaSuccess &&
-            cudaMalloc(&ce, sizeof(float2) * nc) == cudaSuccess && cudaMalloc(&xf, f32) == cudaSuccess &&
-            cudaMalloc(&rf, f32) == cudaSuccess && cudaMalloc(&tf, f32) == cudaSuccess &&
-            cudaMalloc(&tin, fp) == cudaSuccess && cudaMalloc(&tout, fp) == cudaSuccess &&
-            cudaMalloc(&se, fp) == cudaSuccess && cudaMalloc(&sr, fp) == cudaSuccess &&
-            cudaMalloc(&partial, sizeof(float2) * cg_chunks(nc) * 65) == cudaSuccess &&
-            cudaMalloc(&pnorm, sizeof(float) * cg_partials(nc)) == cudaSuccess &&
-            cudaMalloc(&st, sizeof(CgState)) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
-    set_error("mg: out of device memory for the coarse-solve workspace");
-    return DD_ENOMEM;
-  }
+  bufs = {{(void **)&Vc, cv * (kmax + 1)}, {(void **)&w, cv}, {(void **)&w2, cv}, {(void **)&cb, cv}, {(void **)&ce, cv},
+          {(void **)&xf, f32}, {(void **)&rf, f32}, {(void **)&tf, f32}, {&tin, fp}, {&tout, fp}, {&se, fp}, {&sr, fp},
+          {(void **)&partial, sizeof(float2) * cg_chunks(nc) * 65}, {(void **)&pnorm, sizeof(float) * cg_partials(nc)},
+          {&st, sizeof(CgState)}};
+  for (auto &b : bufs)
+    if (!(*b.first = pool_dev_alloc(b.second))) {
+      set_error("mg: out of device memory for the coarse-solve workspace");
+      return DD_ENOMEM;
+    }
   return cuda_fail(cudaMemset(st, 0, sizeof(CgState)), "mg workspace");   // reduction counter = 0
 }
 
@@ -804,14 +800,17 @@ static int mg_enqueue(const Mg *mg, MgWork &W, const float *r, float *x, cudaStr
 // second application on with the same (r, x, scale) it runs as one CUDA graph
 // captured on that call. The first application of a workspace runs eagerly,
 // so that the autotuner has chosen the fine-grid kernels' variants before any
-// capture. DD_MG_GRAPHS=0 disables the graphs; a stream under capture by the
-// caller, or the legacy stream, gets the launches directly.
+// capture. Not in a solve (use_graphs false): there x is one of the m slots of
+// Z, and capturing and instantiating a graph for each of them in every solve
+// took longer than its replays saved. DD_MG_GRAPHS=0 disables the graphs; a
+// stream under capture by the caller, or the legacy stream, gets the launches
+// directly.
 int mg_apply(const Mg *mg, MgWork &W, const float *r, float *x, cudaStream_t st, float scale) {
   NvtxRange range("dd:mg_apply");
   const char *env = getenv("DD_MG_GRAPHS");
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(st, &cap);
-  if ((env && env[0] == '0') || cap != cudaStreamCaptureStatusNone || st == 0 || !W.warm) {
+  if (!W.use_graphs || (env && env[0] == '0') || cap != cudaStreamCaptureStatusNone || st == 0 || !W.warm) {
     W.warm = true;
     return mg_enqueue(mg, W, r, x, st, scale);
   }

@@ -3,6 +3,7 @@
 #include <map>
 #include <string>
 #include <utility>
+#include <vector>
 
 #include "dd_blas.cuh"
 
@@ -23,6 +24,9 @@ struct MgWork {
   float *pnorm = nullptr;
   void *st = nullptr;          // coarse GMRES control state (device)
   bool warm = false;           // one eager application done (variants tuned)
+  bool use_graphs = true;      // replay an application on the same (r, x) as a graph
+  bool cache = false;          // hand the buffers to the workspace cache on destruction (no queued work uses them)
+  std::vector<std::pair<void **, size_t>> bufs;   // the buffers above with their sizes
   std::map<std::string, std::pair<cudaGraphExec_t, size_t>> graphs;   // (r, x, scale) -> graph, nodes
   ~MgWork();
   int init(const Mg *mg);

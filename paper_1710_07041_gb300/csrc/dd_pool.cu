@@ -7,7 +7,12 @@
 // handed to the next solver that asks for the same size. The cache is
 // bounded (half the device memory, 64 MB of pinned host memory); a device
 // allocation that fails releases the cache and is tried once more, and
-// dd_release_workspace() gives everything back.
+// dd_release_workspace() gives everything back. Work fields of single calls
+// (the smoother's) come from a stream-ordered memory pool per device that
+// keeps up to STREAM_KEEP bytes between calls: the device's default pool
+// gives its memory back at every synchronisation, and the next call mapped it
+// again (0.9 ms in front of a 3 ms smoother application on 64x32^3, 0.2 ms in
+// front of a 0.16 ms one on 16x8^3).
 #include <map>
 #include <mutex>
 #include <utility>
@@ -48,6 +53,17 @@ void *take(std::multimap<std::pair<int, size_t>, void *> &m, int dev, size_t n) 
 }
 
 constexpr size_t HOST_CAP = 64u << 20;
+constexpr size_t STREAM_KEEP = (size_t)4 << 30;
+
+// the stream-ordered pools by device (created at first use, never destroyed)
+struct StreamPools {
+  std::mutex mu;
+  std::map<int, cudaMemPool_t> of;
+};
+StreamPools &stream_pools() {
+  static StreamPools *p = new StreamPools;
+  return *p;
+}
 
 }  // namespace
 
@@ -120,12 +136,55 @@ void pool_host_free(void *p, size_t n) {
   cudaFreeHost(p);
 }
 
+void *pool_stream_alloc(size_t n, cudaStream_t st) {
+  if (n == 0) return nullptr;
+  const int d = current_device();
+  cudaMemPool_t mp = nullptr;
+  {
+    StreamPools &S = stream_pools();
+    std::lock_guard<std::mutex> lk(S.mu);
+    auto it = S.of.find(d);
+    if (it == S.of.end()) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = d;
+      uint64_t keep = STREAM_KEEP;
+      if (cudaMemPoolCreate(&mp, &props) != cudaSuccess ||
+          cudaMemPoolSetAttribute(mp, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        if (mp) cudaMemPoolDestroy(mp);
+        mp = nullptr;   // the device's default pool
+      }
+      it = S.of.emplace(d, mp).first;
+    }
+    mp = it->second;
+  }
+  void *p = nullptr;
+  const cudaError_t e = mp ? cudaMallocFromPoolAsync(&p, n, mp, st) : cudaMallocAsync(&p, n, st);
+  if (e == cudaSuccess) return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
 size_t pool_cached_bytes() {
   const int d = current_device();
   Pool &P = pool();
-  std::lock_guard<std::mutex> lk(P.mu);
-  auto it = P.dev_bytes.find(d);
-  return it == P.dev_bytes.end() ? 0 : it->second;
+  size_t n = 0;
+  {
+    std::lock_guard<std::mutex> lk(P.mu);
+    auto it = P.dev_bytes.find(d);
+    if (it != P.dev_bytes.end()) n = it->second;
+  }
+  StreamPools &S = stream_pools();
+  std::lock_guard<std::mutex> lk(S.mu);
+  auto it = S.of.find(d);
+  uint64_t reserved = 0, used = 0;
+  if (it != S.of.end() && it->second &&
+      cudaMemPoolGetAttribute(it->second, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+      cudaMemPoolGetAttribute(it->second, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+    n += (size_t)(reserved - used);
+  return n;
 }
 
 void pool_release() {
@@ -145,6 +204,10 @@ void pool_release() {
   }
   cudaSetDevice(cur);
   for (auto &e : host) cudaFreeHost(e.second);
+  StreamPools &S = stream_pools();
+  std::lock_guard<std::mutex> lk(S.mu);
+  for (auto &e : S.of)
+    if (e.second) cudaMemPoolTrimTo(e.second, 0);
 }
 
 }  // namespace dd

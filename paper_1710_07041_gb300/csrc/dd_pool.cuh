@@ -2,6 +2,8 @@
 // size) and pinned host buffers. pool_dev_free / pool_host_free require that
 // no queued GPU work still uses the buffer.
 #pragma once
+#include <cuda_runtime.h>
+
 #include <cstddef>
 
 namespace dd {
@@ -10,5 +12,8 @@ void pool_dev_free(void *p, size_t bytes);
 void *pool_host_alloc(size_t bytes);
 void pool_host_free(void *p, size_t bytes);
 size_t pool_cached_bytes();   // device bytes cached for the current device
+// stream-ordered device memory for the work fields of one call (n bytes, freed
+// with cudaFreeAsync on the same stream); nullptr where there is none
+void *pool_stream_alloc(size_t n, cudaStream_t st);
 void pool_release();          // free every cached buffer
 }  // namespace dd

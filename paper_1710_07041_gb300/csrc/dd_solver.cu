@@ -147,7 +147,10 @@ BatchSolver::~BatchSolver() {
     if (hpin_) cudaFreeHost(hpin_);
     if (ypin_) cudaFreeHost(ypin_);
   }
-  for (auto &s : slots_) delete s.mgw;
+  for (auto &s : slots_) {
+    if (s.mgw) s.mgw->cache = cache_;
+    delete s.mgw;
+  }
   for (auto &e : ev_)
     if (e) cudaEventDestroy(e);
   if (own_stream_) cudaStreamDestroy(st_);
@@ -171,6 +174,7 @@ int BatchSolver::init() {
     if (rc) return rc;
     if (p_.mg) {
       s.mgw = new (std::nothrow) MgWork;
+      if (s.mgw) s.mgw->use_graphs = false;
       int rc = s.mgw ? s.mgw->init((const Mg *)p_.mg) : DD_ENOMEM;
       if (rc) return rc;
     }

@@ -165,4 +165,49 @@ int tune_lookup(const std::string &key) {
   return it == g_cache.end() ? -1 : it->second;
 }
 
+namespace {
+struct FastEntry {
+  TuneFast k;
+  int chosen = -1;
+};
+thread_local FastEntry t_fast[64];
+unsigned fast_slot(const TuneFast &k) {
+  unsigned h = 2166136261u;
+  const unsigned char *p = (const unsigned char *)&k;
+  for (size_t i = 0; i < sizeof k; i += 4) {
+    unsigned w;
+    memcpy(&w, p + i, 4);
+    h = (h ^ w) * 16777619u;
+  }
+  return (h ^ (h >> 15)) % 64;
+}
+}  // namespace
+
+TuneFast tune_fast_key(int kind, const Geom &g, int prec, int nrhs) {
+  TuneFast k;
+  memset(&k, 0, sizeof k);
+  k.kind = kind;
+  k.prec = prec;
+  k.nrhs = nrhs;
+  cudaGetDevice(&k.dev);
+  for (int mu = 0; mu < 4; mu++) {
+    k.L[mu] = g.L[mu];
+    k.bd[mu] = g.bd[mu];
+  }
+  return k;
+}
+
+bool tune_fast_find(const TuneFast &k, int *chosen) {
+  const FastEntry &e = t_fast[fast_slot(k)];
+  if (e.chosen < 0 || memcmp(&e.k, &k, sizeof k) || getenv("DD_TUNE_VARIANT")) return false;
+  *chosen = e.chosen;
+  return true;
+}
+
+void tune_fast_store(const TuneFast &k, int chosen) {
+  FastEntry &e = t_fast[fast_slot(k)];
+  e.k = k;
+  e.chosen = chosen;
+}
+
 }  // namespace dd

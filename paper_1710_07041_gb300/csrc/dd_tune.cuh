@@ -12,6 +12,16 @@ std::string tune_key(const char *kind, const Geom &g, int prec, int nrhs);
 int tuned_variant(const std::string &key, int nvariants, const std::function<int(int)> &run, cudaStream_t st,
                   int *chosen);
 int tune_lookup(const std::string &key);  // cached choice or -1
+// Choices already made, by a plain key and without a lock: a call whose
+// variant is known then builds no string (a quarter of the host time of the
+// smallest operator product). Per thread; a miss goes through tuned_variant.
+struct TuneFast {
+  int kind, dev, prec, nrhs;
+  int L[4], bd[4];
+};
+bool tune_fast_find(const TuneFast &k, int *chosen);   // false also where DD_TUNE_VARIANT forces one
+void tune_fast_store(const TuneFast &k, int chosen);
+TuneFast tune_fast_key(int kind, const Geom &g, int prec, int nrhs);
 
 // Launches without set-up work, for calls that promise to allocate nothing
 // (dd_solve_noalloc). While a DirectLaunch object lives on a thread, that
