@@ -3,6 +3,8 @@
 // numbers (all FP64 fields share one element order). Reductions are two-stage
 // with a fixed grid and a fixed summation order, so every result is
 // bit-reproducible and independent of what else runs on the device.
+#include <algorithm>
+
 #include "dd_blas.cuh"
 #include "dd_pool.cuh"
 
@@ -88,12 +90,10 @@ __global__ void __launch_bounds__(RED_TPB) k_maxpy_norm(const double2 *__restric
 
 // Sums over the CTAs of a reduction, one CTA per value, fixed summation order
 // (thread t sums blocks t, t + 256, ..., then a fixed-shape tree): value i <
-// nh goes to h[i], value stride - 1 (the norm) to *last and, where inv is
-// given, its reciprocal to *inv - straight to where they are read, with no
-// copies behind the sum (three small copies per Arnoldi step and right-hand
-// side before).
+// nh goes to h[i], value stride - 1 (the norm) to *last: straight to where
+// they are read, with no copies behind the sum.
 __global__ void __launch_bounds__(256) k_sum_partials(const double *partial, int nblk, int stride, int nh, double *h,
-                                                      double *last, double *inv) {
+                                                      double *last) {
   __shared__ double red[256];
   const bool norm = (int)blockIdx.x >= nh;
   const int i = norm ? stride - 1 : blockIdx.x;
@@ -108,7 +108,6 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double *partial, int
   if (threadIdx.x == 0) {
     if (norm) {
       *last = red[0];
-      if (inv) *inv = 1.0 / red[0];
     } else {
       h[i] = red[0];
     }
@@ -230,13 +229,28 @@ __device__ __forceinline__ float4 w_at(const float4 *w, const float *w32, size_t
   return w[e];
 }
 
-// partial[blk] = this block's sums of conj(V_i) w (i < k) and |w|^2, as doubles.
-// Two elements per thread and iteration keep more loads in flight. W32: w is
-// read from the FP32 field w32 (see w_from_f32).
-template <int KMAX, bool W32 = false>
-__global__ void __launch_bounds__(RED_TPB) k_df_mdot(const float4 *__restrict__ V, size_t ldv, int k,
-                                                     const float4 *__restrict__ w, size_t n, double *partial,
-                                                     const float *__restrict__ w32 = nullptr, int lvb = 0) {
+// Right-hand sides of one launch (grid.y): the vectors, coefficients and
+// outputs of each. A slot's sums depend on its own vectors and the fixed
+// grid.x only, so it gets the same bits alone and in any batch.
+constexpr int DF_BATCH = 16;
+struct DfBatch {
+  DfSlot s[DF_BATCH];
+};
+// the slot's vectors of the chunk of 8 from i0: their number (0: none left)
+__device__ __forceinline__ int df_chunk(const DfSlot &t, int i0) { return t.k - i0 < 8 ? t.k - i0 : 8; }
+
+// partial[blk] = this block's sums of conj(V_i) w (i0 <= i < i0 + 8) and |w|^2,
+// as doubles. Two elements per thread and iteration keep more loads in
+// flight. W32: w is read from the FP32 field w32 (see w_from_f32).
+template <int KMAX, bool W32>
+__global__ void __launch_bounds__(RED_TPB) k_df_mdot(const DfBatch B, int i0) {
+  const DfSlot &t = B.s[blockIdx.y];
+  const int k = df_chunk(t, i0);
+  if (k <= 0 && i0 > 0) return;
+  const float4 *__restrict__ V = (const float4 *)t.V + (size_t)i0 * t.ldv, *__restrict__ w = (const float4 *)t.w;
+  const float *__restrict__ w32 = t.w32;
+  const size_t n = t.n, ldv = t.ldv;
+  const int lvb = t.lvb;
   __shared__ double smem[(2 * KMAX + 1) * 32];
   df acc[2 * KMAX + 1];
 #pragma unroll
@@ -272,22 +286,29 @@ __global__ void __launch_bounds__(RED_TPB) k_df_mdot(const float4 *__restrict__ 
       }
     }
   }
-  block_reduce_df<2 * KMAX + 1>(acc, smem, partial + (size_t)blockIdx.x * (2 * KMAX + 1));
+  block_reduce_df<2 * KMAX + 1>(acc, smem, t.partial + (size_t)blockIdx.x * (2 * KMAX + 1));
 }
 
-// w -= sum_i h_i V_i (h complex doubles on the device); partial[blk] = |w|^2.
-// W32: the input w is read from the FP32 field w32 (see w_from_f32) and the
-// result written to w.
-template <int KMAX, bool W32 = false>
-__global__ void __launch_bounds__(RED_TPB) k_df_maxpy_norm(const float4 *__restrict__ V, size_t ldv, int k,
-                                                           const double2 *__restrict__ h, float4 *w, size_t n,
-                                                           double *partial, const float *__restrict__ w32 = nullptr,
-                                                           int lvb = 0, const double *__restrict__ scl = nullptr) {
+// w -= sum_i h_i V_i over the chunk of 8 from i0 (h complex doubles on the
+// device, times scl[i] where given); partial[blk] = |w|^2. W32: the first
+// chunk reads w from the FP32 field w32 (see w_from_f32) and writes it to w.
+template <int KMAX, bool W32>
+__global__ void __launch_bounds__(RED_TPB) k_df_maxpy_norm(const DfBatch B, int i0) {
+  const DfSlot &t = B.s[blockIdx.y];
+  const int k = df_chunk(t, i0);
+  if (k <= 0) return;
+  const float4 *__restrict__ V = (const float4 *)t.V + (size_t)i0 * t.ldv;
+  float4 *w = (float4 *)t.w;
+  const float *__restrict__ w32 = t.w32;
+  const double2 *__restrict__ h = (const double2 *)t.h + i0;
+  const double *__restrict__ scl = t.scl ? t.scl + i0 : nullptr;
+  const size_t n = t.n, ldv = t.ldv;
+  const int lvb = t.lvb;
   __shared__ double smem[32];
   __shared__ float4 hs[KMAX];   // (re_hi, im_hi, re_lo, im_lo)
   if (threadIdx.x < KMAX) {
     double2 c = threadIdx.x < k ? h[threadIdx.x] : make_double2(0, 0);
-    if (scl && threadIdx.x < k) {   // per-vector coefficient factor (see Blas::df_maxpy_norm)
+    if (scl && threadIdx.x < k) {   // per-vector coefficient factor (see DfSlot)
       c.x *= scl[threadIdx.x];
       c.y *= scl[threadIdx.x];
     }
@@ -337,7 +358,32 @@ __global__ void __launch_bounds__(RED_TPB) k_df_maxpy_norm(const float4 *__restr
       df_mac(nrm, im2.h, im2.l, im2.h, im2.l);
     }
   }
-  block_reduce_df<1>(&nrm, smem, partial + blockIdx.x);
+  block_reduce_df<1>(&nrm, smem, t.partial + blockIdx.x);
+}
+
+// the sums of a batch over the CTAs (see k_sum_partials): values 0 .. 2 k - 1 of
+// the chunk from i0 to h, and with norms (value stride - 1) to *norm, its
+// reciprocal to *inv
+__global__ void __launch_bounds__(256) k_df_sums(const DfBatch B, int nblk, int stride, int i0, int nh, int norms) {
+  const DfSlot &t = B.s[blockIdx.y];
+  const int kk = df_chunk(t, i0);
+  const bool norm = (int)blockIdx.x >= nh;
+  double *to = norm ? (norms ? t.norm : nullptr) : (int)blockIdx.x < 2 * kk ? t.h + 2 * i0 + blockIdx.x : nullptr;
+  if (!to) return;
+  __shared__ double red[256];
+  const int i = norm ? stride - 1 : blockIdx.x;
+  double s = 0;
+  for (int b = threadIdx.x; b < nblk; b += 256) s += t.partial[(size_t)b * stride + i];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    *to = red[0];
+    if (norm && norms == 2 && t.inv) *t.inv = 1.0 / red[0];
+  }
 }
 
 // y = a x (DF), a double
@@ -439,9 +485,15 @@ Blas::~Blas() {
   if (hpin) cudaFreeHost(hpin);
 }
 
-int Blas::init(int sms) {
+size_t Blas::partial_bytes(int nblk, int slots) {
+  const size_t values = std::max(2 * 16 + 1, 17 * std::min(slots, DF_BATCH));
+  return sizeof(double) * (size_t)nblk * values;
+}
+
+int Blas::init(int sms, int slots) {
   nblk = sms > 0 ? 4 * sms : 608;
-  partial = (double *)pool_dev_alloc(sizeof(double) * (size_t)nblk * (2 * 16 + 1));
+  nslots = slots;
+  partial = (double *)pool_dev_alloc(partial_bytes(nblk, nslots));
   hpin = (double *)pool_host_alloc(sizeof(double) * 256);
   if (!partial || !hpin) {
     set_error("blas: out of memory for reduction scratch");
@@ -451,7 +503,7 @@ int Blas::init(int sms) {
 }
 
 void Blas::release_to_pool() {
-  pool_dev_free(partial, sizeof(double) * (size_t)nblk * (2 * 16 + 1));
+  pool_dev_free(partial, partial_bytes(nblk, nslots));
   pool_host_free(hpin, sizeof(double) * 256);
   partial = hpin = nullptr;
 }
@@ -471,7 +523,7 @@ int Blas::mdot(const double *V, size_t ldv, int k, const double *w, size_t n, do
     DD_LAUNCHED();
     double *wn = i0 == 0 ? wnorm2_dev : nullptr;
     if (const int n_out = 2 * kk + (wn ? 1 : 0)) {
-      k_sum_partials<<<n_out, 256, 0, st>>>(partial, nblk, stride, 2 * kk, h_dev + 2 * i0, wn, nullptr);
+      k_sum_partials<<<n_out, 256, 0, st>>>(partial, nblk, stride, 2 * kk, h_dev + 2 * i0, wn);
       DD_LAUNCHED();
     }
     if (k == 0) break;
@@ -492,7 +544,7 @@ int Blas::maxpy_norm(const double *V, size_t ldv, int k, const double *h_dev, do
     DD_LAUNCHED();
   }
   if (k == 0) return norm2(w, n, norm2_dev, st);
-  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 0, nullptr, norm2_dev, nullptr);
+  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 0, nullptr, norm2_dev);
   DD_LAUNCHED();
   return DD_OK;
 }
@@ -500,7 +552,7 @@ int Blas::maxpy_norm(const double *V, size_t ldv, int k, const double *h_dev, do
 int Blas::norm2(const double *w, size_t n, double *norm2_dev, cudaStream_t st) {
   k_mdot<4><<<nblk, RED_TPB, 0, st>>>((const double2 *)w, 0, 0, (const double2 *)w, n, partial);
   DD_LAUNCHED();
-  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 9, 0, nullptr, norm2_dev, nullptr);
+  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 9, 0, nullptr, norm2_dev);
   return launched("k_sum_partials");
 }
 
@@ -514,56 +566,67 @@ int Blas::xmy(const double *x, double *y, size_t n, cudaStream_t st) {
   return launched("k_xmy");
 }
 
-int Blas::df_mdot(const float *V, size_t ldv, int k, const float *w, size_t n, double *h_dev, double *wnorm2_dev,
-                  cudaStream_t st, const float *w32, int lvb) {
-  for (int i0 = 0; i0 < k || (k == 0 && i0 == 0); i0 += 8) {
-    int kk = k - i0 < 8 ? k - i0 : 8;
-    if (kk < 0) kk = 0;
-    const float4 *Vi = (const float4 *)V + (size_t)i0 * ldv;
-    if (w32) {
-      if (kk <= 4)
-        k_df_mdot<4, true><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, nullptr, n, partial, w32, lvb);
-      else
-        k_df_mdot<8, true><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, nullptr, n, partial, w32, lvb);
-    } else if (kk <= 4)
-      k_df_mdot<4><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, (const float4 *)w, n, partial);
-    else
-      k_df_mdot<8><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, (const float4 *)w, n, partial);
-    int stride = kk <= 4 ? 9 : 17;
-    DD_LAUNCHED();
-    double *wn = i0 == 0 ? wnorm2_dev : nullptr;
-    if (const int n_out = 2 * kk + (wn ? 1 : 0)) {
-      k_sum_partials<<<n_out, 256, 0, st>>>(partial, nblk, stride, 2 * kk, h_dev + 2 * i0, wn, nullptr);
+// Launches over the slots in groups of DF_BATCH; vectors in chunks of 8.
+int Blas::df_mdot(DfSlot *slots, int ns, cudaStream_t st) {
+  for (int s0 = 0; s0 < ns; s0 += DF_BATCH) {
+    DfBatch B;
+    const int nb = fill(B.s, slots, s0, ns);
+    const bool w32 = B.s[0].w32;
+    int kmax = 0;
+    for (int i = 0; i < nb; i++) kmax = std::max(kmax, B.s[i].k);
+    for (int i0 = 0; i0 < kmax || i0 == 0; i0 += 8) {
+      const bool four = kmax - i0 <= 4;
+      const dim3 grid(nblk, nb);
+      if (w32) {
+        if (four) k_df_mdot<4, true><<<grid, RED_TPB, 0, st>>>(B, i0);
+        else k_df_mdot<8, true><<<grid, RED_TPB, 0, st>>>(B, i0);
+      } else {
+        if (four) k_df_mdot<4, false><<<grid, RED_TPB, 0, st>>>(B, i0);
+        else k_df_mdot<8, false><<<grid, RED_TPB, 0, st>>>(B, i0);
+      }
+      DD_LAUNCHED();
+      const int nh = 2 * std::min(8, kmax - i0);
+      k_df_sums<<<dim3(nh + (i0 == 0), nb), 256, 0, st>>>(B, nblk, four ? 9 : 17, i0, nh, i0 == 0);
       DD_LAUNCHED();
     }
-    if (k == 0) break;
   }
   return DD_OK;
 }
 
-int Blas::df_maxpy_norm(const float *V, size_t ldv, int k, const double *h_dev, float *w, size_t n, double *norm2_dev,
-                        cudaStream_t st, const float *w32, int lvb, const double *scl, double *inv2_dev) {
-  if (k == 0) return df_mdot(V, ldv, 0, w, n, nullptr, norm2_dev, st, w32, lvb);
-  for (int i0 = 0; i0 < k; i0 += 8) {
-    int kk = k - i0 < 8 ? k - i0 : 8;
-    const float4 *Vi = (const float4 *)V + (size_t)i0 * ldv;
-    const double2 *hi = (const double2 *)h_dev + i0;
-    const double *si = scl ? scl + i0 : nullptr;
-    // the first chunk reads the FP32 input (when given) and writes w; later chunks update w
-    const bool from32 = w32 && i0 == 0;
-    if (from32) {
-      if (kk <= 4)
-        k_df_maxpy_norm<4, true><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, hi, (float4 *)w, n, partial, w32, lvb, si);
-      else
-        k_df_maxpy_norm<8, true><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, hi, (float4 *)w, n, partial, w32, lvb, si);
-    } else if (kk <= 4)
-      k_df_maxpy_norm<4><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, hi, (float4 *)w, n, partial, nullptr, 0, si);
-    else
-      k_df_maxpy_norm<8><<<nblk, RED_TPB, 0, st>>>(Vi, ldv, kk, hi, (float4 *)w, n, partial, nullptr, 0, si);
+int Blas::df_maxpy_norm(DfSlot *slots, int ns, cudaStream_t st) {
+  for (int s0 = 0; s0 < ns; s0 += DF_BATCH) {
+    DfBatch B;
+    const int nb = fill(B.s, slots, s0, ns);
+    const bool w32 = B.s[0].w32;
+    int kmax = 0;
+    for (int i = 0; i < nb; i++) kmax = std::max(kmax, B.s[i].k);
+    for (int i0 = 0; i0 < kmax; i0 += 8) {
+      const bool four = kmax - i0 <= 4;
+      const dim3 grid(nblk, nb);
+      // the first chunk reads the FP32 input (when given) and writes w; later chunks update w
+      if (w32 && i0 == 0) {
+        if (four) k_df_maxpy_norm<4, true><<<grid, RED_TPB, 0, st>>>(B, i0);
+        else k_df_maxpy_norm<8, true><<<grid, RED_TPB, 0, st>>>(B, i0);
+      } else {
+        if (four) k_df_maxpy_norm<4, false><<<grid, RED_TPB, 0, st>>>(B, i0);
+        else k_df_maxpy_norm<8, false><<<grid, RED_TPB, 0, st>>>(B, i0);
+      }
+      DD_LAUNCHED();
+    }
+    k_df_sums<<<dim3(1, nb), 256, 0, st>>>(B, nblk, 1, 0, 0, 2);
     DD_LAUNCHED();
   }
-  k_sum_partials<<<1, 256, 0, st>>>(partial, nblk, 1, 0, nullptr, norm2_dev, inv2_dev);
-  return launched("k_sum_partials");
+  return DD_OK;
+}
+
+// slots s0 ... of the batch with their reduction scratch; their number
+int Blas::fill(DfSlot *out, const DfSlot *slots, int s0, int ns) const {
+  int nb = 0;
+  for (; nb < DF_BATCH && s0 + nb < ns; nb++) {
+    out[nb] = slots[s0 + nb];
+    out[nb].partial = partial + (size_t)nb * nblk * 17;
+  }
+  return nb;
 }
 
 __global__ void k_set_double(double *p, double v) { *p = v; }

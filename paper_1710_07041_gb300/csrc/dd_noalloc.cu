@@ -238,13 +238,20 @@ extern "C" int dd_solve_noalloc(dd_op_t opp, const dd_solve_params *p, const dou
         if (rc) return rc;
       }
       const int kk = j + 1;
+      DfSlot slot;
+      slot.V = (const float *)Vb;
+      slot.ldv = vstride;
+      slot.n = n;
+      slot.w = (float *)w;
+      slot.h = hd;
       auto mdot = [&](double *wn2) {
-        return df ? bl.df_mdot((const float *)Vb, vstride, kk, (const float *)w, n, hd, wn2, st)
-                  : bl.mdot(Vb, vstride, kk, w, n, hd, wn2, st);
+        slot.k = kk;
+        slot.norm = wn2;
+        return df ? bl.df_mdot(&slot, 1, st) : bl.mdot(Vb, vstride, kk, w, n, hd, wn2, st);
       };
       auto maxpy = [&]() {
-        return df ? bl.df_maxpy_norm((const float *)Vb, vstride, kk, hd, (float *)w, n, hd + 131, st)
-                  : bl.maxpy_norm(Vb, vstride, kk, hd, w, n, hd + 131, st);
+        slot.norm = hd + 131;
+        return df ? bl.df_maxpy_norm(&slot, 1, st) : bl.maxpy_norm(Vb, vstride, kk, hd, w, n, hd + 131, st);
       };
       if ((rc = mdot(hd + 130)) || (rc = maxpy())) return rc;
       DD_CUDA(cudaMemcpyAsync(hh, hd, sizeof hh, cudaMemcpyDeviceToHost, st));

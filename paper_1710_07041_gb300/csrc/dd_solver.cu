@@ -202,7 +202,7 @@ int BatchSolver::init() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return blas_.init(sms);
+  return blas_.init(sms, n);
 }
 
 int BatchSolver::sync_h() {
@@ -382,32 +382,47 @@ int BatchSolver::end_cycle(Slot &s) {
   return rc;
 }
 
-// Double-float solves: the first Gram-Schmidt pass reads w = D z_j from the
-// FP32 field s->zt (from32) and maxpy writes the result straight into the
-// basis slot j+1 (kk = j+1); the re-orthogonalisation pass works on that
+// One classical Gram-Schmidt pass for the slots of A. Double-float solves:
+// the first pass reads w = D z_j from the FP32 field s->zt and the update
+// writes the result straight into the basis slot j+1 (kk = j+1); the re-orthogonalisation pass works on that
 // slot. The dots h_i = <Vb_i, w> are taken against the stored
 // (unnormalised) vectors; the Hessenberg entry is scl[i] h_i and the update
 // w -= <v_i, w> v_i applies scl[i]^2 h_i to Vb_i (sdev). FP64 solves use s->w.
-int BatchSolver::mdot(Slot *s, int kk, double *h, double *wn2, bool from32) {
-  const Geom &g = s->op->lat->g;
-  const size_t n = (size_t)g.V * 12;
-  const int lvb = g.lbd[0] + g.lbd[1] + g.lbd[2] + g.lbd[3];
-  if (df_)
-    return blas_.df_mdot((const float *)s->Vb, n, kk, (const float *)(s->Vb + 2 * n * kk), n, h, wn2, st_,
-                         from32 ? (const float *)s->zt : nullptr, lvb);
-  return blas_.mdot(s->Vb, n, kk, s->w, n, h, wn2, st_);
-}
-
-// (for a double-float basis also s->sdev[kk] = 1 / |w|^2, the next vector's
-// update coefficient)
-int BatchSolver::maxpy(Slot *s, int kk, const double *h, double *wn2, bool from32) {
-  const Geom &g = s->op->lat->g;
-  const size_t n = (size_t)g.V * 12;
-  const int lvb = g.lbd[0] + g.lbd[1] + g.lbd[2] + g.lbd[3];
-  if (df_)
-    return blas_.df_maxpy_norm((const float *)s->Vb, n, kk, h, (float *)(s->Vb + 2 * n * kk), n, wn2, st_,
-                               from32 ? (const float *)s->zt : nullptr, lvb, s->sdev, s->sdev + kk);
-  return blas_.maxpy_norm(s->Vb, n, kk, h, s->w, n, wn2, st_);
+int BatchSolver::gram_schmidt(const std::vector<Slot *> &A, bool first) {
+  int rc;
+  if (df_) {   // one launch per pass for all slots
+    std::vector<DfSlot> b;
+    for (Slot *s : A) {
+      const Geom &g = s->op->lat->g;
+      double *hd = hdev_ + HSTRIDE * (s - slots_.data());
+      const int kk = s->j + 1;
+      DfSlot t;
+      t.V = (const float *)s->Vb;
+      t.ldv = t.n = (size_t)g.V * 12;
+      t.k = kk;
+      t.w = (float *)(s->Vb + 2 * t.n * kk);
+      t.w32 = first ? (const float *)s->zt : nullptr;
+      t.lvb = g.lbd[0] + g.lbd[1] + g.lbd[2] + g.lbd[3];
+      t.h = hd;
+      t.norm = first ? hd + W0 : nullptr;
+      b.push_back(t);
+    }
+    if ((rc = blas_.df_mdot(b.data(), (int)b.size(), st_))) return rc;
+    for (size_t i = 0; i < A.size(); i++) {
+      b[i].norm = hdev_ + HSTRIDE * (A[i] - slots_.data()) + W1;
+      b[i].scl = A[i]->sdev;
+      b[i].inv = A[i]->sdev + b[i].k;   // the next vector's update coefficient
+    }
+    return blas_.df_maxpy_norm(b.data(), (int)b.size(), st_);
+  }
+  for (Slot *s : A) {
+    const size_t n = (size_t)s->op->lat->g.V * 12;
+    double *hd = hdev_ + HSTRIDE * (s - slots_.data());
+    const int kk = s->j + 1;
+    if ((rc = blas_.mdot(s->Vb, n, kk, s->w, n, hd, first ? hd + W0 : nullptr, st_))) return rc;
+    if ((rc = blas_.maxpy_norm(s->Vb, n, kk, hd, s->w, n, hd + W1, st_))) return rc;
+  }
+  return DD_OK;
 }
 
 // One preconditioned Arnoldi step for every slot in A.
@@ -495,12 +510,7 @@ int BatchSolver::arnoldi_step(std::vector<Slot *> &A) {
       if ((rc = launch_convert_field(s->op->lat->g, zprec_, s->zt, DD_F64, s->w, 1, 1.0, st_))) return rc;
   cudaEventRecord(ev_[2], st_);
   // classical Gram-Schmidt, repeated once for slots whose norm drops below 1e-3 of its value (REORTH2)
-  for (Slot *s : A) {
-    double *hd = hdev_ + HSTRIDE * (s - slots_.data());
-    const int kk = s->j + 1;
-    if ((rc = mdot(s, kk, hd, hd + W0, df_))) return rc;
-    if ((rc = maxpy(s, kk, hd, hd + W1, df_))) return rc;
-  }
+  if ((rc = gram_schmidt(A, true))) return rc;
   if ((rc = sync_h())) return rc;
   std::vector<std::vector<cd>> hcol(A.size());
   std::vector<Slot *> again;
@@ -512,12 +522,7 @@ int BatchSolver::arnoldi_step(std::vector<Slot *> &A) {
     if (hp[W1] < REORTH2 * hp[W0]) again.push_back(s);
   }
   if (!again.empty()) {
-    for (Slot *s : again) {
-      double *hd = hdev_ + HSTRIDE * (s - slots_.data());
-      const int kk = s->j + 1;
-      if ((rc = mdot(s, kk, hd, nullptr))) return rc;
-      if ((rc = maxpy(s, kk, hd, hd + W1))) return rc;
-    }
+    if ((rc = gram_schmidt(again, false))) return rc;
     if ((rc = sync_h())) return rc;
     for (size_t i = 0; i < A.size(); i++) {
       Slot *s = A[i];

@@ -90,8 +90,8 @@ class BatchSolver {
   // the slot's buffers with their sizes for lattice volume V (allocation and
   // release walk the same list)
   std::vector<std::pair<void **, size_t>> slot_buffers(Slot &s, long long V) const;
-  int mdot(Slot *s, int kk, double *h, double *wn2, bool from32 = false);
-  int maxpy(Slot *s, int kk, const double *h, double *wn2, bool from32 = false);
+  // one Gram-Schmidt pass of the slots' new vectors against their bases (first: from D z_j, with |w|^2 before)
+  int gram_schmidt(const std::vector<Slot *> &A, bool first);
 
   const Op *op_;
   dd_solve_params p_;
