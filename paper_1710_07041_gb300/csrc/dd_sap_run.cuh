@@ -94,6 +94,12 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
 template <bool MULTI>
 int sap_fine_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
                cudaStream_t st) {
+  static std::once_flag once;   // 32-site blocks need a little over 48 KB (never raised during a capture)
+  static cudaError_t limit = cudaSuccess;
+  std::call_once(once, [&] {
+    limit = cudaFuncSetAttribute(k_sap_fine<MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  });
+  DD_CUDA(limit);
   const SapGroups G = sap_groups(L, nl, tile);
   const AuxPtrs none{};
   for (int sw = 0; sw < p.sweeps; sw++)
