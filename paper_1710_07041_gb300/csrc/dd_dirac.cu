@@ -6,6 +6,7 @@
 // threads of one site share its link and clover loads in L1. The kernel is
 // HBM-bound: per site it moves 24 (in) + 24 (out) + 72 (links) + 72 (clover)
 // reals once, neighbour spinors being re-read from L1/L2.
+#include "dd_fine.cuh"
 #include "dd_tune.cuh"
 
 namespace dd {
@@ -191,6 +192,55 @@ int dirac_v(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st)
   return launched("k_dirac");
 }
 
+// FP64 on small lattices: twelve threads per site (see dd_fine.cuh), 16 sites
+// per CTA (of one right-hand side; every block holds a multiple of 16). One or
+// two threads a site leave most of the chip's 608 FP64 units idle here and take
+// the length of one thread's chain, ~1130 instructions of 64 clocks: 40.5 us on
+// 4^4 as on 16 x 8^3. A thread of this kernel runs ~115: 8.1 us on 4^4.
+constexpr int FINE_SITES = 16;
+__global__ void __launch_bounds__(12 * FINE_SITES) k_dirac_fine(Geom g, const double2 *__restrict__ links,
+                                                               const double2 *__restrict__ clov, const RhsPtrs rp) {
+  __shared__ double2 X[24 * FINE_SITES];   // [upper: half 0, half 1; lower: half 0, half 1][6][site]
+  const int tiles = g.Vb / FINE_SITES, cta = (int)(blockIdx.x / rp.n), rhs = (int)(blockIdx.x - (unsigned)cta * rp.n);
+  const int b = cta / tiles, s0 = (cta - b * tiles) * FINE_SITES;
+  FineThread T;
+  T.d = threadIdx.x >= 6 * FINE_SITES;
+  const int t = threadIdx.x - T.d * 6 * FINE_SITES;
+  T.k = t / FINE_SITES;
+  T.q = t - T.k * FINE_SITES;
+  T.h = T.k / 3;
+  T.c = T.k - 3 * T.h;
+  T.sh = T.h ? -1.0 : 1.0;
+#pragma unroll
+  for (int j = 0; j < 6; j++) {
+    const int i0 = j < T.k ? j : T.k, j0 = j < T.k ? T.k : j;
+    T.off[j] = j == T.k ? T.k >> 1 : herm_off(i0, j0);
+  }
+  const int s = s0 + T.q;
+  const Site st = decode(g, b, s);
+  const double2 *in = (const double2 *)rp.in[rhs], *own = in + ((size_t)b * 12 + 6 * T.d) * g.Vb + s;
+  const double2 y = fine_row(T, clov + ((size_t)b * 36 + 18 * T.d) * g.Vb + s, g.Vb,
+                             [&](int j) { return own[(size_t)j * g.Vb]; });
+  FineAcc o;
+  fine_global(T, g, st, links, in, false, false, o);
+  const int lk = T.d ? T.k : T.c + 3 * (1 - T.h);   // lower component of o.l
+  X[(6 * T.d + T.k) * FINE_SITES + T.q] = o.u;
+  X[(12 + 6 * T.d + lk) * FINE_SITES + T.q] = o.l;
+  __syncthreads();
+  const double2 *Xd = X + (12 * T.d + T.k) * FINE_SITES + T.q;
+  ((double2 *)rp.out[rhs])[((size_t)b * 12 + 6 * T.d + T.k) * g.Vb + s] = add(y, add(Xd[0], Xd[6 * FINE_SITES]));
+}
+// Twelve threads run 1.22 times the instructions of one, so the gain ends where
+// the chip is full. The line depends on the lattice alone (a right-hand side's
+// result must not depend on its batch). Measured, one thread per site -> this
+// kernel, in us:
+//   sites   1 rhs          4 rhs          12 rhs
+//     256   40.5 ->  8.1   41.2 ->  8.1    42.6 ->  14.2
+//    1024   40.8 ->  8.3   41.6 -> 14.3    42.6 ->  38.7
+//    4096   40.1 -> 14.3   41.3 -> 45.3   115.2 -> 130.8
+// (at 1024 sites the two meet at 15 right-hand sides)
+inline bool fine_lattice(const Geom &g) { return g.V <= 1024; }
+
 // Launch variants (threads per CTA, CTAs per SM the register budget must
 // allow): (128, 5) ~100 registers, (128, 6) ~80, (256, 2) ~128 and (256, 3)
 // ~85; for FP64 (128, 4) ~128, (128, 3) ~168, (256, 2) ~128, (256, 1) 255;
@@ -223,6 +273,13 @@ int dirac_t(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st)
   auto run = [&](int v) {
     return v >= 4 ? shape(v - 4, std::true_type{}) : shape(v, std::false_type{});
   };
+  if constexpr (std::is_same<S, double>::value) {
+    if (fine_lattice(g)) {
+      k_dirac_fine<<<(unsigned)(g.V / FINE_SITES * p.n), 12 * FINE_SITES, 0, st>>>(
+          g, (const double2 *)f.links, (const double2 *)f.clov, p);
+      return launched("k_dirac_fine");
+    }
+  }
   int v = 0;
   const TuneFast fast = tune_fast_key(1, g, f.prec, p.n);
   if (!tune_fast_find(fast, &v)) {

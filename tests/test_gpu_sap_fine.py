@@ -52,3 +52,22 @@ def test_small_block_kernel_several_lattices():
         assert torch.equal(fx, single)
     for s in setups:
         s.close()
+
+
+@pytest.mark.parametrize("dims,block,anti", [((4, 4, 4, 4), (2, 2, 2, 2), True), ((4, 4, 4, 4), (2, 2, 2, 2), False),
+                                             ((4, 12, 4, 4), (2, 2, 2, 2), True), ((8, 8, 4, 4), (4, 2, 2, 2), True)])
+def test_small_lattice_operator(dims, block, anti):
+    """The FP64 Dslash of the smallest lattices (up to 1024 sites): each of
+    three right-hand sides against the oracle (bound: rounding order, as in
+    test_gpu_operator.py), and the same bits alone."""
+    s = Setup(dims, block, eps=0.3, n_stout=1, c_sw=1.7, m0=-0.02, prec=dd.F64, seed=65, antiperiodic=anti)
+    psi = np.stack([synth.gaussian_spinor(s.V, 66 + r) for r in range(3)])
+    out = s.lat.new_field(dd.F64, 3)
+    s.op.apply_D(dd.F64, s.lat.to_field(psi, dd.F64), out, nrhs=3)
+    got = s.lat.from_field(out, dd.F64, 3)
+    for r in range(3):
+        assert relerr(got[r], s.ref.apply(psi[r])) <= 1e-13, r
+        one = s.lat.new_field(dd.F64)
+        s.op.apply_D(dd.F64, s.lat.to_field(psi[r], dd.F64), one)
+        assert np.array_equal(s.lat.from_field(one, dd.F64), got[r])
+    s.close()
