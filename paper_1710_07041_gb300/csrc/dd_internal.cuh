@@ -26,6 +26,7 @@
 #include <cstdio>
 #include <string>
 #include <type_traits>
+#include <utility>
 
 #include "../../include/dd.h"
 
@@ -49,6 +50,31 @@ void count_launches(int n);  // kernels launched through a replayed graph
     cudaError_t e_ = (call);                                   \
     if (e_ != cudaSuccess) return ::dd::cuda_fail(e_, #call);  \
   } while (0)
+
+// ---------------------------------------------------------------- launches
+#ifdef __CUDACC__
+// Programmatic launch: this grid lets the next one of the stream start before
+// it ends; the next one waits for it (complete, its writes visible) in grid_wait.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// kern<<<grid, block, smem, st>>>(args...); `ahead`: as a programmatic launch (it
+// may start before the kernel before it ends, see grid_wait)
+template <typename... P, typename... A>
+inline cudaError_t launch_ahead(bool ahead, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = ahead ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+#endif
 
 // -------------------------------------------------------------- geometry
 struct Geom {

@@ -65,62 +65,71 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 acc) {  // acc
 // fields V: out[(h * N + k)] of this CTA's aggregate, optionally only over the
 // sites of one face (face = 2 mu + side, side 1 = upper; -1 = all sites).
 // Returns through smem; thread t < 2N writes result t to dst[t * dst_stride].
-template <int NMAX, typename SV>
+// The vectors go in groups of RG: a thread's 4 RG partial sums (re and im for
+// both chiralities) are summed over the warp by halving: at distance 16, 8, ..
+// a lane gives away one half of its values and keeps the other, 31 shuffles
+// for 32 sums instead of 5 each, the additions and their order those of a
+// butterfly. 32 partial sums fit beside the site's spinor and two vectors'
+// loads at 3 CTAs per SM. N = 16 on 48 x 24^3 (574 MB): 146 us with all sums
+// at once and five shuffles each, 97 us so (5.9 TB/s).
+constexpr int RG = 8, RN_MAX = 32;
+template <typename SV>
 __device__ void restrict_block(const Geom &g, int b, const void *V, size_t fbytes, int N, const float *in, int face,
                                float2 *dst, int dst_stride) {
-  __shared__ float2 red[MG_TPB / 32][2 * NMAX];
-  const int s = threadIdx.x;
-  float2 acc[2 * NMAX];
+  __shared__ float red[MG_TPB / 32][2][RN_MAX][2];
+  const int s = threadIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  bool take = s < g.Vb;
+  if (take && face >= 0) {
+    int lc[4];
+    local_coords(g, s, lc);
+    const int mu = face >> 1;
+    take = lc[mu] == ((face & 1) ? g.bd[mu] - 1 : 0);
+  }
+  Spinor<float> r;
+  if (take) load_spinor<float, float>(in, g, b, s, r);
+  for (int k0 = 0; k0 < N; k0 += RG) {
+    float acc[4 * RG];   // [chirality][vector][re, im]
 #pragma unroll
-  for (int q = 0; q < 2 * NMAX; q++) acc[q] = make_float2(0.f, 0.f);
-  if (s < g.Vb) {
-    bool take = true;
-    if (face >= 0) {
-      int lc[4];
-      local_coords(g, s, lc);
-      const int mu = face >> 1;
-      take = lc[mu] == ((face & 1) ? g.bd[mu] - 1 : 0);
-    }
+    for (int q = 0; q < 4 * RG; q++) acc[q] = 0.f;
     if (take) {
-      Spinor<float> r;
-      load_spinor<float, float>(in, g, b, s, r);
 #pragma unroll
-      for (int k = 0; k < NMAX; k++) {
-        if (k < N) {
+      for (int k = 0; k < RG; k++) {
+        if (k0 + k < N) {
           Spinor<float> v;
-          load_spinor<SV, float>((const char *)V + k * fbytes, g, b, s, v);
+          load_spinor<SV, float>((const char *)V + (k0 + k) * fbytes, g, b, s, v);
           float2 up = make_float2(0.f, 0.f), dn = make_float2(0.f, 0.f);
 #pragma unroll
           for (int c = 0; c < 6; c++) {
             up = cfma_c(make_float2(v.c[c].re, v.c[c].im), make_float2(r.c[c].re, r.c[c].im), up);
             dn = cfma_c(make_float2(v.c[6 + c].re, v.c[6 + c].im), make_float2(r.c[6 + c].re, r.c[6 + c].im), dn);
           }
-          acc[k] = up;
-          acc[NMAX + k] = dn;
+          acc[2 * k] = up.x;
+          acc[2 * k + 1] = up.y;
+          acc[2 * RG + 2 * k] = dn.x;
+          acc[2 * RG + 2 * k + 1] = dn.y;
         }
       }
     }
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    static_assert(4 * RG == 32, "one sum per lane");
 #pragma unroll
-  for (int q = 0; q < 2 * NMAX; q++) {
-    if ((q % NMAX) >= N) continue;
-    float2 v = acc[q];
+    for (int o = 16; o > 0; o >>= 1) {   // lane l ends with the sum of index l
+      const bool up = lane & o;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+      for (int q = 0; q < o; q++) {
+        const float keep = up ? acc[q + o] : acc[q], give = up ? acc[q] : acc[q + o];
+        acc[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
     }
-    if (lane == 0) red[w][q] = v;
+    const int k = k0 + ((lane >> 1) & (RG - 1));
+    if (k < N) red[w][lane >> 4][k][lane & 1] = acc[0];
   }
   __syncthreads();
   if (threadIdx.x < 2 * N) {
     const int h = threadIdx.x / N, k = threadIdx.x - h * N;
     float2 t = make_float2(0.f, 0.f);
     for (int i = 0; i < nw; i++) {
-      float2 u = red[i][h * NMAX + k];
-      t.x += u.x;
-      t.y += u.y;
+      t.x += red[i][h][k][0];
+      t.y += red[i][h][k][1];
     }
     dst[threadIdx.x * dst_stride] = t;
   }
@@ -128,10 +137,9 @@ __device__ void restrict_block(const Geom &g, int b, const void *V, size_t fbyte
 }
 
 // restriction with the FP16 interpolation fields
-template <int NMAX>
-__global__ void __launch_bounds__(MG_TPB) k_restrict(Geom g, const __half *V, size_t fbytes, int N, const float *in,
+__global__ void __launch_bounds__(MG_TPB, 3) k_restrict(Geom g, const __half *V, size_t fbytes, int N, const float *in,
                                                     float2 *out) {
-  restrict_block<NMAX, __half>(g, blockIdx.x, V, fbytes, N, in, -1, out + (size_t)blockIdx.x * 2 * N, 1);
+  restrict_block<__half>(g, blockIdx.x, V, fbytes, N, in, -1, out + (size_t)blockIdx.x * 2 * N, 1);
 }
 
 // Column (h', j) of D_c for aggregates coupled to colour class c16: w = D u
@@ -139,19 +147,18 @@ __global__ void __launch_bounds__(MG_TPB) k_restrict(Geom g, const __half *V, si
 // colour c16 receives its self block; one whose colour differs in exactly one
 // direction bit mu receives the +mu block through its upper mu-face and the
 // -mu block through its lower one. Dc layout: [a][d][col][row].
-template <int NMAX>
 __global__ void __launch_bounds__(MG_TPB) k_restrict_dc(Geom g, const float *V, size_t fstride, int N,
                                                        const float *w, float2 *Dc, int c16, int col) {
   const int a = blockIdx.x, diff = colour16(g, a) ^ c16;
   const int n2 = 2 * N;
   float2 *base = Dc + (size_t)a * 9 * n2 * n2;
   if (diff == 0) {
-    restrict_block<NMAX, float>(g, a, V, fstride * 4, N, w, -1, base + (size_t)col * n2, 1);
+    restrict_block<float>(g, a, V, fstride * 4, N, w, -1, base + (size_t)col * n2, 1);
   } else if ((diff & (diff - 1)) == 0) {
     const int mu = __ffs(diff) - 1;
-    restrict_block<NMAX, float>(g, a, V, fstride * 4, N, w, 2 * mu + 1,
+    restrict_block<float>(g, a, V, fstride * 4, N, w, 2 * mu + 1,
                                 base + ((size_t)(1 + 2 * mu) * n2 + col) * n2, 1);
-    restrict_block<NMAX, float>(g, a, V, fstride * 4, N, w, 2 * mu, base + ((size_t)(2 + 2 * mu) * n2 + col) * n2, 1);
+    restrict_block<float>(g, a, V, fstride * 4, N, w, 2 * mu, base + ((size_t)(2 + 2 * mu) * n2 + col) * n2, 1);
   }
 }
 
@@ -270,12 +277,20 @@ static inline void coarse_shape(int N, int *R, int *Q) {
 // loads them as one 16-byte chunk per column; the Q column groups' partial
 // sums are added in shared memory in a fixed order. With NPRE > 0 a thread
 // issues all its (at most NPRE) chunk loads before gathering x, so the
-// operator stream overlaps the gather. With vnext != null the CTA also stores
-// its own part of s x there (the next Krylov basis vector).
+// operator stream overlaps the gather. A CTA is one chain (loads, product, sum
+// over the groups), so what counts is how many of them are resident: NPRE = 9,
+// the chunks per thread of N = 16, fits four per SM, 12 three (on 48 x 24^3,
+// 95 MB, an application of kmax = 24 steps then takes 80 us longer). Loads
+// ahead of grid_wait, or that keep their lines in L2, made it longer as well
+// (by 70 and 40 us). With vnext != null the CTA also stores its own part of s x
+// there (the next Krylov basis vector).
+constexpr int coarse_ctas(int npre) { return npre == 9 ? 4 : 1; }
 template <int NPRE>
-__global__ void __launch_bounds__(256) k_coarse_apply(Geom g, const __half2 *__restrict__ Dc, int N, int R, int Q,
-                                                      const float2 *__restrict__ x, float2 *y, const float *scale,
-                                                      float2 *vnext, const int *done) {
+__global__ void __launch_bounds__(256, coarse_ctas(NPRE))
+    k_coarse_apply(Geom g, const __half2 *__restrict__ Dc, int N, int R, int Q, const float2 *x, float2 *y,
+                   const float *scale, float2 *vnext, const int *done) {
+  grid_launch_dependents();
+  grid_wait();
   if (done && *done) return;
   extern __shared__ float2 sm[];   // xs[9 * 2N], then red[Q][rows]
   const int a = blockIdx.x, n2 = 2 * N, np = 4 * R, ncol = 9 * n2;
@@ -420,6 +435,8 @@ __device__ __forceinline__ float cta_sum_partials(const float *partial, int P) {
 // c * 256 * CG_EPT + t + 256 u, u < CG_EPT; all its loads are issued together.
 __global__ void __launch_bounds__(256) k_cg_proj(const float2 *Vc, size_t n, const float2 *w, float2 *partial,
                                                  int chunks, CgState *st) {
+  grid_launch_dependents();
+  grid_wait();
   if (st->done) return;
   __shared__ float2 red[8][CG_ROWS];
   const int k = st->j + 1, i0 = blockIdx.y * CG_ROWS;
@@ -537,6 +554,8 @@ __device__ void cg_givens(float n2, CgState *st, int kmax) {
 // Thread t of CTA c owns float4 (two complex numbers) c * 256 + t.
 __global__ void __launch_bounds__(256) k_cg_update_w(const float2 *Vc, size_t n, float2 *w, float *partial,
                                                      CgState *st, int kmax) {
+  grid_launch_dependents();
+  grid_wait();
   if (st->done) return;
   __shared__ float2 hs[64];
   const int k = st->j + 1;
@@ -640,14 +659,7 @@ __global__ void __launch_bounds__(256) k_cg_update(const float2 *Vc, size_t n, f
   }
 }
 
-// fine FP32 fields: y = a - b
-__global__ void k_sub(const float4 *a, const float4 *b, float4 *y, size_t n4) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
-    const float4 u = a[e], v = b[e];
-    y[e] = make_float4(u.x - v.x, u.y - v.y, u.z - v.z, u.w - v.w);
-  }
-}
-// y = (a + b) * s
+// fine FP32 fields: y = (a + b) * s
 __global__ void k_add_scale(const float4 *a, const float4 *b, float4 *y, float s, size_t n4) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
     const float4 u = a[e], v = b[e];
@@ -699,9 +711,7 @@ static int restrict_launch(const Mg *mg, const float *in, float2 *out, cudaStrea
     return DD_EINVAL;
   }
   const size_t fb = fs * sizeof(__half);
-  if (mg->N <= 8) k_restrict<8><<<g.nblocks, MG_TPB, 0, st>>>(g, mg->Vh, fb, mg->N, in, out);
-  else if (mg->N <= 16) k_restrict<16><<<g.nblocks, MG_TPB, 0, st>>>(g, mg->Vh, fb, mg->N, in, out);
-  else k_restrict<32><<<g.nblocks, MG_TPB, 0, st>>>(g, mg->Vh, fb, mg->N, in, out);
+  k_restrict<<<g.nblocks, MG_TPB, 0, st>>>(g, mg->Vh, fb, mg->N, in, out);
   return launched("k_restrict");
 }
 
@@ -715,25 +725,33 @@ int mg_prolong(const Mg *mg, const float2 *c, float *out, cudaStream_t st) {
 }
 
 static int coarse_apply_launch(const Mg *mg, const float2 *x, float2 *y, const float *scale, float2 *vnext,
-                               const int *done, cudaStream_t st) {
+                               const int *done, bool ahead, cudaStream_t st) {
   const Geom &g = mg->op->lat->g;
   int R, Q;
   coarse_shape(mg->N, &R, &Q);
   const size_t shm = sizeof(float2) * (18 * (size_t)mg->N + (size_t)Q * 4 * R);
   const int per = (18 * mg->N + Q - 1) / Q;   // chunks per thread
   const dim3 grid(g.nblocks), blk(R * Q);
-  if (per <= 4) k_coarse_apply<4><<<grid, blk, shm, st>>>(g, mg->Dc, mg->N, R, Q, x, y, scale, vnext, done);
-  else if (per <= 8) k_coarse_apply<8><<<grid, blk, shm, st>>>(g, mg->Dc, mg->N, R, Q, x, y, scale, vnext, done);
-  else if (per <= 12) k_coarse_apply<12><<<grid, blk, shm, st>>>(g, mg->Dc, mg->N, R, Q, x, y, scale, vnext, done);
-  else k_coarse_apply<0><<<grid, blk, shm, st>>>(g, mg->Dc, mg->N, R, Q, x, y, scale, vnext, done);
+  auto *kern = per <= 4    ? k_coarse_apply<4>
+               : per <= 8  ? k_coarse_apply<8>
+               : per <= 9  ? k_coarse_apply<9>
+               : per <= 12 ? k_coarse_apply<12>
+                           : k_coarse_apply<0>;
+  DD_CUDA(launch_ahead(ahead, kern, grid, blk, shm, st, g, (const __half2 *)mg->Dc, mg->N, R, Q, x, y, scale, vnext,
+                       done));
   return launched("k_coarse_apply");
 }
 
 int mg_coarse_apply(const Mg *mg, const float2 *x, float2 *y, cudaStream_t st) {
-  return coarse_apply_launch(mg, x, y, nullptr, nullptr, nullptr, st);
+  return coarse_apply_launch(mg, x, y, nullptr, nullptr, nullptr, false, st);
 }
 
-// e = GMRES_kmax(D_c, b) from 0 (device-side control, 3 launches per step)
+// e = GMRES_kmax(D_c, b) from 0 (device-side control, 3 launches per step).
+// Programmatic launches: a step's kernels are short (16 + 6 + 5 us on the 2592
+// aggregates of 48 x 24^3), so each one starts while the one before ends and
+// waits for it; every CTA waits before it reads or writes anything, so the end
+// of a kernel means the end of all before it. An application whose coarse solve
+// ends early (half of 72 launches empty): 1.69 -> 1.54 ms.
 int mg_coarse_solve(const Mg *mg, MgWork &W, const float2 *b, float2 *e, cudaStream_t st) {
   const size_t n = W.nc;
   const int kmax = mg->p.coarse_max_iter, grid = cg_grid(n);
@@ -745,10 +763,12 @@ int mg_coarse_solve(const Mg *mg, MgWork &W, const float2 *b, float2 *e, cudaStr
   int rc;
   for (int j = 0; j < kmax; j++) {
     float2 *wj = wbuf[j & 1];
-    if ((rc = coarse_apply_launch(mg, src, wj, &cs->hn, W.Vc + (size_t)j * n, &cs->done, st))) return rc;
-    k_cg_proj<<<dim3(cg_chunks(n), (j + CG_ROWS) / CG_ROWS), 256, 0, st>>>(W.Vc, n, wj, W.partial, cg_chunks(n), cs);
+    if ((rc = coarse_apply_launch(mg, src, wj, &cs->hn, W.Vc + (size_t)j * n, &cs->done, true, st))) return rc;
+    DD_CUDA(launch_ahead(true, k_cg_proj, dim3(cg_chunks(n), (j + CG_ROWS) / CG_ROWS), dim3(256), 0, st,
+                         (const float2 *)W.Vc, n, (const float2 *)wj, W.partial, cg_chunks(n), cs));
     DD_LAUNCHED();
-    k_cg_update_w<<<cg_upd_grid(n), 256, 0, st>>>(W.Vc, n, wj, W.pnorm, cs, kmax);
+    DD_CUDA(launch_ahead(true, k_cg_update_w, dim3(cg_upd_grid(n)), dim3(256), 0, st, (const float2 *)W.Vc, n, wj,
+                         W.pnorm, cs, kmax));
     DD_LAUNCHED();
     src = wj;
   }
@@ -758,10 +778,6 @@ int mg_coarse_solve(const Mg *mg, MgWork &W, const float2 *b, float2 *e, cudaStr
   return launched("k_cg_update");
 }
 
-int mg_sub(const float *a, const float *b, float *y, size_t n_floats, cudaStream_t st) {
-  k_sub<<<1024, 256, 0, st>>>((const float4 *)a, (const float4 *)b, (float4 *)y, n_floats / 4);
-  return launched("k_sub");
-}
 int mg_add_scale(const float *a, const float *b, float *y, float s, size_t n_floats, cudaStream_t st) {
   k_add_scale<<<1024, 256, 0, st>>>((const float4 *)a, (const float4 *)b, (float4 *)y, s, n_floats / 4);
   return launched("k_add_scale");
@@ -776,8 +792,8 @@ static int mg_enqueue(const Mg *mg, MgWork &W, const float *r, float *x, cudaStr
   if ((rc = mg_restrict(mg, r, W.cb, st))) return rc;
   if ((rc = mg_coarse_solve(mg, W, W.cb, W.ce, st))) return rc;
   if ((rc = mg_prolong(mg, W.ce, W.xf, st))) return rc;
-  if ((rc = launch_dirac(g, op->f32, W.xf, W.tf, 1, st))) return rc;
-  if ((rc = mg_sub(r, W.tf, W.rf, nf, st))) return rc;   // r1 = r - D x
+  if ((rc = launch_residual(g, op->f32, contiguous(W.xf, W.rf, 1, 4 * nf), contiguous(r, nullptr, 1, 4 * nf), st)))
+    return rc;   // r1 = r - D x
   dd_sap_params sp = mg->p.smoother;
   sp.x_is_zero = 1;
   SapWork ax;   // the smoother's work fields (corrections, block residuals)
@@ -870,9 +886,7 @@ static int build_coarse(Mg *mg, cudaStream_t st) {
       k_column<<<(unsigned)((g.V + 127) / 128), 128, 0, st>>>(g, mg->V + j * fs, hp, c16, u);
       if ((rc = launched("k_column"))) break;
       if ((rc = launch_dirac(g, op->f32, u, wv, 1, st))) break;
-      if (N <= 8) k_restrict_dc<8><<<g.nblocks, MG_TPB, 0, st>>>(g, mg->V, fs, N, wv, dcf, c16, col);
-      else if (N <= 16) k_restrict_dc<16><<<g.nblocks, MG_TPB, 0, st>>>(g, mg->V, fs, N, wv, dcf, c16, col);
-      else k_restrict_dc<32><<<g.nblocks, MG_TPB, 0, st>>>(g, mg->V, fs, N, wv, dcf, c16, col);
+      k_restrict_dc<<<g.nblocks, MG_TPB, 0, st>>>(g, mg->V, fs, N, wv, dcf, c16, col);
       rc = launched("k_restrict_dc");
     }
   if (rc == DD_OK) {

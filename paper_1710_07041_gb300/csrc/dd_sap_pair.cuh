@@ -920,11 +920,6 @@ __device__ __forceinline__ void flux_out_x(const PairThread &T, const Geom &g, i
   for (int k = 0; k < 3; k++) F[(3 * T.h + k) * R + T.r] = to_pair<P, float>(o[2 * k], o[2 * k + 1]);
 }
 
-// Programmatic launch: this grid lets the next one of the stream start before
-// it ends; the next one waits for it (complete, its writes visible) in grid_wait.
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-
 // One colour phase. Work items (lattice group, block of the colour, tile of
 // right-hand sides), one per CTA. mode: SAP_INCR is implied.
 template <typename S, int SHAPE, bool MULTI>

@@ -72,19 +72,9 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
       // programmatic launch: a phase's CTAs stage their operator tiles while
       // the phase before drains, and wait for it (griddepcontrol.wait) before
       // they read what it wrote
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)G.nitems);
-      cfg.blockDim = dim3(PG::NT);
-      cfg.dynamicSmemBytes = PG::SMEM;
-      cfg.stream = st;
-      cudaLaunchAttribute at = {};
-      at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      at.val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      DD_CUDA(cudaLaunchKernelEx(&cfg, kern, G, sw ? rp : first, (const AuxPtrs &)ax, colour,
-                                 (int)(p.x_is_zero && sw == 0), mode, (int)p.mr_steps, tile, ahead,
-                                 sap_timeout_counter()));
+      DD_CUDA(launch_ahead(true, kern, dim3((unsigned)G.nitems), dim3(PG::NT), PG::SMEM, st, G, sw ? rp : first,
+                           (const AuxPtrs &)ax, colour, (int)(p.x_is_zero && sw == 0), mode, (int)p.mr_steps, tile,
+                           ahead, sap_timeout_counter()));
       DD_LAUNCHED();
     }
   return DD_OK;
