@@ -144,7 +144,11 @@ void *pool_stream_alloc(size_t n, cudaStream_t st) {
     StreamPools &S = stream_pools();
     std::lock_guard<std::mutex> lk(S.mu);
     auto it = S.of.find(d);
-    if (it == S.of.end()) {
+    // not during a capture: a first call there takes the default pool
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (it == S.of.end() && (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
+      cudaGetLastError();
+    } else if (it == S.of.end()) {
       cudaMemPoolProps props = {};
       props.allocType = cudaMemAllocationTypePinned;
       props.location.type = cudaMemLocationTypeDevice;
@@ -158,7 +162,7 @@ void *pool_stream_alloc(size_t n, cudaStream_t st) {
       }
       it = S.of.emplace(d, mp).first;
     }
-    mp = it->second;
+    if (it != S.of.end()) mp = it->second;
   }
   void *p = nullptr;
   const cudaError_t e = mp ? cudaMallocFromPoolAsync(&p, n, mp, st) : cudaMallocAsync(&p, n, st);
