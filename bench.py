@@ -444,9 +444,9 @@ def run_ours(args, rank, world):
     sap_tflops = sap_flops_launch / (sap_launch_ms * 1e-3) / 1e12
     sap_bytes_launch = SAP_REALS_PER_SWEEP * real_b[prec] * V / 2
     mean_info = {k: float(np.mean([i[k] for i in infos])) for k in ("ms_sap", "ms_dirac", "ms_orth", "ms_total")}
-    roofline_sap = {"kernel": "k_sap_phase", "bound": "alu", "achieved": sap_tflops, "peak": alu_peak,
+    roofline_sap = {"kernel": "k_sap_pair", "bound": "alu", "achieved": sap_tflops, "peak": alu_peak,
                     "unit": "TFLOP/s", "frac": sap_tflops / alu_peak,
-                    "traffic": kernel_traffic("k_sap_phase"),
+                    "traffic": kernel_traffic("k_sap_pair"),
                     "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 x {peaks['sm_max_mhz']:.0f} MHz",
                     "algorithmic_bytes_per_launch": sap_bytes_launch,
                     "hbm_frac": sap_bytes_launch / (sap_launch_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],

@@ -6,9 +6,7 @@
 //
 // One CTA per block (x one right-hand side). Per phase the CTA
 //   1. stages the block's links, odd-site clover A_oo and even-site inverse
-//      A_ee^-1 into shared memory with bulk (TMA) copies (overlapping step 2;
-//      in one layout the clover blocks go to tensor memory instead, each
-//      thread's two blocks into its own TMEM lane),
+//      A_ee^-1 into shared memory with bulk (TMA) copies (overlapping step 2),
 //   2. forms its residual: r = b - D x on its sites (neighbour x read from
 //      the other colour's blocks in HBM; skipped when x = 0), or, given work
 //      fields, incrementally: after its own solve a block's residual is zero
@@ -29,7 +27,10 @@
 // (chirality block h of the clover) and evaluates the hops in directions
 // {2h, 2h+1}; the two halves exchange partial hop sums through shared memory.
 // With Vh = block sites / 2 a multiple of 32, h is warp-uniform, so the
-// per-direction code never diverges inside a warp.
+// per-direction code never diverges inside a warp. That is the general kernel;
+// the 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage run the same method with
+// two sites per thread in packed arithmetic (dd_sap_pair.cuh), FP64 blocks of
+// 16 and 32 sites with twelve threads per site (dd_sap_fine.cuh).
 // This file holds the host side (variant dispatch per storage precision, the
 // graph cache, the wait counter); the kernel templates are in
 // dd_sap_kernels.cuh and instantiated per precision in dd_sap_<prec>.cu.

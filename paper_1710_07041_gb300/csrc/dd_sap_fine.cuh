@@ -7,7 +7,9 @@
 // 340 us with one of four sub-partitions of 8 SMs at work. Here a thread (see
 // dd_fine.cuh) runs ~90 per half-step. In a direction of extent 2 a site has
 // one neighbour in the block, forward or backward: both kinds run as one hop,
-// its direction a sign and a choice of link entries.
+// its direction a sign and a choice of link entries. The phase: 43 us, still the
+// FP64 issue rate of one thread's chain (2 x 3 MR half-steps and the first and
+// last ones).
 //
 // The even sites' correction is accumulated over the MR steps (e_e = te_0 -
 // sum_k alpha_k te_k with te = A_ee^-1 D_eo rho), which saves the last

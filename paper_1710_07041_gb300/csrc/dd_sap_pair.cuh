@@ -31,6 +31,14 @@
 // needs (2 x 54 words): 252 of 256 columns. Two CTAs of 128 threads per SM.
 //
 // Links are stored times -1/2 (exact), the hop's coefficient.
+//
+// Bound and figures. A CTA lives 55000 clocks at 4 MR steps: 37000 in the half
+// steps (76% of what the register ports allow a stream of packed multiply-adds
+// with three distinct operands), 6100 receiving flux, 5000 sending it, the rest
+// staging. Per phase, general kernel (clover blocks in tensor memory, one site
+// pair per two threads) -> this one: 64x32^3 FP32 0.514 -> 0.374 ms; FP16 48x24^3
+// with 12 right-hand sides 1.62 -> 1.28 ms; 16x8^3 FP32, where it is the latency
+// of one block, 24.3 -> 19.5 us.
 #pragma once
 #include "dd_sap_kernels.cuh"
 
