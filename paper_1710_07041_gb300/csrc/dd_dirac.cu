@@ -94,7 +94,8 @@ __device__ __forceinline__ void clover_apply_no_l1(const void *clov, size_t n, i
   }
 }
 
-template <int MU, typename S, typename C>
+// PAIRED: links from the smoother's full-link field in the packed order
+template <int MU, typename S, typename C, bool PAIRED = false>
 __device__ __forceinline__ void dirac_dir(const Geom &g, const Site &t, const void *links, const void *in,
                                           Spinor<C> &acc) {
   int nb, ns;
@@ -110,11 +111,13 @@ __device__ __forceinline__ void dirac_dir(const Geom &g, const Site &t, const vo
   };
   neighbour(g, t, MU, +1, &nb, &ns, &sg, &inside);
   C f = load_spinor_unscaled<S, C>(in, g, nb, ns, psi);
-  load_link<S, C>(links, g, t.b, t.s, MU, u);
+  if constexpr (PAIRED) load_full_link<S, true>(links, g, t.b, t.s, MU, u);
+  else load_link<S, C>(links, g, t.b, t.s, MU, u);
   hop<MU, true>(acc, u, psi, coef(f));
   neighbour(g, t, MU, -1, &nb, &ns, &sg, &inside);
   f = load_spinor_unscaled<S, C>(in, g, nb, ns, psi);
-  load_link<S, C>(links, g, nb, ns, MU, u);
+  if constexpr (PAIRED) load_full_link<S, true>(links, g, nb, ns, MU, u);
+  else load_link<S, C>(links, g, nb, ns, MU, u);
   hop<MU, false>(acc, u, psi, coef(f));
 }
 
@@ -147,39 +150,54 @@ __global__ void __launch_bounds__(TPB, MINB) k_dirac(Geom g_in, const void *__re
   store_spinor<SO, C>(p.out[r], g, b, s, acc);
 }
 
-// r = b - D x, r as an FP32 field (the first iterate's residual of the
-// Schwarz smoother; the arithmetic of k_dirac, the result not rounded to the
-// storage of x and b)
-template <typename S, int SHAPE>
+// r = b - D x, r as an FP32 field, on the blocks of one colour or on all
+// (colour < 0): the residual of the Schwarz smoother's phases from a given
+// iterate (the arithmetic of k_dirac, the result not rounded to the storage of
+// x and b). PAIRED: with the smoother's own links, all nine entries as rounded
+// to the storage (a third row rebuilt from the rounded two is another operator:
+// in BF16 the smoothed x then differed by 1.8e-3)
+template <typename S, int SHAPE, bool PAIRED>
 __global__ void __launch_bounds__(128, 5) k_residual(Geom g_in, const void *__restrict__ links,
                                                      const void *__restrict__ clov, const RhsPtrs px,
-                                                     const RhsPtrs pb) {
+                                                     const RhsPtrs pb, int colour) {
   using C = typename Store<S>::comp_t;
   const Geom g = block_shape<SHAPE>(g_in);
   const int nrhs = px.n;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= g.V * nrhs) return;
+  if (t >= (colour < 0 ? g.V : g.V / 2) * nrhs) return;
   const long long site = t / nrhs;
   const int r = (int)(t - site * nrhs);
-  const int b = (int)(site / g.Vb), s = (int)(site - (long long)b * g.Vb);
+  const int bi = (int)(site / g.Vb), s = (int)(site - (long long)bi * g.Vb);
+  const int b = colour < 0 ? bi : sap_block_of(g, colour, bi);
   const Site st = decode(g, b, s);
   Spinor<C> x, acc;
   load_spinor<S, C>(px.in[r], g, b, s, x);
   clover_apply_no_l1<S, C>(clov, g.Vb, b, s, x, acc);
-  dirac_dir<0, S, C>(g, st, links, px.in[r], acc);
-  dirac_dir<1, S, C>(g, st, links, px.in[r], acc);
-  dirac_dir<2, S, C>(g, st, links, px.in[r], acc);
-  dirac_dir<3, S, C>(g, st, links, px.in[r], acc);
+  dirac_dir<0, S, C, PAIRED>(g, st, links, px.in[r], acc);
+  dirac_dir<1, S, C, PAIRED>(g, st, links, px.in[r], acc);
+  dirac_dir<2, S, C, PAIRED>(g, st, links, px.in[r], acc);
+  dirac_dir<3, S, C, PAIRED>(g, st, links, px.in[r], acc);
   load_spinor<S, C>(pb.in[r], g, b, s, x);
 #pragma unroll
   for (int i = 0; i < 12; i++) acc.c[i] = {x.c[i].re - acc.c[i].re, x.c[i].im - acc.c[i].im};
   store_spinor<float, C>(px.out[r], g, b, s, acc);
 }
 template <typename S>
-int residual_t(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, cudaStream_t st) {
-  const unsigned grid = (unsigned)((g.V * x.n + 127) / 128);
-  if (shape_of(g) == 1) k_residual<S, 1><<<grid, 128, 0, st>>>(g, f.links, f.clov, x, b);
-  else k_residual<S, 0><<<grid, 128, 0, st>>>(g, f.links, f.clov, x, b);
+int residual_t(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, int colour, cudaStream_t st) {
+  const unsigned grid = (unsigned)(((colour < 0 ? g.V : g.V / 2) * x.n + 127) / 128);
+  auto launch = [&](auto kern, const void *links) { kern<<<grid, 128, 0, st>>>(g, links, f.clov, x, b, colour); };
+  if (colour >= 0) {
+    if (!paired_links(g, f.prec)) {
+      set_error("residual of one colour: packed links only");
+      return DD_EINVAL;
+    }
+    if (shape_of(g) == 1) launch(k_residual<S, 1, true>, f.links_full);
+    else launch(k_residual<S, 2, true>, f.links_full);
+  } else if (shape_of(g) == 1) {
+    launch(k_residual<S, 1, false>, f.links);
+  } else {
+    launch(k_residual<S, 0, false>, f.links);
+  }
   return launched("k_residual");
 }
 
@@ -319,12 +337,12 @@ int launch_dirac(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_
   return DD_EINVAL;
 }
 
-int launch_residual(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, cudaStream_t st) {
+int launch_residual(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, int colour, cudaStream_t st) {
   switch (f.prec) {
-    case DD_F32: return residual_t<float>(g, f, x, b, st);
-    case DD_F16: return residual_t<__half>(g, f, x, b, st);
-    case DD_BF16: return residual_t<__nv_bfloat16>(g, f, x, b, st);
-    case DD_F16N: return residual_t<hn16>(g, f, x, b, st);
+    case DD_F32: return residual_t<float>(g, f, x, b, colour, st);
+    case DD_F16: return residual_t<__half>(g, f, x, b, colour, st);
+    case DD_BF16: return residual_t<__nv_bfloat16>(g, f, x, b, colour, st);
+    case DD_F16N: return residual_t<hn16>(g, f, x, b, colour, st);
   }
   set_error("residual: precision %d not available", f.prec);
   return DD_EINVAL;

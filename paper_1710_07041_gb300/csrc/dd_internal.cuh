@@ -129,6 +129,12 @@ __host__ __device__ inline void block_coords(const Geom &g, int b, int bc[4]) {
   bc[2] = r % g.nb[2];
   bc[3] = r / g.nb[2];
 }
+// the i-th block of colour `colour`: blocks 2i and 2i+1 differ in colour
+__host__ __device__ inline int sap_block_of(const Geom &g, int colour, int bi) {
+  int bb = 2 * bi, bc[4];
+  block_coords(g, bb, bc);
+  return (((bc[0] + bc[1] + bc[2] + bc[3]) & 1) != colour) ? bb + 1 : bb;
+}
 
 __host__ __device__ inline Site decode(const Geom &g, int b, int s) {
   Site t;
@@ -601,6 +607,20 @@ template <typename C, typename P> __device__ __forceinline__ cpx<C> paired_link_
   const R *e = (const R *)tile + 2 * ((size_t)i * n + (s & ~1)) + (s & 1);
   return {(C)-2 * (C)real_of(e[0]), (C)-2 * (C)real_of(e[2])};
 }
+// full link mu of site (b, s) from OpFields::links_full
+template <typename S, bool PAIRED, typename C>
+__device__ __forceinline__ void load_full_link(const void *links, const Geom &g, int b, int s, int mu, Link<C> &u) {
+  if constexpr (PAIRED) {
+    using P = typename Store<S>::pair_t;
+    DD_CHECK_INDEX(b, g.nblocks);
+    DD_CHECK_INDEX(s, g.Vb);
+#pragma unroll
+    for (int i = 0; i < 9; i++)
+      u.m[i] = paired_link_entry<C, P>((const P *)links + (size_t)b * 36 * g.Vb, g.Vb, 9 * mu + i, s);
+  } else {
+    load_link<S, C, 9, false>(links, g, b, s, mu, u);
+  }
+}
 
 template <typename C> __device__ __forceinline__ cpx<C> cmul(cpx<C> a, cpx<C> b) {
   return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
@@ -896,8 +916,8 @@ struct AuxPtrs {
   void *r[MAX_RHS] = {};
 };
 // What a smoother call is given: the work fields its kernels take, and FP32
-// fields for b - D x of a given first iterate (x_is_zero = 0; packed links
-// only, may be null: then every phase forms b - D x).
+// fields for b - D x in the phases of the first sweep from a given iterate
+// (x_is_zero = 0; packed links only, may be null: then every phase forms b - D x).
 struct SapWork : AuxPtrs {
   void *r0[MAX_RHS] = {};
 };
@@ -919,8 +939,10 @@ int launch_build_clover(const Geom &g, const double *links_canon, double c_sw, d
 int launch_convert_clover(int prec, const double *in, void *out, size_t ntiles, int n, cudaStream_t st);
 int launch_dirac(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st);
 int launch_dirac(const Geom &g, const OpFields &f, const void *in, void *out, int nrhs, cudaStream_t st);
-// r = b - D x with r as FP32 fields: x.in = x, x.out = r, b.in = b (32- and 16-bit storage)
-int launch_residual(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, cudaStream_t st);
+// r = b - D x with r as FP32 fields: x.in = x, x.out = r, b.in = b (32- and 16-bit storage).
+// colour >= 0: on the blocks of that Schwarz colour and with the smoother's links (links_full
+// in the packed order); colour < 0: on all, with those of launch_dirac
+int launch_residual(const Geom &g, const OpFields &f, const RhsPtrs &x, const RhsPtrs &b, int colour, cudaStream_t st);
 // y = D x with double-float fields (f = op->fdf) and double-float inputs p.in
 // (FP64 fields split by launch_split_pairs), FP64 outputs p.out
 int launch_dirac_df(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st);

@@ -792,7 +792,8 @@ static int mg_enqueue(const Mg *mg, MgWork &W, const float *r, float *x, cudaStr
   if ((rc = mg_restrict(mg, r, W.cb, st))) return rc;
   if ((rc = mg_coarse_solve(mg, W, W.cb, W.ce, st))) return rc;
   if ((rc = mg_prolong(mg, W.ce, W.xf, st))) return rc;
-  if ((rc = launch_residual(g, op->f32, contiguous(W.xf, W.rf, 1, 4 * nf), contiguous(r, nullptr, 1, 4 * nf), st)))
+  if ((rc = launch_residual(g, op->f32, contiguous(W.xf, W.rf, 1, 4 * nf), contiguous(r, nullptr, 1, 4 * nf), -1,
+                            st)))
     return rc;   // r1 = r - D x
   dd_sap_params sp = mg->p.smoother;
   sp.x_is_zero = 1;

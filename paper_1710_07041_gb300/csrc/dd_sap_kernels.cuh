@@ -204,21 +204,6 @@ __device__ __forceinline__ void hops_inner(int Vh, int s, int h, uint2 nbr, int 
   }
 }
 
-// full link mu of site (b, s) from the global field
-template <typename S, bool PAIRED, typename C>
-__device__ __forceinline__ void load_full_link(const void *links, const Geom &g, int b, int s, int mu, Link<C> &u) {
-  if constexpr (PAIRED) {
-    using P = typename Store<S>::pair_t;
-    DD_CHECK_INDEX(b, g.nblocks);
-    DD_CHECK_INDEX(s, g.Vb);
-#pragma unroll
-    for (int i = 0; i < 9; i++)
-      u.m[i] = paired_link_entry<C, P>((const P *)links + (size_t)b * 36 * g.Vb, g.Vb, 9 * mu + i, s);
-  } else {
-    load_link<S, C, 9, false>(links, g, b, s, mu, u);
-  }
-}
-
 // acc += hops into site t from the global field x, directions {2h, 2h+1};
 // neighbours inside the block are skipped when self_zero (x known to be 0
 // there), neighbours outside when halo_zero. SW: acc's spin halves swapped.
@@ -599,13 +584,6 @@ __device__ __forceinline__ int sap_group_of(const SapGroups &G, int item) {
   while (k + 1 < G.n && item >= G.grp[k + 1].item0) k++;
   return k;
 }
-// the i-th block of colour `colour`: blocks 2i and 2i+1 differ in colour
-__device__ __forceinline__ int sap_block_of(const Geom &g, int colour, int bi) {
-  int bb = 2 * bi, bc[4];
-  block_coords(g, bb, bc);
-  return (((bc[0] + bc[1] + bc[2] + bc[3]) & 1) != colour) ? bb + 1 : bb;
-}
-
 // STAGE: 0 operator tiles read through L1/L2; 1 links, A_oo and A_ee^-1 staged
 // in shared memory; 2 links staged, the clover blocks (each read by one
 // thread only) through L1/L2, which halves the footprint.

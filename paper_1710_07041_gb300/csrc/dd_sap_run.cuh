@@ -25,9 +25,11 @@ int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
 }
 
 // One smoother application in the packed kernel (dd_sap_pair.cuh). From a
-// given x the first sweep works on the residual b - D x, formed once as an
-// FP32 field by the operator's kernel; after that, as from x = 0, every phase
-// takes its residual from the stored one and the neighbours' flux.
+// given x each phase of the first sweep works on the residual b - D x of x as
+// stored, formed on its colour's blocks as an FP32 field by the operator's
+// kernel (so the rounding of x in the first colour's update is seen by the
+// second); after that, as from x = 0, every phase takes its residual from the
+// stored one and the neighbours' flux.
 template <typename S, int SHAPE, bool MULTI>
 int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork &ax, int tile,
                cudaStream_t st) {
@@ -49,8 +51,7 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int ahead = sms * (SHAPE == 1 ? 2 : 1) / 4;
-  RhsPtrs first = rp;   // the first sweep's right-hand sides
-  if (!p.x_is_zero) {
+  auto residual = [&](int colour) -> int {   // ax.r0 = b - D x on the blocks of a colour
     RhsPtrs x, b;
     for (int k = 0, r = 0; k < nl; k++) {
       x.n = b.n = L[k].nrhs;
@@ -59,21 +60,27 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
         x.out[i] = ax.r0[r];
         b.in[i] = rp.in[r];
         b.out[i] = nullptr;
-        first.in[r] = ax.r0[r];
       }
-      if (int rc = launch_residual(L[k].g, L[k].f, x, b, st)) return rc;
+      if (int rc = launch_residual(L[k].g, L[k].f, x, b, colour, st)) return rc;
     }
-  }
+    return DD_OK;
+  };
+  RhsPtrs from_r0 = rp;
+  for (int r = 0; r < rp.n; r++) from_r0.in[r] = ax.r0[r];
   for (int sw = 0; sw < p.sweeps; sw++)
     for (int colour = 0; colour < 2; colour++) {
-      int mode = sw ? SAP_HALO_E : SAP_FROM_B | (colour ? SAP_HALO_E : 0) | (p.x_is_zero ? 0 : SAP_B32);
-      if (!(sw == p.sweeps - 1 && colour == 1)) mode |= SAP_WRITE_E;   // read by the next phase
+      const bool given = sw == 0 && !p.x_is_zero;
+      int mode = sw ? SAP_HALO_E : given ? SAP_FROM_B | SAP_B32 : SAP_FROM_B | (colour ? SAP_HALO_E : 0);
+      if (given)
+        if (int rc = residual(colour)) return rc;
+      // read by the next phase, unless that is the last's or forms b - D x
+      if (!(sw == p.sweeps - 1 && colour == 1) && !(given && colour == 0)) mode |= SAP_WRITE_E;
       if (sw + 1 < p.sweeps) mode |= SAP_WRITE_R;                      // by this colour's next one
       // programmatic launch: a phase's CTAs stage their operator tiles while
       // the phase before drains, and wait for it (griddepcontrol.wait) before
       // they read what it wrote (64x32^3: 0.388 -> 0.374 ms per phase; 16x8^3:
       // 23.1 -> 20.3 us)
-      DD_CUDA(launch_ahead(true, kern, dim3((unsigned)G.nitems), dim3(PG::NT), PG::SMEM, st, G, sw ? rp : first,
+      DD_CUDA(launch_ahead(true, kern, dim3((unsigned)G.nitems), dim3(PG::NT), PG::SMEM, st, G, given ? from_r0 : rp,
                            (const AuxPtrs &)ax, colour, (int)(p.x_is_zero && sw == 0), mode, (int)p.mr_steps, tile,
                            ahead, sap_timeout_counter()));
       DD_LAUNCHED();
@@ -219,7 +226,7 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
     int c = tune_lookup(key);
     k = c >= 0 && c < nvar ? c : 0;
   }
-  return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps + (p.x_is_zero || !pair ? 0 : nl), rp, ax,
+  return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps + (p.x_is_zero || !pair ? 0 : 2 * nl), rp, ax,
                              [&] { return run(k); }, st);
 }
 
