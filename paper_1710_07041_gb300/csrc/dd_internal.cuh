@@ -915,9 +915,11 @@ struct AuxPtrs {
   void *e[MAX_RHS] = {};
   void *r[MAX_RHS] = {};
 };
-// What a smoother call is given: the work fields its kernels take, and FP32
-// fields for b - D x in the phases of the first sweep from a given iterate
-// (x_is_zero = 0; packed links only, may be null: then every phase forms b - D x).
+// What a smoother call is given: the work fields its kernels take (e and r both
+// or neither), and FP32 fields for b - D x, one per right-hand side (packed
+// links only). From a given iterate (x_is_zero = 0) the phases of the first
+// sweep use r0; without it, or without e and r, every phase forms b - D x: in
+// the packed kernel when r0 is given, else in the general one.
 struct SapWork : AuxPtrs {
   void *r0[MAX_RHS] = {};
 };

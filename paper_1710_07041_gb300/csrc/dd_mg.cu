@@ -684,11 +684,12 @@ int MgWork::init(const Mg *mg) {
   const size_t f32 = (size_t)g.V * 24 * 4, fp = (size_t)g.V * spinor_site_bytes(mg->op->prec), cv = sizeof(float2) * nc;
   const int kmax = mg->p.coarse_max_iter;
   bufs = {{(void **)&Vc, cv * (kmax + 1)}, {(void **)&w, cv}, {(void **)&w2, cv}, {(void **)&cb, cv}, {(void **)&ce, cv},
-          {(void **)&xf, f32}, {(void **)&rf, f32}, {(void **)&tf, f32}, {&tin, fp}, {&tout, fp}, {&se, fp}, {&sr, fp},
+          {(void **)&xf, f32}, {(void **)&rf, f32}, {(void **)&tf, f32}, {&tin, fp}, {&tout, fp},
           {(void **)&partial, sizeof(float2) * cg_chunks(nc) * 65}, {(void **)&pnorm, sizeof(float) * cg_partials(nc)},
-          {&st, sizeof(CgState)}};
+          {&st, sizeof(CgState)}, {&sfine, mg->op->prec == DD_F64 ? 2 * fp : 0}};
   for (auto &b : bufs)
-    if (!(*b.first = pool_dev_alloc(b.second))) {
+    // (without sfine the smoother forms b - D x in every phase)
+    if (!(*b.first = pool_dev_alloc(b.second)) && b.first != &sfine) {
       set_error("mg: out of device memory for the coarse-solve workspace");
       return DD_ENOMEM;
     }
@@ -697,7 +698,7 @@ int MgWork::init(const Mg *mg) {
 
 size_t MgWork::bytes(const Geom &g, int prec, int N, int kmax) {
   const size_t nc = (size_t)g.nblocks * 2 * N;
-  return sizeof(float2) * nc * (kmax + 5) + (size_t)g.V * 24 * (4 * 3 + 4 * real_bytes(prec)) +
+  return sizeof(float2) * nc * (kmax + 5) + (size_t)g.V * 24 * (4 * 3 + 2 * real_bytes(prec)) +
          sizeof(float2) * cg_chunks(nc) * 65 + sizeof(float) * cg_partials(nc) + sizeof(CgState);
 }
 
@@ -797,10 +798,21 @@ static int mg_enqueue(const Mg *mg, MgWork &W, const float *r, float *x, cudaStr
     return rc;   // r1 = r - D x
   dd_sap_params sp = mg->p.smoother;
   sp.x_is_zero = 1;
-  SapWork ax;   // the smoother's work fields (corrections, block residuals)
-  ax.e[0] = W.se;
-  ax.r[0] = W.sr;
+  // The smoother's work fields (corrections, block residuals). FP32: tin and
+  // tout, which only other storages fill. 16 bits: none, so that what passes
+  // between its phases is x alone; every phase forms b - D x in FP32, for
+  // which rf is free once it is converted.
+  SapWork ax;
   const size_t fb = (size_t)g.V * spinor_site_bytes(op->prec);
+  if (op->prec == DD_F32) {
+    ax.e[0] = W.tin;
+    ax.r[0] = W.tout;
+  } else if (op->prec == DD_F64) {
+    ax.e[0] = W.sfine;
+    ax.r[0] = W.sfine ? (char *)W.sfine + fb : nullptr;
+  } else {
+    ax.r0[0] = W.rf;
+  }
   auto smooth = [&](const void *b, void *x) { return launch_sap(g, op->fp, sp, contiguous(b, x, 1, fb), st, &ax); };
   if (op->prec == DD_F32) {
     if ((rc = smooth(W.rf, W.tf))) return rc;
@@ -920,9 +932,18 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
   }
   if (cudaMalloc(&nrm, sizeof(double)) != cudaSuccess) rc = DD_ENOMEM;
   if (cudaMalloc(&pin, fs * real_bytes(op->prec)) != cudaSuccess ||
-      cudaMalloc(&pout, fs * real_bytes(op->prec)) != cudaSuccess ||
-      cudaMalloc(&aux, sap_work_bytes(g, op->prec, 1)) != cudaSuccess)
+      cudaMalloc(&pout, fs * real_bytes(op->prec)) != cudaSuccess)
     rc = DD_ENOMEM;
+  // the smoother's work fields as in mg_enqueue; without room for them every phase forms b - D x
+  const bool wide = op->prec == DD_F32 || op->prec == DD_F64;
+  const size_t ab = wide ? sap_work_bytes(g, op->prec, 1) : fs * 4;
+  SapWork ax;
+  if (rc == DD_OK && cudaMalloc(&aux, ab) != cudaSuccess) {
+    cudaGetLastError();
+    aux = nullptr;
+  }
+  (wide ? ax.e[0] : ax.r0[0]) = aux;
+  if (wide && aux) ax.r[0] = (char *)aux + ab / 2;
   const double sigma = std::sqrt(24.0 * (double)g.V);
   for (int k = 0; k < N && rc == DD_OK; k++) {
     float *vk = mg->V + k * fs;
@@ -933,7 +954,7 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
     for (int it = 0; it < mg->p.setup_iters && rc == DD_OK; it++) {
       dd_sap_params sp = mg->p.smoother;
       sp.x_is_zero = 1;
-      if ((rc = launch_sap(g, op->fp, sp, pin, pout, 1, st, aux))) break;
+      if ((rc = launch_sap(g, op->fp, sp, contiguous(pin, pout, 1, fs * real_bytes(op->prec)), st, &ax))) break;
       if ((rc = launch_unpack(g, op->prec, pout, canon, 1, 1.0, st))) break;
       if ((rc = bl.norm2(canon, fs / 2, nrm, st))) break;
       double n2 = 0;

@@ -19,7 +19,7 @@ struct MgWork {
   float2 *w = nullptr, *w2 = nullptr, *cb = nullptr, *ce = nullptr;
   float *xf = nullptr, *rf = nullptr, *tf = nullptr;   // fine FP32 fields
   void *tin = nullptr, *tout = nullptr;                // smoother-precision fields
-  void *se = nullptr, *sr = nullptr;                   // its work fields (corrections, block residuals)
+  void *sfine = nullptr;       // FP64 smoother: its work fields (two)
   float2 *partial = nullptr;   // coarse reduction partials
   float *pnorm = nullptr;
   void *st = nullptr;          // coarse GMRES control state (device)

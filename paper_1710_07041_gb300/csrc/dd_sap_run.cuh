@@ -29,7 +29,10 @@ int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
 // stored, formed on its colour's blocks as an FP32 field by the operator's
 // kernel (so the rounding of x in the first colour's update is seen by the
 // second); after that, as from x = 0, every phase takes its residual from the
-// stored one and the neighbours' flux.
+// stored one and the neighbours' flux. With r0 alone (no e and r) every phase
+// but the first from x = 0 does so: the two-level preconditioner's 16-bit
+// smoother, whose residual and corrections are not to pass between phases in 16
+// bits (dd_mg.cu).
 template <typename S, int SHAPE, bool MULTI>
 int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork &ax, int tile,
                cudaStream_t st) {
@@ -67,15 +70,20 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
   };
   RhsPtrs from_r0 = rp;
   for (int r = 0; r < rp.n; r++) from_r0.in[r] = ax.r0[r];
+  const bool incr = ax.e[0] != nullptr;
+  if (!incr && p.x_is_zero)   // the second phase's residual reads x on every block
+    for (int k = 0, r = 0; k < nl; k++)
+      for (int i = 0; i < L[k].nrhs; i++, r++)
+        DD_CUDA(cudaMemsetAsync(rp.out[r], 0, (size_t)L[k].g.V * spinor_site_bytes(Store<S>::prec), st));
   for (int sw = 0; sw < p.sweeps; sw++)
     for (int colour = 0; colour < 2; colour++) {
-      const bool given = sw == 0 && !p.x_is_zero;
-      int mode = sw ? SAP_HALO_E : given ? SAP_FROM_B | SAP_B32 : SAP_FROM_B | (colour ? SAP_HALO_E : 0);
+      const bool given = incr ? sw == 0 && !p.x_is_zero : sw || colour || !p.x_is_zero;   // works on b - D x
+      int mode = given ? SAP_FROM_B | SAP_B32 : sw ? SAP_HALO_E : SAP_FROM_B | (colour ? SAP_HALO_E : 0);
       if (given)
         if (int rc = residual(colour)) return rc;
-      // read by the next phase, unless that is the last's or forms b - D x
-      if (!(sw == p.sweeps - 1 && colour == 1) && !(given && colour == 0)) mode |= SAP_WRITE_E;
-      if (sw + 1 < p.sweeps) mode |= SAP_WRITE_R;                      // by this colour's next one
+      // e is read by the next phase, unless this is the last or that forms b - D x
+      if (incr && !(sw == p.sweeps - 1 && colour == 1) && !(given && colour == 0)) mode |= SAP_WRITE_E;
+      if (incr && sw + 1 < p.sweeps) mode |= SAP_WRITE_R;   // r by this colour's next one
       // programmatic launch: a phase's CTAs stage their operator tiles while
       // the phase before drains, and wait for it (griddepcontrol.wait) before
       // they read what it wrote (64x32^3: 0.388 -> 0.374 ms per phase; 16x8^3:
@@ -128,7 +136,8 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
                  cudaStream_t st) {
   const Geom &g = L[0].g;
   const bool paired = paired_links(g, L[0].f.prec);
-  if (paired && ax && !p.x_is_zero && !ax->r0[0]) ax = nullptr;
+  const bool incr = ax && ax->e[0], r0 = ax && ax->r0[0];
+  if (paired ? !r0 && !(incr && p.x_is_zero) : !incr) ax = nullptr;
   const bool pair = paired && ax, fine = Store<S>::prec == DD_F64 && fine_block(g);
   const size_t limit = 227 * 1024, half = 113 * 1024;
   const bool stage1 = SapSmem<S>::bytes(g, 1) <= limit;
@@ -216,7 +225,7 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
   for (int k = 0; k < nl; k++)
     fields += std::to_string((uintptr_t)L[k].f.links_full) + "," + std::to_string((uintptr_t)L[k].f.clov) + "," +
               std::to_string((uintptr_t)L[k].f.cinv) + "," + std::to_string((uintptr_t)L[k].f.links) + ";";
-  if (!p.x_is_zero && pair)
+  if (pair && r0)
     for (int r = 0; r < rp.n; r++) fields += std::to_string((uintptr_t)ax->r0[r]) + ",";
   // x is pure output when x_is_zero, so trial runs leave the same result
   if (p.x_is_zero) {
@@ -226,8 +235,10 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
     int c = tune_lookup(key);
     k = c >= 0 && c < nvar ? c : 0;
   }
-  return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps + (p.x_is_zero || !pair ? 0 : 2 * nl), rp, ax,
-                             [&] { return run(k); }, st);
+  // launches of an application: the phases and, in the packed kernel, the residuals formed ahead of them
+  const int nres = !pair ? 0 : !incr ? 2 * p.sweeps - (p.x_is_zero ? 1 : 0) : p.x_is_zero ? 0 : 2;
+  return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps + nres * nl, rp, ax, [&] { return run(k); },
+                             st);
 }
 
 }  // namespace

@@ -1,6 +1,6 @@
 """The residual b - D x of a Schwarz phase sees x as it is stored, in FP32, and
 the links of the block solves (16-bit storage): in the first sweep from a given
-x.
+x, and in every phase of the two-level preconditioner's smoother.
 
 The FP64 oracle works on the very fields of the kernels: c_sw = 0 and m0 = 0 (A
 = 4, A^-1 = 1/4), and links that 16 bits hold exactly (colour permutations
@@ -31,9 +31,9 @@ def exact_links(V, seed):
     return U.reshape(V, 4, 3, 3)
 
 
-def rounded_links(U, prec):
-    """All nine entries rounded to the storage, to nearest even."""
-    v = parts(U)
+def rounded(z, prec):
+    """Every component rounded to the storage, to nearest even."""
+    v = parts(z)
     if prec == dd.BF16:
         m, e = np.frexp(v)
         v = np.ldexp(np.rint(np.ldexp(m, 8)), e - 8)
@@ -78,7 +78,7 @@ def test_second_colour_sees_the_stored_iterate(prec, dims, block, links):
     lat = dd.Lattice(dims, block)
     gauge = dd.Gauge(lat, U)
     op = dd.Op(gauge, 0.0, 0.0, prec)
-    ref = oracle.Operator(dims, U if links == "exact" else rounded_links(U, prec), 0.0, 0.0)
+    ref = oracle.Operator(dims, U if links == "exact" else rounded(U, prec), 0.0, 0.0)
     fb, fx = lat.to_field(synth.gaussian_spinor(V, 6), prec), lat.to_field(synth.gaussian_spinor(V, 7), prec)
     b, x = lat.from_field(fb, prec), lat.from_field(fx, prec)
     op.sap_smooth(fb, fx, 1, 4, x_is_zero=False)
@@ -92,6 +92,44 @@ def test_second_colour_sees_the_stored_iterate(prec, dims, block, links):
         step = ULP[prec] * 2.0 ** np.floor(np.log2(np.abs(want)))
     off = np.abs(parts(got[second]) - want) - 0.5 * step - 2.0 ** -17 * np.abs(want).max()
     assert off.max() <= 0, (int((off > 0).sum()), off.size)
+    op.close()
+    gauge.close()
+    lat.close()
+
+
+@pytest.mark.parametrize("prec", [dd.F16, dd.BF16])
+@pytest.mark.parametrize("dims,block", [((8, 8, 8, 8), (4, 4, 4, 4)), ((8, 4, 8, 8), (4, 2, 4, 4))])
+def test_two_level_smoother_works_on_the_stored_iterate(prec, dims, block):
+    """Test vectors on two colours and a residual on the third: the coarse part
+    vanishes, so the preconditioner's result is the smoother's x, whose phases
+    are followed one by one, x rounded to the storage after each. FP32 noise
+    of 8 roundoffs (2^-21) crosses a rounding boundary in one of ULP / 2^-19
+    components, an error of sqrt(2^-19 / ULP) ULP <= ULP / 22 in the 2-norm;
+    bound ULP / 16. (Residuals or corrections handed on in 16 bits: each a
+    rounding of 0.2 to 0.3 ULP.)"""
+    V = int(np.prod(dims))
+    U = exact_links(V, 8)
+    lat = dd.Lattice(dims, block)
+    gauge = dd.Gauge(lat, U)
+    op = dd.Op(gauge, 0.0, 0.0, prec)
+    ref = oracle.Operator(dims, U, 0.0, 0.0)
+    tv = np.stack([synth.gaussian_spinor(V, 20 + k) for k in range(4)])
+    tv[..., 2] = 0
+    mg = dd.Multigrid(op, tv, setup_iters=0, sweeps=2, mr_steps=4)
+    r = synth.gaussian_spinor(V, 9)
+    r[..., :2] = 0
+    r = lat.from_field(lat.to_field(r, prec), prec)
+    rf, xf = lat.to_field(r, dd.F32), lat.new_field(dd.F32)
+    mg.precondition(rf, xf)
+    got = lat.from_field(xf, dd.F32)
+    x = np.zeros_like(r)
+    for _ in range(2):
+        for colour in range(2):
+            x = rounded(x + phase(ref, block, colour, r, x, 4), prec)
+    err = np.linalg.norm(got - x) / np.linalg.norm(x)
+    print(f"two-level smoother error {err / ULP[prec]:.4f} ULP")
+    assert err <= ULP[prec] / 16
+    mg.close()
     op.close()
     gauge.close()
     lat.close()
