@@ -360,6 +360,8 @@ __device__ __forceinline__ int slot(int s, int r) { return r ^ (((s ^ (s >> 1)) 
 // first colour of spin s at row r
 __device__ __forceinline__ int spin_at(int rows, int s, int r) { return 3 * s * rows + slot(s, r); }
 
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 // What a thread knows about its row: neighbours in the block, signs
 struct PairThread {
   int h, r, y, z, t, q;
@@ -970,6 +972,8 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
   constexpr unsigned SB = (unsigned)spinor_site_bytes(Store<S>::prec);
   constexpr unsigned RQ = QuadStore<S, true>::bytes, RB = 6 * NT * RQ;   // stored residual of a block
   constexpr unsigned FB = Flux<SHAPE>::total * sizeof(P);
+  constexpr bool APART = Store<S>::prec == DD_F32;   // how e is summed, see the MR loop
+  static_assert(!APART || 12u * NT * 8 <= FB, "step 0's te fits the block's flux");
 
   // this thread's clover blocks: chirality h of the even and the odd pair, both
   // sites' chunks (neighbours in memory) in one 32-byte load
@@ -1169,7 +1173,13 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
       //     D_oe te, alpha = <p, rho> / <p, p>, e_o += alpha rho, rho -= alpha p
       //   reconstruction: e_e = A_ee^-1 (r_e - D_eo e_o) with e_o = sum_k alpha_k
       //     rho_k is step 0's te minus sum_k alpha_k (step k's te): the steps
-      //     accumulate it, and no half-step is spent on D_eo e_o
+      //     accumulate it, and no half-step is spent on D_eo e_o. In FP32
+      //     storage this must not be less exact than that half-step was: there
+      //     the products are rounded apart from the sums, and the sum over k
+      //     is kept apart from step 0's te, which waits where the block's
+      //     incoming flux was (errors against 64 bits, 16x8^3, 1 to 4 sweeps of
+      //     2 to 5 steps: 1.24..1.44e-7 with the half-step, 1.27..1.55e-7
+      //     accumulated on te, 1.23..1.42e-7 so; 64x32^3: 2.97 -> 3.05 ms).
       u64 rh[12], eo[12], ee[12];
       uint32_t cl[72], xl[54];
       {
@@ -1180,6 +1190,13 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
         for (int i = 0; i < 36; i++) m[i] = word2(cl, i);
         herm6_pair(m, r_e, ee);
         st6(T, V, R, ee);
+      }
+      char *const te0 = (char *)ax.e[r] + (size_t)b * FB;   // FP32: step 0's te
+      if constexpr (APART) {
+#pragma unroll
+        for (int i = 0; i < 6; i++) quad_st<S, true>(te0, i * NT + threadIdx.x, ee[2 * i], ee[2 * i + 1]);
+#pragma unroll
+        for (int i = 0; i < 12; i++) ee[i] = 0ull;
       }
 #pragma unroll
       for (int i = 0; i < 12; i++) {
@@ -1220,6 +1237,9 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
               e = fma2(w[2 * i + 1], w[2 * i + 1], e);
             }
             float pr = lo(a) + hi(a), pi = lo(c) + hi(c), pp = lo(e) + hi(e);
+            if (APART && step == last)
+#pragma unroll
+              for (int i = 0; i < 6; i++) prefetch_l1(te0 + (size_t)(i * NT + threadIdx.x) * 16);
             cta_sum3<NT / 32>(pr, pi, pp, red);
             float ar = 0.f, ai = 0.f;
             if (pp > 0.f) {
@@ -1231,10 +1251,17 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
             ld6(T, V, R, te);
 #pragma unroll
             for (int i = 0; i < 6; i++) {
-              eo[2 * i] = fma2(Ar, rh[2 * i], fma2(neg2(Ai), rh[2 * i + 1], eo[2 * i]));
-              eo[2 * i + 1] = fma2(Ar, rh[2 * i + 1], fma2(Ai, rh[2 * i], eo[2 * i + 1]));
-              ee[2 * i] = fma2(neg2(Ar), te[2 * i], fma2(Ai, te[2 * i + 1], ee[2 * i]));
-              ee[2 * i + 1] = fma2(neg2(Ar), te[2 * i + 1], fma2(neg2(Ai), te[2 * i], ee[2 * i + 1]));
+              if constexpr (APART) {
+                eo[2 * i] = add2(eo[2 * i], fma2(Ar, rh[2 * i], mul2(neg2(Ai), rh[2 * i + 1])));
+                eo[2 * i + 1] = add2(eo[2 * i + 1], fma2(Ar, rh[2 * i + 1], mul2(Ai, rh[2 * i])));
+                ee[2 * i] = sub2(ee[2 * i], fma2(Ar, te[2 * i], mul2(neg2(Ai), te[2 * i + 1])));
+                ee[2 * i + 1] = sub2(ee[2 * i + 1], fma2(Ar, te[2 * i + 1], mul2(Ai, te[2 * i])));
+              } else {
+                eo[2 * i] = fma2(Ar, rh[2 * i], fma2(neg2(Ai), rh[2 * i + 1], eo[2 * i]));
+                eo[2 * i + 1] = fma2(Ar, rh[2 * i + 1], fma2(Ai, rh[2 * i], eo[2 * i + 1]));
+                ee[2 * i] = fma2(neg2(Ar), te[2 * i], fma2(Ai, te[2 * i + 1], ee[2 * i]));
+                ee[2 * i + 1] = fma2(neg2(Ar), te[2 * i + 1], fma2(neg2(Ai), te[2 * i], ee[2 * i + 1]));
+              }
               rh[2 * i] = fma2(neg2(Ar), w[2 * i], fma2(Ai, w[2 * i + 1], rh[2 * i]));
               rh[2 * i + 1] = fma2(neg2(Ar), w[2 * i + 1], fma2(neg2(Ai), w[2 * i], rh[2 * i + 1]));
             }
@@ -1250,6 +1277,14 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
       // is read ahead of the flux, whose arithmetic covers the wait)
       // (every thread is past its last hops at the sum's barrier; without MR steps there was none)
       if (nmr == 0) __syncthreads();
+      if constexpr (APART) {
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+          const quad v = quad_of<S, true>(quad_raw<S, true>(te0, i * NT + threadIdx.x));
+          ee[2 * i] = add2(v.x, ee[2 * i]);
+          ee[2 * i + 1] = add2(v.y, ee[2 * i + 1]);
+        }
+      }
       st6(T, V, R, ee);
       st6(T, V + PG::VEC, R, eo);
       cpx<float> xe[2][6], xo[2][6];
