@@ -440,7 +440,7 @@ int launch_pack_links(const Geom &g, int prec, const double *canon, void *out, i
 }
 
 // canonical FP64 links -> the packed kernel's tiles (OpFields::links_full
-// where paired_links holds): [b][36][site pair] {re, re, im, im} of -U/2, one
+// where paired_links holds): [b][36][site pair] {re, re, im, im} of U times paired_scale, one
 // thread per entry of a pair of neighbouring sites (pairs fastest: whole
 // lines written)
 template <typename P> __global__ void k_pack_links_paired(Geom g, const double2 *__restrict__ canon, P *out) {
@@ -450,8 +450,9 @@ template <typename P> __global__ void k_pack_links_paired(Geom g, const double2 
   const int j = (int)(t - bi * g.Vh), b = (int)(bi / 36), i = (int)(bi - 36LL * b);
   const double2 va = canon[canonical_index(g, b, 2 * j) * 36 + i], vb = canon[canonical_index(g, b, 2 * j + 1) * 36 + i];
   P *q = out + 2 * t;
-  q[0] = to_pair<P, double>(-0.5 * va.x, -0.5 * vb.x);
-  q[1] = to_pair<P, double>(-0.5 * va.y, -0.5 * vb.y);
+  constexpr double c = paired_scale<P>();
+  q[0] = to_pair<P, double>(c * va.x, c * vb.x);
+  q[1] = to_pair<P, double>(c * va.y, c * vb.y);
 }
 
 int launch_pack_links_full(const Geom &g, int prec, const double *canon, void *out, cudaStream_t st) {

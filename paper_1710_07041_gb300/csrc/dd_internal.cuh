@@ -595,8 +595,13 @@ __device__ __forceinline__ void load_link(const void *links, const Geom &g, int 
   if constexpr (LP == 6) su3_third_row(u);
 }
 
+// What the packed tiles hold a link times: the hop's coefficient -1/2, exact in
+// FP32 and BF16 down to entries of 2^-125. FP16 is subnormal below 2^-14 = 6e-5,
+// where half of an entry loses its last bit: there -1, and the packed kernel
+// halves as it converts.
+template <typename P> constexpr float paired_scale() { return std::is_same<P, __half2>::value ? -1.f : -0.5f; }
 // Entry i (0..35) of site s in a links tile of the packed layout (see
-// OpFields::links_full; n sites): the link times -1/2 of two neighbouring
+// OpFields::links_full; n sites): the link times paired_scale of two neighbouring
 // sites interleaved {re, re, im, im}.
 __device__ __forceinline__ float real_of(float v) { return v; }
 __device__ __forceinline__ float real_of(__half v) { return __half2float(v); }
@@ -605,7 +610,8 @@ __device__ __forceinline__ double real_of(double v) { return v; }
 template <typename C, typename P> __device__ __forceinline__ cpx<C> paired_link_entry(const P *tile, int n, int i, int s) {
   using R = std::remove_const_t<std::remove_reference_t<decltype(tile->x)>>;
   const R *e = (const R *)tile + 2 * ((size_t)i * n + (s & ~1)) + (s & 1);
-  return {(C)-2 * (C)real_of(e[0]), (C)-2 * (C)real_of(e[2])};
+  constexpr C back = (C)(1 / paired_scale<P>());
+  return {back * (C)real_of(e[0]), back * (C)real_of(e[2])};
 }
 // full link mu of site (b, s) from OpFields::links_full
 template <typename S, bool PAIRED, typename C>
@@ -864,7 +870,7 @@ struct OpFields {
   // (its block solve reads each link about ten times per phase from L1 or
   // shared memory, where the rebuild would cost more issue slots than the
   // bytes it saves); the same array as `links` for FP64. Where paired_links
-  // holds: the links times -1/2 (exact), the reals of sites 2j and 2j + 1
+  // holds: the links times paired_scale, the reals of sites 2j and 2j + 1
   // interleaved {re, re, im, im} (the packed kernel's operand order)
   void *links_full = nullptr;
   void *clov = nullptr;   // A, chunked tiles of 36 pairs x Vb sites per block (clover_slot)

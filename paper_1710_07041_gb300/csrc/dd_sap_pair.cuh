@@ -30,7 +30,8 @@
 // (2 x 72 words) and its row's x-links in the orientation each half-step
 // needs (2 x 54 words): 252 of 256 columns. Two CTAs of 128 threads per SM.
 //
-// Links are stored times -1/2 (exact), the hop's coefficient.
+// The links in shared memory are times -1/2, the hop's coefficient (in the
+// operator field as paired_scale says).
 //
 // Bound and figures. A CTA lives 55000 clocks at 4 MR steps: 37000 in the half
 // steps (76% of what the register ports allow a stream of packed multiply-adds
@@ -306,7 +307,7 @@ __device__ __forceinline__ void herm6_pair(const u64 *m, const u64 *x, u64 *y) {
 // A hop (1 -+ g) W psi projected on spin h is chi = u_h + phase * d, with
 // d = d_{1-h} for x and y, d_h for z and t; its upper part adds to u, its
 // lower part, the conjugate phase times that with the hop's sign, to b (x, y)
-// or a (z, t). hv holds -1/2 W chi (links stored times -1/2).
+// or a (z, t). hv holds -1/2 W chi (the tile's links are times -1/2).
 struct PairAcc {
   u64 u[6], a[6], b[6];
 };
@@ -1067,7 +1068,8 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
 #pragma unroll
         for (int e = 0; e < 2; e++) {
           const cpx<float> a = from_pair<float, P>(p[2 * e]), c = from_pair<float, P>(p[2 * e + 1]);
-          d[e] = quad{pk(a.re, a.im), pk(c.re, c.im)};
+          constexpr float f = -0.5f / paired_scale<P>();
+          d[e] = quad{pk(f * a.re, f * a.im), pk(f * c.re, f * c.im)};
         }
       }
     }

@@ -62,3 +62,27 @@ def test_fp32_error_is_no_larger_than_the_general_kernels(block, guess, tmp_path
         e = e.mean(axis=1)
         print(f"{nmr} MR steps: packed {e[0]:.4g}, general {e[1]:.4g}")
         assert e[0] <= 1.03 * e[1], nmr
+
+
+@pytest.mark.parametrize("dims,block", [((8, 8, 8, 8), (4, 4, 4, 4)), ((16, 8, 8, 8), (8, 4, 4, 4)),
+                                        ((8, 4, 8, 8), (4, 2, 4, 4))])
+def test_fp16_keeps_small_link_entries(dims, block):
+    """Links exp(i eps lambda_1) with eps = 3 * 2^-24: FP16 holds their off-
+    diagonal entries exactly (subnormal). Colour 1 of the smoothed x then comes
+    from colour 0 of b through those entries alone, in proportion to eps. Bound:
+    a few roundings of FP16 (2^-11 each; half of an entry, rounded, is off by a
+    third)."""
+    V, eps = int(np.prod(dims)), 3 * 2.0 ** -24
+    U = np.tile(np.eye(3, dtype=np.complex128), (V, 4, 1, 1))
+    U[..., 0, 0] = U[..., 1, 1] = np.cos(eps)
+    U[..., 0, 1] = U[..., 1, 0] = 1j * np.sin(eps)
+    s = Setup(dims, block, c_sw=0.0, m0=0.0, prec=dd.F16, U=U)
+    b = 1e4 * synth.gaussian_spinor(V, 70)
+    b[..., 1:] = 0
+    fb, fx = s.lat.to_field(b, dd.F16), s.lat.new_field(dd.F16)
+    s.op.sap_smooth(fb, fx, 2, 3)
+    got, want = s.lat.from_field(fx, dd.F16), s.ref.sap(block, s.lat.from_field(fb, dd.F16), 2, 3)
+    err = relerr(got[..., 1], want[..., 1])
+    print(f"colour reached through the small entries: relerr {err:.3g}")
+    assert err <= 3e-3
+    s.close()
