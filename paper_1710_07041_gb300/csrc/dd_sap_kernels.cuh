@@ -91,14 +91,18 @@ __device__ __noinline__ void wait_expired(unsigned *timeouts, unsigned mbar, uns
 // and a column range chosen by t / 128. Allocation is per CTA (a power of two
 // of at least 32 columns); the launch keeps at most 512 / NCOLS CTAs of TMEM
 // kernels on an SM through their shared-memory size, so an allocation never
-// waits for columns.
+// waits for columns. The instructions want the whole warp together: every
+// wrapper converges it first (a lane may come out of a branch of its own, with
+// a wait in it).
 template <int NCOLS> __device__ __forceinline__ void tmem_alloc(unsigned dst_smem) {
   static_assert(NCOLS >= 32 && NCOLS <= 512 && (NCOLS & (NCOLS - 1)) == 0, "TMEM columns");
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dst_smem), "n"(NCOLS)
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
 }
 template <int NCOLS> __device__ __forceinline__ void tmem_dealloc(uint32_t taddr) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "n"(NCOLS) : "memory");
 }
 // a CTA barrier that orders the threads' tensor-memory operations around it
@@ -108,7 +112,10 @@ __device__ __forceinline__ void tmem_sync() {
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
 // the stores of this thread have landed (before the columns are read)
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() {
+  __syncwarp();
+  asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+}
 // Strided view of one block's pair tile: pair-major (the links: element
 // (i, site) at p[i * stride + site]) or chunked (the clover: see
 // clover_block_chunked, stride = sites per chunk row). PAIRED: a links tile

@@ -102,6 +102,7 @@ template <int SHAPE> struct PairGeom {
 // ---- tensor memory: N words of this thread's lane from column taddr
 template <int N> __device__ __forceinline__ void tm_st(uint32_t a, const uint32_t *u) {
   static_assert(N == 2 || N == 4 || N == 8 || N == 16 || N == 32, "tcgen05.st width");
+  __syncwarp();
   if constexpr (N == 2) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};\n" ::"r"(a), "r"(u[0]), "r"(u[1]) : "memory");
   } else if constexpr (N == 4) {
