@@ -4,9 +4,9 @@
 #pragma once
 #include <algorithm>
 #include <functional>
-#include <mutex>
 #include <string>
 
+#include "dd_device_once.cuh"
 #include "dd_tune.cuh"
 
 namespace dd {
@@ -1005,9 +1005,21 @@ inline SapPhase sap_phase(const dd_sap_params &p, int sw, int colour, bool incr)
   return f;
 }
 
+// The kernel's dynamic shared-memory limit on the current device (`once`: one
+// object per kernel).
+template <typename K> int raise_smem(K *kern, int bytes, DeviceOnce &once) {
+  int dev = 0;
+  DD_CUDA(cudaGetDevice(&dev));
+  return once.run(dev, [&] {
+    return cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes),
+                     "sap: shared-memory limit");
+  });
+}
+
+// prepare: only what has to be done ahead of a capture
 template <typename S, int STAGE, int MINB, int NT, int SHAPE, bool MULTI = false>
 int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
-          bool persistent, cudaStream_t st) {
+          bool persistent, bool prepare, cudaStream_t st) {
   if (nl > 1 && !MULTI) {
     set_error("sap: this launch variant covers one lattice");
     return DD_EINVAL;
@@ -1015,16 +1027,9 @@ int sap_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
   const Geom &g = L[0].g;   // every lattice of the launch has this block shape
   size_t smem = SapSmem<S>::bytes(g, STAGE);
   auto kern = k_sap_phase<S, STAGE, MINB, NT, SHAPE, MULTI>;
-  // raise the kernel's dynamic shared-memory limit once (never during a capture)
-  static std::mutex mu;
-  static int raised = 0;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    if (raised < (int)smem) {
-      DD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-      raised = 227 * 1024;
-    }
-  }
+  static DeviceOnce once;
+  if (int rc = raise_smem(kern, 227 * 1024, once)) return rc;
+  if (prepare) return DD_OK;
   const SapGroups G = sap_groups(L, nl, tile);
   const int nitems = G.nitems;
   int grid = nitems;

@@ -11,17 +11,17 @@ namespace {
 // 32- and 16-bit storage only without staging: the form without work fields)
 template <typename S, int STAGE, int MINB, int NT = 256>
 int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
-          bool persistent, cudaStream_t st) {
+          bool persistent, bool prepare, cudaStream_t st) {
   constexpr int SH = NT == 256 ? 1 : 2;   // the shape this thread count fits
   if (shape_of(L[0].g) == SH) {
     if constexpr (STAGE == 0 || Store<S>::prec == DD_F64)
-      return nl > 1 ? sap_k<S, STAGE, MINB, NT, SH, true>(L, nl, p, rp, ax, tile, persistent, st)
-                    : sap_k<S, STAGE, MINB, NT, SH>(L, nl, p, rp, ax, tile, persistent, st);
+      return nl > 1 ? sap_k<S, STAGE, MINB, NT, SH, true>(L, nl, p, rp, ax, tile, persistent, prepare, st)
+                    : sap_k<S, STAGE, MINB, NT, SH>(L, nl, p, rp, ax, tile, persistent, prepare, st);
     set_error("sap: no staged layout for this block shape");
     return DD_EINVAL;
   }
-  return nl > 1 ? sap_k<S, STAGE, MINB, NT, 0, true>(L, nl, p, rp, ax, tile, persistent, st)
-                : sap_k<S, STAGE, MINB, NT, 0>(L, nl, p, rp, ax, tile, persistent, st);
+  return nl > 1 ? sap_k<S, STAGE, MINB, NT, 0, true>(L, nl, p, rp, ax, tile, persistent, prepare, st)
+                : sap_k<S, STAGE, MINB, NT, 0>(L, nl, p, rp, ax, tile, persistent, prepare, st);
 }
 
 // One smoother application in the packed kernel (dd_sap_pair.cuh). From a
@@ -35,15 +35,12 @@ int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp
 // bits (dd_mg.cu).
 template <typename S, int SHAPE, bool MULTI>
 int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork &ax, int tile,
-               cudaStream_t st) {
+               bool prepare, cudaStream_t st) {
   using PG = PairGeom<SHAPE>;
   auto kern = k_sap_pair<S, SHAPE, MULTI>;
-  static std::once_flag once;   // raise the kernel's shared-memory limit (never during a capture)
-  static cudaError_t limit = cudaSuccess;
-  std::call_once(once, [&] {
-    limit = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG::SMEM);
-  });
-  DD_CUDA(limit);
+  static DeviceOnce once;
+  if (int rc = raise_smem(kern, (int)PG::SMEM, once)) return rc;
+  if (prepare) return DD_OK;
   const SapGroups G = sap_groups(L, nl, tile);
   // Each CTA requests into L2 the operator of the block that a quarter of the
   // resident CTAs ahead of it starts on (a block's start then waits for L2
@@ -99,13 +96,10 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
 // one smoother application in the FP64 small-block kernel (dd_sap_fine.cuh)
 template <bool MULTI>
 int sap_fine_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
-               cudaStream_t st) {
-  static std::once_flag once;   // 32-site blocks need a little over 48 KB (never raised during a capture)
-  static cudaError_t limit = cudaSuccess;
-  std::call_once(once, [&] {
-    limit = cudaFuncSetAttribute(k_sap_fine<MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-  });
-  DD_CUDA(limit);
+               bool prepare, cudaStream_t st) {
+  static DeviceOnce once;   // 32-site blocks need a little over 48 KB
+  if (int rc = raise_smem(k_sap_fine<MULTI>, 64 * 1024, once)) return rc;
+  if (prepare) return DD_OK;
   const SapGroups G = sap_groups(L, nl, tile);
   const AuxPtrs none{};
   for (int sw = 0; sw < p.sweeps; sw++)
@@ -170,32 +164,33 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
   }
   // variant k: layout k % nlay, RHS tile (k / nlay) % nt, persistent grid if
   // k >= nlay * nt; packed and small-block kernels: RHS tile k
-  auto run = [&](int k) {
+  auto variant = [&](int k, bool prepare) {
     if constexpr (Store<S>::prec != DD_F64) {
       if (pair) {
         if (shape_of(g) == 1)
-          return nl > 1 ? sap_pair_k<S, 1, true>(L, nl, p, rp, *ax, tiles[k], st)
-                        : sap_pair_k<S, 1, false>(L, nl, p, rp, *ax, tiles[k], st);
-        return nl > 1 ? sap_pair_k<S, 2, true>(L, nl, p, rp, *ax, tiles[k], st)
-                      : sap_pair_k<S, 2, false>(L, nl, p, rp, *ax, tiles[k], st);
+          return nl > 1 ? sap_pair_k<S, 1, true>(L, nl, p, rp, *ax, tiles[k], prepare, st)
+                        : sap_pair_k<S, 1, false>(L, nl, p, rp, *ax, tiles[k], prepare, st);
+        return nl > 1 ? sap_pair_k<S, 2, true>(L, nl, p, rp, *ax, tiles[k], prepare, st)
+                      : sap_pair_k<S, 2, false>(L, nl, p, rp, *ax, tiles[k], prepare, st);
       }
     }
     if constexpr (Store<S>::prec == DD_F64) {
       if (fine)
-        return nl > 1 ? sap_fine_k<true>(L, nl, p, rp, ax, tiles[k], st)
-                      : sap_fine_k<false>(L, nl, p, rp, ax, tiles[k], st);
+        return nl > 1 ? sap_fine_k<true>(L, nl, p, rp, ax, tiles[k], prepare, st)
+                      : sap_fine_k<false>(L, nl, p, rp, ax, tiles[k], prepare, st);
     }
     const int layout = layouts[k % nlay], tile = tiles[(k / nlay) % nt];
     const bool pers = k >= nlay * nt;
     switch (layout) {
-      case 1: return sap_t<S, 1, 2>(L, nl, p, rp, ax, tile, pers, st);
-      case 2: return sap_t<S, 0, 2>(L, nl, p, rp, ax, tile, pers, st);
-      case 3: return sap_t<S, 1, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
-      case 4: return sap_t<S, 0, 1, 512>(L, nl, p, rp, ax, tile, pers, st);
-      case 5: return sap_t<S, 2, 2>(L, nl, p, rp, ax, tile, pers, st);
-      default: return sap_t<S, 1, 1>(L, nl, p, rp, ax, tile, pers, st);
+      case 1: return sap_t<S, 1, 2>(L, nl, p, rp, ax, tile, pers, prepare, st);
+      case 2: return sap_t<S, 0, 2>(L, nl, p, rp, ax, tile, pers, prepare, st);
+      case 3: return sap_t<S, 1, 1, 512>(L, nl, p, rp, ax, tile, pers, prepare, st);
+      case 4: return sap_t<S, 0, 1, 512>(L, nl, p, rp, ax, tile, pers, prepare, st);
+      case 5: return sap_t<S, 2, 2>(L, nl, p, rp, ax, tile, pers, prepare, st);
+      default: return sap_t<S, 1, 1>(L, nl, p, rp, ax, tile, pers, prepare, st);
     }
   };
+  auto run = [&](int k) { return variant(k, false); };
   const int nvar = pair || fine ? nt : 2 * nlay * nt;
   int k = 0;
   // the tuner's key: lattice, precision, right-hand-side count, smoother
@@ -235,6 +230,8 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
     int c = tune_lookup(key);
     k = c >= 0 && c < nvar ? c : 0;
   }
+  // (the launches below may be captured: with one variant nothing has run it yet)
+  if (int rc = variant(k, true)) return rc;
   // launches of an application: the phases and, in the packed kernel, the residuals formed ahead of them
   const int nres = !pair ? 0 : !incr ? 2 * p.sweeps - (p.x_is_zero ? 1 : 0) : p.x_is_zero ? 0 : 2;
   return sap_launch_as_graph(key + shape + "|" + fields, k, 2 * p.sweeps + nres * nl, rp, ax, [&] { return run(k); },
