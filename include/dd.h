@@ -275,8 +275,12 @@ int dd_solve(dd_op_t op, const dd_solve_params *p, const double *b, double *x, i
  * restart 16) is cached when the call ends and reused by the next dd_solve
  * that needs buffers of the same sizes on the same device, which saves the
  * allocation and release (milliseconds, and a device synchronisation) per
- * call. A solve that cannot allocate releases the cache first; the cache
- * holds at most half of the device memory and 64 MB of pinned host memory;
+ * call; so is the workspace of its two-level preconditioner. The cache holds
+ * at most half of the device memory and 64 MB of pinned host memory. Besides,
+ * the work fields of dd_sap_smooth and dd_sap_smooth_multi come from a memory
+ * pool of the device that keeps up to 4 GB between calls. A call of this
+ * library that cannot allocate device memory releases all of this and tries
+ * once more (not inside a stream capture; dd_solve_noalloc allocates nothing);
  * dd_server_create releases it (the server budgets device memory itself and
  * its workers free their buffers). This call frees every cached buffer (all
  * devices), e.g. to return the memory to other users. Returns DD_OK. */

@@ -185,7 +185,7 @@ int dd_create_gauge(dd_lattice_t lat, const double *links, dd_gauge_t *out) {
   Gauge *g = new (std::nothrow) Gauge;
   if (!g) return DD_ENOMEM;
   size_t bytes = (size_t)l->g.V * 72 * sizeof(double);
-  if (cudaMalloc(&g->links_canon, bytes) != cudaSuccess) {
+  if (dev_malloc(&g->links_canon, bytes) != cudaSuccess) {
     delete g;
     set_error("dd_create_gauge: out of device memory (%zu bytes)", bytes);
     return DD_ENOMEM;
@@ -207,10 +207,10 @@ int dd_create_gauge(dd_lattice_t lat, const double *links, dd_gauge_t *out) {
 static int alloc_fields(const Geom &g, int prec, OpFields &f) {
   f.prec = prec;
   size_t pb = pair_bytes(prec);
-  if (cudaMalloc(&f.links, (size_t)g.V * 4 * link_pairs_of(prec) * pb) != cudaSuccess ||
-      (link_pairs_of(prec) != 9 && cudaMalloc(&f.links_full, (size_t)g.V * 36 * pb) != cudaSuccess) ||
-      cudaMalloc(&f.clov, (size_t)g.V * 36 * pb) != cudaSuccess ||
-      cudaMalloc(&f.cinv, (size_t)g.V / 2 * 36 * pb) != cudaSuccess) {
+  if (dev_malloc(&f.links, (size_t)g.V * 4 * link_pairs_of(prec) * pb) != cudaSuccess ||
+      (link_pairs_of(prec) != 9 && dev_malloc(&f.links_full, (size_t)g.V * 36 * pb) != cudaSuccess) ||
+      dev_malloc(&f.clov, (size_t)g.V * 36 * pb) != cudaSuccess ||
+      dev_malloc(&f.cinv, (size_t)g.V / 2 * 36 * pb) != cudaSuccess) {
     free_fields(f);
     set_error("dd_create_op: out of device memory");
     return DD_ENOMEM;
@@ -239,7 +239,7 @@ static int create_op(Gauge *ga, double c_sw, double m0, int prec, Fill fill, dd_
   if (rc == DD_OK) rc = alloc_fields(g, DD_F32, op->f32);
   if (rc == DD_OK && half_tiles(prec)) rc = alloc_fields(g, prec, op->fp);
   int *bad = nullptr;
-  if (rc == DD_OK && cudaMalloc(&bad, sizeof(int)) != cudaSuccess) rc = DD_ENOMEM;
+  if (rc == DD_OK && dev_malloc(&bad, sizeof(int)) != cudaSuccess) rc = DD_ENOMEM;
   cudaStream_t st = 0;
   if (rc == DD_OK) rc = cuda_fail(cudaMemsetAsync(bad, 0, sizeof(int), st), "memset");
   if (rc == DD_OK) rc = fill(g, (double *)op->f64.clov, (double *)op->f64.cinv, bad, st);
@@ -258,8 +258,8 @@ static int create_op(Gauge *ga, double c_sw, double m0, int prec, Fill fill, dd_
     // double-float copies of the FP64 links and site blocks (the true residual of mixed-precision solves)
     op->fdf.prec = DD_PREC_DF;
     const size_t np = (size_t)g.V * 36;
-    if (cudaMalloc(&op->fdf.links, np * sizeof(float4)) != cudaSuccess ||
-        cudaMalloc(&op->fdf.clov, np * sizeof(float4)) != cudaSuccess) {
+    if (dev_malloc(&op->fdf.links, np * sizeof(float4)) != cudaSuccess ||
+        dev_malloc(&op->fdf.clov, np * sizeof(float4)) != cudaSuccess) {
       cudaGetLastError();
       set_error("dd_create_op: out of device memory");
       rc = DD_ENOMEM;
@@ -319,7 +319,7 @@ int dd_create_op_clover(dd_gauge_t gauge, const double *clover_host, int prec, d
   }
   const size_t bytes = (size_t)ga->lat->g.V * 144 * sizeof(double);
   double *dev = nullptr;
-  if (cudaMalloc(&dev, bytes) != cudaSuccess) {
+  if (dev_malloc(&dev, bytes) != cudaSuccess) {
     cudaGetLastError();
     set_error("dd_create_op_clover: out of device memory (%zu bytes)", bytes);
     return DD_ENOMEM;
@@ -419,7 +419,7 @@ int dd_apply_D(dd_op_t opp, int prec, const void *in, void *out, int nrhs, void 
     const Geom &g = op->lat->g;
     const size_t fb = (size_t)g.V * 24 * 8, n = (size_t)g.V * 12;
     void *tmp = nullptr;   // the split input, one right-hand side at a time
-    DD_CUDA(cudaMalloc(&tmp, fb));
+    DD_CUDA(dev_malloc(&tmp, fb));
     int rc = DD_OK;
     for (int r = 0; r < nrhs && rc == DD_OK; r++) {
       rc = launch_split_pairs((const double *)((const char *)in + r * fb), tmp, n, (cudaStream_t)stream);

@@ -884,8 +884,8 @@ static int build_coarse(Mg *mg, cudaStream_t st) {
   float *u = nullptr, *wv = nullptr;
   float2 *dcf = nullptr;   // FP32 coarse operator while it is assembled
   const size_t ndc = (size_t)g.nblocks * 9 * n2 * n2;
-  DD_CUDA(cudaMalloc(&u, fs * 4));
-  if (cudaMalloc(&wv, fs * 4) != cudaSuccess || cudaMalloc(&dcf, sizeof(float2) * ndc) != cudaSuccess) {
+  DD_CUDA(dev_malloc(&u, fs * 4));
+  if (dev_malloc(&wv, fs * 4) != cudaSuccess || dev_malloc(&dcf, sizeof(float2) * ndc) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(u);
     cudaFree(wv);
@@ -920,7 +920,7 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
   const int N = mg->N;
   double *canon = nullptr, *nrm = nullptr;
   void *pin = nullptr, *pout = nullptr, *aux = nullptr;
-  DD_CUDA(cudaMalloc(&canon, fs * 8));
+  DD_CUDA(dev_malloc(&canon, fs * 8));
   int rc = DD_OK;
   Blas bl;
   int dev = 0, sms = 0;
@@ -930,15 +930,15 @@ int mg_setup(Mg *mg, const double *tv_host, cudaStream_t st) {
     cudaFree(canon);
     return rc;
   }
-  if (cudaMalloc(&nrm, sizeof(double)) != cudaSuccess) rc = DD_ENOMEM;
-  if (cudaMalloc(&pin, fs * real_bytes(op->prec)) != cudaSuccess ||
-      cudaMalloc(&pout, fs * real_bytes(op->prec)) != cudaSuccess)
+  if (dev_malloc(&nrm, sizeof(double)) != cudaSuccess) rc = DD_ENOMEM;
+  if (dev_malloc(&pin, fs * real_bytes(op->prec)) != cudaSuccess ||
+      dev_malloc(&pout, fs * real_bytes(op->prec)) != cudaSuccess)
     rc = DD_ENOMEM;
   // the smoother's work fields as in mg_enqueue; without room for them every phase forms b - D x
   const bool wide = op->prec == DD_F32 || op->prec == DD_F64;
   const size_t ab = wide ? sap_work_bytes(g, op->prec, 1) : fs * 4;
   SapWork ax;
-  if (rc == DD_OK && cudaMalloc(&aux, ab) != cudaSuccess) {
+  if (rc == DD_OK && dev_malloc(&aux, ab) != cudaSuccess) {
     cudaGetLastError();
     aux = nullptr;
   }
@@ -1022,9 +1022,9 @@ int dd_create_mg(dd_op_t opp, const dd_mg_params *p, const double *tv_host, dd_m
   mg->p = *p;
   mg->N = p->n_vectors;
   const size_t n2 = 2 * (size_t)mg->N;
-  if (cudaMalloc(&mg->V, (size_t)g.V * 24 * 4 * mg->N) != cudaSuccess ||
-      cudaMalloc(&mg->Vh, (size_t)g.V * 24 * 2 * mg->N) != cudaSuccess ||
-      cudaMalloc(&mg->Dc, sizeof(__half2) * (size_t)g.nblocks * 9 * n2 * dc_rows(mg->N)) != cudaSuccess) {
+  if (dev_malloc(&mg->V, (size_t)g.V * 24 * 4 * mg->N) != cudaSuccess ||
+      dev_malloc(&mg->Vh, (size_t)g.V * 24 * 2 * mg->N) != cudaSuccess ||
+      dev_malloc(&mg->Dc, sizeof(__half2) * (size_t)g.nblocks * 9 * n2 * dc_rows(mg->N)) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(mg->V);
     cudaFree(mg->Vh);

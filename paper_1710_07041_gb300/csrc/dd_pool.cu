@@ -6,8 +6,9 @@
 // Buffers a solver releases are kept here, keyed by (device, size), and
 // handed to the next solver that asks for the same size. The cache is
 // bounded (half the device memory, 64 MB of pinned host memory); a device
-// allocation that fails releases the cache and is tried once more, and
-// dd_release_workspace() gives everything back. Work fields of single calls
+// allocation of the library that fails (a workspace, work fields, the fields
+// of a gauge field, an operator or a multigrid object) releases the cache and
+// is tried once more, and dd_release_workspace() gives everything back. Work fields of single calls
 // (the smoother's) come from a stream-ordered memory pool per device that
 // keeps up to STREAM_KEEP bytes between calls: the device's default pool
 // gives its memory back at every synchronisation, and the next call mapped it
@@ -79,12 +80,21 @@ void *pool_dev_alloc(size_t n) {
     }
   }
   void *p = nullptr;
-  if (cudaMalloc(&p, n) == cudaSuccess) return p;
-  cudaGetLastError();
-  pool_release();   // the cached buffers may be what stands in the way
-  if (cudaMalloc(&p, n) == cudaSuccess) return p;
+  if (dev_malloc_bytes(&p, n) == cudaSuccess) return p;
   cudaGetLastError();
   return nullptr;
+}
+
+cudaError_t dev_malloc_bytes(void **p, size_t n) {
+  *p = nullptr;
+  if (cudaMalloc(p, n) == cudaSuccess) return cudaSuccess;
+  cudaGetLastError();
+  // the cached buffers may be what stands in the way (a stream's work fields
+  // count as free once the work in front of their release is done)
+  cudaDeviceSynchronize();
+  pool_release();
+  *p = nullptr;
+  return cudaMalloc(p, n);
 }
 
 void pool_dev_free(void *p, size_t n) {
@@ -136,36 +146,50 @@ void pool_host_free(void *p, size_t n) {
   cudaFreeHost(p);
 }
 
+namespace {
+// the device's stream-ordered pool, made at its first use outside a capture;
+// null: the default pool for now (another call tries again)
+cudaMemPool_t stream_pool(int d, bool capturing) {
+  StreamPools &S = stream_pools();
+  std::lock_guard<std::mutex> lk(S.mu);
+  auto it = S.of.find(d);
+  if (it != S.of.end()) return it->second;
+  if (capturing) return nullptr;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = d;
+  uint64_t keep = STREAM_KEEP;
+  cudaMemPool_t mp = nullptr;
+  if (cudaMemPoolCreate(&mp, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(mp, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaGetLastError();
+    if (mp) cudaMemPoolDestroy(mp);
+    return nullptr;
+  }
+  S.of.emplace(d, mp);
+  return mp;
+}
+}  // namespace
+
 void *pool_stream_alloc(size_t n, cudaStream_t st) {
   if (n == 0) return nullptr;
-  const int d = current_device();
-  cudaMemPool_t mp = nullptr;
-  {
-    StreamPools &S = stream_pools();
-    std::lock_guard<std::mutex> lk(S.mu);
-    auto it = S.of.find(d);
-    // not during a capture: a first call there takes the default pool
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (it == S.of.end() && (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
-      cudaGetLastError();
-    } else if (it == S.of.end()) {
-      cudaMemPoolProps props = {};
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = d;
-      uint64_t keep = STREAM_KEEP;
-      if (cudaMemPoolCreate(&mp, &props) != cudaSuccess ||
-          cudaMemPoolSetAttribute(mp, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
-        if (mp) cudaMemPoolDestroy(mp);
-        mp = nullptr;   // the device's default pool
-      }
-      it = S.of.emplace(d, mp).first;
-    }
-    if (it != S.of.end()) mp = it->second;
-  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (capturing) cudaGetLastError();
+  const cudaMemPool_t mp = stream_pool(current_device(), capturing);
   void *p = nullptr;
-  const cudaError_t e = mp ? cudaMallocFromPoolAsync(&p, n, mp, st) : cudaMallocAsync(&p, n, st);
+  auto take_n = [&] { return mp ? cudaMallocFromPoolAsync(&p, n, mp, st) : cudaMallocAsync(&p, n, st); };
+  if (take_n() == cudaSuccess) return p;
+  cudaGetLastError();
+  if (capturing) return nullptr;
+  // cached workspaces may stand in the way (their release must not disturb a
+  // capture that another thread has running)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  pool_release();
+  const cudaError_t e = take_n();
+  cudaThreadExchangeStreamCaptureMode(&mode);
   if (e == cudaSuccess) return p;
   cudaGetLastError();
   return nullptr;
@@ -184,7 +208,7 @@ size_t pool_cached_bytes() {
   std::lock_guard<std::mutex> lk(S.mu);
   auto it = S.of.find(d);
   uint64_t reserved = 0, used = 0;
-  if (it != S.of.end() && it->second &&
+  if (it != S.of.end() &&
       cudaMemPoolGetAttribute(it->second, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
       cudaMemPoolGetAttribute(it->second, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
     n += (size_t)(reserved - used);
@@ -210,13 +234,13 @@ void pool_release() {
   for (auto &e : host) cudaFreeHost(e.second);
   StreamPools &S = stream_pools();
   std::lock_guard<std::mutex> lk(S.mu);
-  for (auto &e : S.of)
-    if (e.second) cudaMemPoolTrimTo(e.second, 0);
+  for (auto &e : S.of) cudaMemPoolTrimTo(e.second, 0);
 }
 
 }  // namespace dd
 
 extern "C" int dd_release_workspace(void) {
+  cudaDeviceSynchronize();   // work fields count as free once the work in front of their release is done
   dd::pool_release();
   return DD_OK;
 }
