@@ -437,20 +437,29 @@ int dd_apply_D(dd_op_t opp, int prec, const void *in, void *out, int nrhs, void 
   return launch_dirac(op->lat->g, *f, in, out, nrhs, (cudaStream_t)stream);
 }
 
+// Work fields of the incremental colour residual, stream-ordered; where they do
+// not fit for all right-hand sides, for as many at a time as they do (the
+// results do not depend on it). Without any every phase forms b - D x.
+static int smooth(const Op *op, const dd_sap_params &p, const char *b, char *x, int nrhs, cudaStream_t st) {
+  const Geom &g = op->lat->g;
+  const size_t per = sap_work_bytes(g, op->fp.prec, p.x_is_zero), fb = (size_t)g.V * spinor_site_bytes(op->fp.prec);
+  int n = nrhs, rc = DD_OK;
+  void *aux;
+  while (!(aux = pool_stream_alloc(n * per, st)) && n > 1) n = (n + 1) / 2;
+  if (!aux) n = nrhs;
+  for (int r = 0; r < nrhs && rc == DD_OK; r += n)
+    rc = launch_sap(g, op->fp, p, b + r * fb, x + r * fb, n < nrhs - r ? n : nrhs - r, st, aux);
+  if (aux) cudaFreeAsync(aux, st);
+  return rc;
+}
+
 int dd_sap_smooth(dd_op_t opp, const dd_sap_params *p, const void *b, void *x, int nrhs, void *stream) {
   Op *op = (Op *)opp;
   if (!op || op->magic != MAGIC_OP || !p || !b || !x || b == x || nrhs < 1 || p->sweeps < 1 || p->mr_steps < 0) {
     set_error("dd_sap_smooth: bad argument");
     return DD_EINVAL;
   }
-  // work fields of the incremental colour residual, stream-ordered (without
-  // them, e.g. when this allocation fails, every phase forms b - D x)
-  cudaStream_t st = (cudaStream_t)stream;
-  const Geom &g = op->lat->g;
-  void *aux = pool_stream_alloc((size_t)nrhs * sap_work_bytes(g, op->fp.prec, p->x_is_zero), st);
-  int rc = launch_sap(g, op->fp, *p, b, x, nrhs, st, aux);
-  if (aux) cudaFreeAsync(aux, st);
-  return rc;
+  return smooth(op, *p, (const char *)b, (char *)x, nrhs, (cudaStream_t)stream);
 }
 
 int dd_sap_smooth_multi(int nops, const dd_op_t *ops, const int *nrhs, const dd_sap_params *p,
@@ -481,8 +490,13 @@ int dd_sap_smooth_multi(int nops, const dd_op_t *ops, const int *nrhs, const dd_
   // work fields of the incremental colour residual, stream-ordered
   cudaStream_t st = (cudaStream_t)stream;
   char *aux = (char *)pool_stream_alloc(aux_bytes, st);
+  if (!aux) {   // not for all at once: operator by operator
+    for (int k = 0; k < nops; k++)
+      if (int rc = smooth((const Op *)ops[k], *p, (const char *)b[k], (char *)x[k], nrhs[k], st)) return rc;
+    return DD_OK;
+  }
   SapWork ax;
-  for (int k = 0, i = 0; aux && k < nops; k++) {
+  for (int k = 0, i = 0; k < nops; k++) {
     const size_t fb = (size_t)lats[k].g.V * spinor_site_bytes(lats[k].f.prec);
     for (int r = 0; r < nrhs[k]; r++, i++) {
       ax.e[i] = aux;
@@ -491,8 +505,8 @@ int dd_sap_smooth_multi(int nops, const dd_op_t *ops, const int *nrhs, const dd_
       aux += sap_work_bytes(lats[k].g, lats[k].f.prec, p->x_is_zero);
     }
   }
-  int rc = launch_sap_lattices(lats, nops, *p, rp, st, ax.e[0] ? &ax : nullptr);
-  if (ax.e[0]) cudaFreeAsync(ax.e[0], st);
+  int rc = launch_sap_lattices(lats, nops, *p, rp, st, &ax);
+  cudaFreeAsync(ax.e[0], st);
   return rc;
 }
 

@@ -608,7 +608,6 @@ __global__ void __launch_bounds__(NT, MINB) k_sap_phase(const SapGroups G, const
   // the 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage hold their links in
   // the packed kernel's layout
   constexpr bool PAIRED = SHAPE != 0 && sizeof(C) == 4;
-  static_assert(!PAIRED || STAGE == 0, "packed links are read from global memory here");
   extern __shared__ __align__(16) unsigned char smem[];
   // every group of a launch has the same block shape (checked on the host)
   const int Vh = block_shape<SHAPE>(G.grp[0].g).Vh, Vb = block_shape<SHAPE>(G.grp[0].g).Vb;

@@ -7,19 +7,14 @@
 namespace dd {
 namespace {
 
-// the kernel specialised for the lattice's block shape when there is one (in
-// 32- and 16-bit storage only without staging: the form without work fields)
+// the kernel specialised for the lattice's block shape when there is one
 template <typename S, int STAGE, int MINB, int NT = 256>
 int sap_t(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtrs &rp, const SapWork *ax, int tile,
           bool persistent, bool prepare, cudaStream_t st) {
   constexpr int SH = NT == 256 ? 1 : 2;   // the shape this thread count fits
-  if (shape_of(L[0].g) == SH) {
-    if constexpr (STAGE == 0 || Store<S>::prec == DD_F64)
-      return nl > 1 ? sap_k<S, STAGE, MINB, NT, SH, true>(L, nl, p, rp, ax, tile, persistent, prepare, st)
-                    : sap_k<S, STAGE, MINB, NT, SH>(L, nl, p, rp, ax, tile, persistent, prepare, st);
-    set_error("sap: no staged layout for this block shape");
-    return DD_EINVAL;
-  }
+  if (shape_of(L[0].g) == SH)
+    return nl > 1 ? sap_k<S, STAGE, MINB, NT, SH, true>(L, nl, p, rp, ax, tile, persistent, prepare, st)
+                  : sap_k<S, STAGE, MINB, NT, SH>(L, nl, p, rp, ax, tile, persistent, prepare, st);
   return nl > 1 ? sap_k<S, STAGE, MINB, NT, 0, true>(L, nl, p, rp, ax, tile, persistent, prepare, st)
                 : sap_k<S, STAGE, MINB, NT, 0>(L, nl, p, rp, ax, tile, persistent, prepare, st);
 }
@@ -114,9 +109,11 @@ int sap_fine_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
 
 // Launch variants. The 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage run
 // in the packed kernel, whatever the lattice size and right-hand-side count (it
-// won from 32 to 8192 blocks: 24.3 -> 19.5 us per phase on 16x8^3, 0.514 -> 0.374
-// ms on 64x32^3); only a call without work fields (or DD_SAP_INCR=0) takes the unstaged
-// general kernel there. FP64 blocks of 16 and 32 sites (a warp or less of
+// won from 32 to 8192 blocks: 24.3 -> 19.9 us per phase on 16x8^3, 0.514 -> 0.381
+// ms on 64x32^3); only a call without work fields (or DD_SAP_INCR=0) takes the
+// general kernel there, whose layouts read the packed links one real at a time
+// (four sweeps without work fields, unstaged alone -> the layouts below: FP32
+// 16x8^3 273 -> 224 us, 64x32^3 5.52 -> 5.51 ms, FP16 5.47 -> 4.85 ms). FP64 blocks of 16 and 32 sites (a warp or less of
 // the general kernel's threads) run in the small-block kernel: 340 -> 43 us per
 // phase on 4^4 (blocks of 256 sites fill the general kernel's warps). Everything else runs in the general kernel:
 // tiles staged in shared memory with one CTA per SM; tiles staged with two
@@ -143,9 +140,7 @@ int sap_variants(const SapLattice *L, int nl, const dd_sap_params &p, const RhsP
     return DD_EINVAL;
   }
   int layouts[4], nlay = 0;
-  if (paired) {
-    layouts[nlay++] = g.Vb > 256 ? 4 : 2;
-  } else if (g.Vb > 256) {
+  if (g.Vb > 256) {
     // 512-site blocks (e.g. 8 x 4^3): 512 threads, one CTA per SM
     layouts[nlay++] = stage1 ? 3 : 4;
   } else {

@@ -1,7 +1,8 @@
 """Memory that the library keeps between calls is given back where an
 allocation needs it: the set-up of an operator beside kept work fields, and the
 work fields of a smoother call beside a kept solver workspace (without them the
-call takes the general kernel, whose bits differ).
+call takes the general kernel, whose bits differ). Where the work fields do not
+fit for all right-hand sides the call takes as many at a time as they do for.
 
 Other memory of the device is taken by a filler, all but MARGIN bytes."""
 import numpy as np
@@ -74,6 +75,35 @@ def test_work_fields_take_back_a_kept_workspace():
     try:
         op.sap_smooth(b, y, 2, 3, nrhs=n)
         torch.cuda.synchronize()
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    assert torch.equal(x, y)
+    op.close()
+
+
+@pytest.mark.parametrize("guess", [False, True])
+@pytest.mark.parametrize("several", [False, True])
+def test_work_fields_for_some_right_hand_sides_at_a_time(guess, several):
+    assert dd.lib().dd_release_workspace() == 0
+    lat, op = small_op()
+    n = 64   # work fields: 64 x 25 MB, from a given x 64 x 38 MB
+    b = lat.to_field(np.stack([synth.gaussian_spinor(lat.V, 82)] * n), dd.F32)
+    x, y = lat.new_field(dd.F32, n), lat.new_field(dd.F32, n)
+
+    def smooth(x):
+        if several:
+            h = b.numel() // 2
+            dd.sap_smooth_multi([(op, b[:h], x[:h], n // 2), (op, b[h:], x[h:], n // 2)], 2, 3, x_is_zero=not guess)
+        else:
+            op.sap_smooth(b, x, 2, 3, nrhs=n, x_is_zero=not guess)
+        torch.cuda.synchronize()
+
+    smooth(x)
+    assert dd.lib().dd_release_workspace() == 0
+    held = fill()
+    try:
+        smooth(y)
     finally:
         del held
         torch.cuda.empty_cache()
