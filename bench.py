@@ -73,14 +73,22 @@ def fp32_alu_peak_tflops(sm_mhz, sms):
     return sms * 128 * 2 * sm_mhz * 1e6 / 1e12
 
 
-def kernel_traffic(kernel):
+def sap_kernel(block, prec_name):
+    """The Schwarz kernel that runs for a block shape (T, Z, Y, X) and storage."""
+    if prec_name == "f64":
+        return "k_sap_fine" if int(np.prod(block)) in (16, 32) else "k_sap_phase"
+    return "k_sap_pair" if tuple(block) in ((4, 4, 4, 4), (8, 4, 4, 4)) else "k_sap_phase"
+
+
+def kernel_traffic(kernel, **case):
     """Per-launch DRAM bytes from the committed ncu summary, only while the
-    kernel's source is unchanged since the capture."""
+    kernel's source is unchanged since the capture, and only for the case they
+    were captured for and scaled to (storage, block, sites per launch)."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
     d = json.load(open(p)).get(kernel)
-    if not d:
+    if not d or any(d.get("case", {}).get(k) != v for k, v in case.items()):
         return None
     h = hashlib.sha256()
     for src in d["sources"]:
@@ -444,16 +452,18 @@ def run_ours(args, rank, world):
     sap_tflops = sap_flops_launch / (sap_launch_ms * 1e-3) / 1e12
     sap_bytes_launch = SAP_REALS_PER_SWEEP * real_b[prec] * V / 2
     mean_info = {k: float(np.mean([i[k] for i in infos])) for k in ("ms_sap", "ms_dirac", "ms_orth", "ms_total")}
-    roofline_sap = {"kernel": "k_sap_pair", "bound": "alu", "achieved": sap_tflops, "peak": alu_peak,
+    kernel = sap_kernel(wl["block"], args.prec)
+    roofline_sap = {"kernel": kernel, "bound": "alu", "achieved": sap_tflops, "peak": alu_peak,
                     "unit": "TFLOP/s", "frac": sap_tflops / alu_peak,
-                    "traffic": kernel_traffic("k_sap_pair"),
+                    "traffic": kernel_traffic(kernel, storage=args.prec, block=list(wl["block"]), sites=V // 2),
                     "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 x {peaks['sm_max_mhz']:.0f} MHz",
                     "algorithmic_bytes_per_launch": sap_bytes_launch,
                     "hbm_frac": sap_bytes_launch / (sap_launch_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                     "ms_per_launch": sap_launch_ms}
     roofline_dslash = {"kernel": "k_dirac<float>", "bound": "hbm", "achieved": dslash_gbs,
                        "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": dslash_gbs / peaks["hbm_gbs"],
-                       "traffic": kernel_traffic("k_dirac<float>"), "peak_source": peaks["src"],
+                       "traffic": kernel_traffic("k_dirac<float>", block=list(wl["block"]), sites=V),
+                       "peak_source": peaks["src"],
                        "ms_per_launch": dslash_ms}
     dominant = roofline_sap if mean_info["ms_sap"] >= mean_info["ms_dirac"] else roofline_dslash
     out = {
