@@ -163,16 +163,19 @@ __global__ void k_update_x(Geom g, double *x, const void *Z, size_t zbytes, int 
 
 struct df { float h, l; };
 
+// Every operation is rounded as written (the _rn forms are never contracted):
+// the transformations are error-free, and all instances of a kernel, whatever
+// their KMAX, give the same bits.
 // s += a * b   (a, b double-float; lazy accumulation: error terms collected in s.l)
 __device__ __forceinline__ void df_mac(df &s, float ah, float al, float bh, float bl) {
-  float p = ah * bh;
-  float pe = fmaf(ah, bh, -p);                  // exact error of the product
-  float c = fmaf(ah, bl, al * bh);              // cross terms
-  float t = s.h + p;                            // TwoSum(s.h, p)
-  float z = t - s.h;
-  float e = (s.h - (t - z)) + (p - z);
+  const float p = __fmul_rn(ah, bh);
+  const float pe = __fmaf_rn(ah, bh, -p);                  // exact error of the product
+  const float c = __fmaf_rn(ah, bl, __fmul_rn(al, bh));    // cross terms
+  const float t = __fadd_rn(s.h, p);                       // TwoSum(s.h, p)
+  const float z = __fsub_rn(t, s.h);
+  const float e = __fadd_rn(__fsub_rn(s.h, __fsub_rn(t, z)), __fsub_rn(p, z));
   s.h = t;
-  s.l += e + pe + c;
+  s.l = __fadd_rn(s.l, __fadd_rn(__fadd_rn(e, pe), c));
 }
 // s -= a * b
 __device__ __forceinline__ void df_msub(df &s, float ah, float al, float bh, float bl) {
@@ -180,14 +183,14 @@ __device__ __forceinline__ void df_msub(df &s, float ah, float al, float bh, flo
 }
 __device__ __forceinline__ double df_val(const df &s) { return (double)s.h + (double)s.l; }
 __device__ __forceinline__ df df_norm(float h, float l) {
-  float t = h + l;
-  return {t, l - (t - h)};
+  const float t = __fadd_rn(h, l);
+  return {t, __fsub_rn(l, __fsub_rn(t, h))};
 }
 __device__ __forceinline__ df df_add(df a, df b) {
-  float t = a.h + b.h;
-  float z = t - a.h;
-  float e = (a.h - (t - z)) + (b.h - z);
-  return {t, a.l + b.l + e};
+  const float t = __fadd_rn(a.h, b.h);
+  const float z = __fsub_rn(t, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(t, z)), __fsub_rn(b.h, z));
+  return {t, __fadd_rn(__fadd_rn(a.l, b.l), e)};
 }
 
 // Block-reduce NV double-float values: warp shuffles in DF, then the warp
@@ -231,7 +234,9 @@ __device__ __forceinline__ float4 w_at(const float4 *w, const float *w32, size_t
 
 // Right-hand sides of one launch (grid.y): the vectors, coefficients and
 // outputs of each. A slot's sums depend on its own vectors and the fixed
-// grid.x only, so it gets the same bits alone and in any batch.
+// grid.x only, and no rounding on the instance that runs (a slot with few
+// vectors beside one with more takes the larger KMAX; see df_mac), so it gets
+// the same bits alone and in any batch.
 constexpr int DF_BATCH = 16;
 struct DfBatch {
   DfSlot s[DF_BATCH];
