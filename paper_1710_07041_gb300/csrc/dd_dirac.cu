@@ -229,9 +229,10 @@ int dirac_v(const Geom &g, const OpFields &f, const RhsPtrs &p, cudaStream_t st)
 
 // FP64 on small lattices: twelve threads per site (see dd_fine.cuh), 16 sites
 // per CTA (of one right-hand side; every block holds a multiple of 16). One or
-// two threads a site leave most of the chip's 608 FP64 units idle here and take
-// the length of one thread's chain, ~1130 instructions of 64 clocks: 40.5 us on
-// 4^4 as on 16 x 8^3. A thread of this kernel runs ~115: 8.1 us on 4^4.
+// two threads a site leave most of the chip's 608 SM sub-partitions (each half
+// an FP64 lane per clock) idle here and take the length of one thread's chain,
+// ~1130 instructions of 64 clocks: 40.5 us on 4^4 as on 16 x 8^3. A thread of
+// this kernel runs ~115: 8.1 us on 4^4.
 constexpr int FINE_SITES = 16;
 __global__ void __launch_bounds__(12 * FINE_SITES) k_dirac_fine(Geom g, const double2 *__restrict__ links,
                                                                const double2 *__restrict__ clov, const RhsPtrs rp) {

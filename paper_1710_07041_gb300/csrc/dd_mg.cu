@@ -278,13 +278,15 @@ static inline void coarse_shape(int N, int *R, int *Q) {
 // sums are added in shared memory in a fixed order. With NPRE > 0 a thread
 // issues all its (at most NPRE) chunk loads before gathering x, so the
 // operator stream overlaps the gather. A CTA is one chain (loads, product, sum
-// over the groups), so what counts is how many of them are resident: NPRE = 9,
-// the chunks per thread of N = 16, fits four per SM, 12 three (on 48 x 24^3,
-// 95 MB, an application of kmax = 24 steps then takes 80 us longer). Loads
+// over the groups), so what counts is how many of them are resident: four per SM
+// wherever the chunks' registers allow it without spills, up to 9 of them (12
+// would spill 40 bytes; 4 need no bound). 48 x 24^3, an application alone, three
+// CTAs per SM -> four: N = 12 18.5 -> 16.4 us, N = 14 18.6 -> 17.4 us; a solve
+// 107.6 -> 105.0 and 101.8 -> 98.8 ms; N = 16 (95 MB) 85.3 -> 82.9 ms. Loads
 // ahead of grid_wait, or that keep their lines in L2, made it longer as well
 // (by 70 and 40 us). With vnext != null the CTA also stores its own part of s x
 // there (the next Krylov basis vector).
-constexpr int coarse_ctas(int npre) { return npre == 9 ? 4 : 1; }
+constexpr int coarse_ctas(int npre) { return npre > 0 && npre <= 9 ? 4 : 1; }
 template <int NPRE>
 __global__ void __launch_bounds__(256, coarse_ctas(NPRE))
     k_coarse_apply(Geom g, const __half2 *__restrict__ Dc, int N, int R, int Q, const float2 *x, float2 *y,

@@ -993,7 +993,9 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
     bulk_g2s(V, (const char *)ax.e[r] + (size_t)b * FB, FB, fbar);
   };
   // The next phase's CTAs may start as soon as every CTA of this one has: up to
-  // grid_wait they touch the operator only, which no phase writes.
+  // grid_wait they touch the operator only, which no phase writes. (Threads 0
+  // and 32 wait below, so the CTA as a whole gets past tmem_sync only once the
+  // phase before is complete.)
   grid_launch_dependents();
   // one thread of each warp asks for what comes later
   if (threadIdx.x == 0) {

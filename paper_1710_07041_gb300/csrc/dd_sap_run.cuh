@@ -76,10 +76,12 @@ int sap_pair_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
       // e is read by the next phase, unless this is the last or that forms b - D x
       if (incr && !(sw == p.sweeps - 1 && colour == 1) && !(given && colour == 0)) mode |= SAP_WRITE_E;
       if (incr && sw + 1 < p.sweeps) mode |= SAP_WRITE_R;   // r by this colour's next one
-      // programmatic launch: a phase's CTAs stage their operator tiles while
-      // the phase before drains, and wait for it (griddepcontrol.wait) before
-      // they read what it wrote (64x32^3: 0.388 -> 0.374 ms per phase; 16x8^3:
-      // 23.1 -> 20.3 us)
+      // programmatic launch: while the phase before drains a phase's CTAs start,
+      // load their clover blocks, ask for the links (a bulk copy in FP32) and
+      // for a later block's operator; at the CTA barrier in front of the
+      // tensor-memory stores they wait for it (griddepcontrol.wait in the threads
+      // that fetch what it wrote), so the rest of the staging does not overlap
+      // (64x32^3: 0.388 -> 0.374 ms per phase; 16x8^3: 23.1 -> 20.3 us)
       DD_CUDA(launch_ahead(true, kern, dim3((unsigned)G.nitems), dim3(PG::NT), PG::SMEM, st, G, given ? from_r0 : rp,
                            (const AuxPtrs &)ax, colour, (int)(p.x_is_zero && sw == 0), mode, (int)p.mr_steps, tile,
                            ahead, sap_timeout_counter()));
