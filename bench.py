@@ -442,7 +442,7 @@ def run_ours(args, rank, world):
     e2e_s = max_over_ranks((time.perf_counter() - t0) / max(1, args.steps // 2), dist)
 
     peaks = measured_peaks()
-    real_b = {dd.F64: 8, dd.F32: 4, dd.F16: 2, dd.BF16: 2}
+    real_b = {dd.F64: 8, dd.F32: 4, dd.F16: 2, dd.BF16: 2, dd.F16N: 2}
     dslash_bytes = DSLASH_REALS_12 * 4 * V
     dslash_gbs = dslash_bytes / (dslash_ms * 1e-3) / 1e9
     clocks = clk.summary()
