@@ -33,13 +33,14 @@
 // The links in shared memory are times -1/2, the hop's coefficient (in the
 // operator field as paired_scale says).
 //
-// Bound and figures. A CTA lives 55000 clocks at 4 MR steps: 37000 in the half
-// steps (76% of what the register ports allow a stream of packed multiply-adds
-// with three distinct operands), 6100 receiving flux, 5000 sending it, the rest
-// staging. Per phase, general kernel (clover blocks in tensor memory, one site
-// pair per two threads) -> this one: 64x32^3 FP32 0.514 -> 0.374 ms; FP16 48x24^3
-// with 12 right-hand sides 1.62 -> 1.28 ms; 16x8^3 FP32, where it is the latency
-// of one block, 24.3 -> 19.5 us.
+// Bound and figures (profiles/k_sap_pair_clocks.md). A CTA of FP32 64x32^3 lives
+// 55000 clocks at 4 MR steps: 37000 in the half-steps (three quarters of what the
+// register ports allow a stream of packed multiply-adds with three distinct
+// operands), 5500 taking in residual and flux, 4700 sending the flux, 1700 on x,
+// the rest staging. Per phase, general kernel (clover blocks in tensor memory,
+// one site pair per two threads) -> this one: 64x32^3 FP32 0.514 -> 0.370 ms; FP16
+// 48x24^3 with 12 right-hand sides 1.62 -> 1.26 ms; 16x8^3 FP32, where it is the
+// latency of one block, 24.3 -> 19.5 us.
 #pragma once
 #include "dd_sap_kernels.cuh"
 
@@ -277,29 +278,46 @@ __device__ __forceinline__ void su3_one(const float *W, const float *c, float *h
 }
 
 // y = M x for the packed Hermitian block of both sites (36 packed reals in the
-// order of herm6_mv)
-__device__ __forceinline__ void herm6_pair(const u64 *m, const u64 *x, u64 *y) {
+// order of herm6_mv). LAST: the diagonal term, the largest by far, is added when
+// the row's others are summed, so that one rounding has its size and not ten. In
+// FP32 storage this more than pays for the even sites' correction being summed
+// over the MR steps (errors against 64 bits, 16x8^3, 1 to 4 sweeps of 2 to 5 steps:
+// 1.24..1.43e-7 general kernel, 1.27..1.55e-7 here with the diagonal first,
+// 0.90..1.22e-7 last; a phase on 64x32^3 0.372 and 0.370 ms); in 16-bit storage,
+// where the fields' rounding hides it, it would cost 3% (the MR loop's registers).
+template <bool LAST> __device__ __forceinline__ void herm6_pair(const u64 *m, const u64 *x, u64 *y) {
   u64 n[12];
 #pragma unroll
   for (int i = 0; i < 12; i++) n[i] = neg2(x[i]);
+  auto diag = [&](int i) {
+    y[2 * i] = fma2(m[i], x[2 * i], y[2 * i]);
+    y[2 * i + 1] = fma2(m[i], x[2 * i + 1], y[2 * i + 1]);
+  };
+  if constexpr (!LAST) {
 #pragma unroll
-  for (int i = 0; i < 6; i++) {
-    y[2 * i] = mul2(m[i], x[2 * i]);
-    y[2 * i + 1] = mul2(m[i], x[2 * i + 1]);
+    for (int i = 0; i < 6; i++) {
+      y[2 * i] = mul2(m[i], x[2 * i]);
+      y[2 * i + 1] = mul2(m[i], x[2 * i + 1]);
+    }
   }
 #pragma unroll
   for (int i = 0; i < 6; i++)
 #pragma unroll
     for (int j = i + 1; j < 6; j++) {
       const u64 ar = m[2 * herm_off(i, j)], ai = m[2 * herm_off(i, j) + 1];
-      y[2 * i] = fma2(ar, x[2 * j], y[2 * i]);
-      y[2 * i + 1] = fma2(ar, x[2 * j + 1], y[2 * i + 1]);
-      y[2 * j] = fma2(ar, x[2 * i], y[2 * j]);
-      y[2 * j + 1] = fma2(ar, x[2 * i + 1], y[2 * j + 1]);
+      const bool fi = LAST && i == 0 && j == 1, fj = LAST && i == 0;   // the first term of row i, of row j
+      y[2 * i] = fi ? mul2(ar, x[2 * j]) : fma2(ar, x[2 * j], y[2 * i]);
+      y[2 * i + 1] = fi ? mul2(ar, x[2 * j + 1]) : fma2(ar, x[2 * j + 1], y[2 * i + 1]);
+      y[2 * j] = fj ? mul2(ar, x[2 * i]) : fma2(ar, x[2 * i], y[2 * j]);
+      y[2 * j + 1] = fj ? mul2(ar, x[2 * i + 1]) : fma2(ar, x[2 * i + 1], y[2 * j + 1]);
       y[2 * i] = fma2(ai, n[2 * j + 1], y[2 * i]);
       y[2 * i + 1] = fma2(ai, x[2 * j], y[2 * i + 1]);
       y[2 * j] = fma2(ai, x[2 * i + 1], y[2 * j]);
       y[2 * j + 1] = fma2(ai, n[2 * i], y[2 * j + 1]);
+      if (LAST && j == 5) {   // row i is complete but for its diagonal, with i = 4 row 5 too
+        diag(i);
+        if (i == 4) diag(5);
+      }
     }
 }
 
@@ -361,8 +379,6 @@ __device__ __forceinline__ void proj_si(const u64 *u, const u64 *d, u64 s, u64 n
 __device__ __forceinline__ int slot(int s, int r) { return r ^ (((s ^ (s >> 1)) & 1) << 2); }
 // first colour of spin s at row r
 __device__ __forceinline__ int spin_at(int rows, int s, int r) { return 3 * s * rows + slot(s, r); }
-
-__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 // What a thread knows about its row: neighbours in the block, signs
 struct PairThread {
@@ -974,8 +990,7 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
   constexpr unsigned SB = (unsigned)spinor_site_bytes(Store<S>::prec);
   constexpr unsigned RQ = QuadStore<S, true>::bytes, RB = 6 * NT * RQ;   // stored residual of a block
   constexpr unsigned FB = Flux<SHAPE>::total * sizeof(P);
-  constexpr bool APART = Store<S>::prec == DD_F32;   // how e is summed, see the MR loop
-  static_assert(!APART || 12u * NT * 8 <= FB, "step 0's te fits the block's flux");
+  constexpr bool LAST = Store<S>::prec == DD_F32;   // order of the site blocks' sums, see herm6_pair
 
   // this thread's clover blocks: chirality h of the even and the odd pair, both
   // sites' chunks (neighbours in memory) in one 32-byte load
@@ -1178,13 +1193,7 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
       //     D_oe te, alpha = <p, rho> / <p, p>, e_o += alpha rho, rho -= alpha p
       //   reconstruction: e_e = A_ee^-1 (r_e - D_eo e_o) with e_o = sum_k alpha_k
       //     rho_k is step 0's te minus sum_k alpha_k (step k's te): the steps
-      //     accumulate it, and no half-step is spent on D_eo e_o. In FP32
-      //     storage this must not be less exact than that half-step was: there
-      //     the products are rounded apart from the sums, and the sum over k
-      //     is kept apart from step 0's te, which waits where the block's
-      //     incoming flux was (errors against 64 bits, 16x8^3, 1 to 4 sweeps of
-      //     2 to 5 steps: 1.24..1.44e-7 with the half-step, 1.27..1.55e-7
-      //     accumulated on te, 1.23..1.42e-7 so; 64x32^3: 2.97 -> 3.05 ms).
+      //     accumulate it, and no half-step is spent on D_eo e_o.
       u64 rh[12], eo[12], ee[12];
       uint32_t cl[72], xl[54];
       {
@@ -1193,15 +1202,8 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
         tm_wait72(cl);
 #pragma unroll
         for (int i = 0; i < 36; i++) m[i] = word2(cl, i);
-        herm6_pair(m, r_e, ee);
+        herm6_pair<LAST>(m, r_e, ee);
         st6(T, V, R, ee);
-      }
-      char *const te0 = (char *)ax.e[r] + (size_t)b * FB;   // FP32: step 0's te
-      if constexpr (APART) {
-#pragma unroll
-        for (int i = 0; i < 6; i++) quad_st<S, true>(te0, i * NT + threadIdx.x, ee[2 * i], ee[2 * i + 1]);
-#pragma unroll
-        for (int i = 0; i < 12; i++) ee[i] = 0ull;
       }
 #pragma unroll
       for (int i = 0; i < 12; i++) {
@@ -1228,7 +1230,7 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
             for (int i = 0; i < 12; i++) rh[i] = sub2(rh[i], hv[i]);
           } else {
             u64 w[12];
-            herm6_pair(m, rh, w);
+            herm6_pair<LAST>(m, rh, w);
             u64 a = 0ull, c = 0ull, e = 0ull;
 #pragma unroll
             for (int i = 0; i < 12; i++) w[i] = sub2(w[i], hv[i]);
@@ -1242,9 +1244,6 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
               e = fma2(w[2 * i + 1], w[2 * i + 1], e);
             }
             float pr = lo(a) + hi(a), pi = lo(c) + hi(c), pp = lo(e) + hi(e);
-            if (APART && step == last)
-#pragma unroll
-              for (int i = 0; i < 6; i++) prefetch_l1(te0 + (size_t)(i * NT + threadIdx.x) * 16);
             cta_sum3<NT / 32>(pr, pi, pp, red);
             float ar = 0.f, ai = 0.f;
             if (pp > 0.f) {
@@ -1256,17 +1255,10 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
             ld6(T, V, R, te);
 #pragma unroll
             for (int i = 0; i < 6; i++) {
-              if constexpr (APART) {
-                eo[2 * i] = add2(eo[2 * i], fma2(Ar, rh[2 * i], mul2(neg2(Ai), rh[2 * i + 1])));
-                eo[2 * i + 1] = add2(eo[2 * i + 1], fma2(Ar, rh[2 * i + 1], mul2(Ai, rh[2 * i])));
-                ee[2 * i] = sub2(ee[2 * i], fma2(Ar, te[2 * i], mul2(neg2(Ai), te[2 * i + 1])));
-                ee[2 * i + 1] = sub2(ee[2 * i + 1], fma2(Ar, te[2 * i + 1], mul2(Ai, te[2 * i])));
-              } else {
-                eo[2 * i] = fma2(Ar, rh[2 * i], fma2(neg2(Ai), rh[2 * i + 1], eo[2 * i]));
-                eo[2 * i + 1] = fma2(Ar, rh[2 * i + 1], fma2(Ai, rh[2 * i], eo[2 * i + 1]));
-                ee[2 * i] = fma2(neg2(Ar), te[2 * i], fma2(Ai, te[2 * i + 1], ee[2 * i]));
-                ee[2 * i + 1] = fma2(neg2(Ar), te[2 * i + 1], fma2(neg2(Ai), te[2 * i], ee[2 * i + 1]));
-              }
+              eo[2 * i] = fma2(Ar, rh[2 * i], fma2(neg2(Ai), rh[2 * i + 1], eo[2 * i]));
+              eo[2 * i + 1] = fma2(Ar, rh[2 * i + 1], fma2(Ai, rh[2 * i], eo[2 * i + 1]));
+              ee[2 * i] = fma2(neg2(Ar), te[2 * i], fma2(Ai, te[2 * i + 1], ee[2 * i]));
+              ee[2 * i + 1] = fma2(neg2(Ar), te[2 * i + 1], fma2(neg2(Ai), te[2 * i], ee[2 * i + 1]));
               rh[2 * i] = fma2(neg2(Ar), w[2 * i], fma2(Ai, w[2 * i + 1], rh[2 * i]));
               rh[2 * i + 1] = fma2(neg2(Ar), w[2 * i + 1], fma2(neg2(Ai), w[2 * i], rh[2 * i + 1]));
             }
@@ -1274,7 +1266,7 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
           if (step < last) st6(T, V + PG::VEC, R, rh);
         } else {
           u64 te[12];
-          herm6_pair(m, hv, te);
+          herm6_pair<LAST>(m, hv, te);
           st6(T, V, R, te);
         }
       }
@@ -1282,14 +1274,6 @@ __global__ void __launch_bounds__(PairGeom<SHAPE>::NT, SHAPE == 1 ? 2 : 1)
       // is read ahead of the flux, whose arithmetic covers the wait)
       // (every thread is past its last hops at the sum's barrier; without MR steps there was none)
       if (nmr == 0) __syncthreads();
-      if constexpr (APART) {
-#pragma unroll
-        for (int i = 0; i < 6; i++) {
-          const quad v = quad_of<S, true>(quad_raw<S, true>(te0, i * NT + threadIdx.x));
-          ee[2 * i] = add2(v.x, ee[2 * i]);
-          ee[2 * i + 1] = add2(v.y, ee[2 * i + 1]);
-        }
-      }
       st6(T, V, R, ee);
       st6(T, V + PG::VEC, R, eo);
       cpx<float> xe[2][6], xo[2][6];

@@ -111,7 +111,7 @@ int sap_fine_k(const SapLattice *L, int nl, const dd_sap_params &p, const RhsPtr
 
 // Launch variants. The 4^4 and 8 x 4^3 blocks in 32- and 16-bit storage run
 // in the packed kernel, whatever the lattice size and right-hand-side count (it
-// won from 32 to 8192 blocks: 24.3 -> 19.9 us per phase on 16x8^3, 0.514 -> 0.381
+// won from 32 to 8192 blocks: 24.3 -> 19.5 us per phase on 16x8^3, 0.514 -> 0.370
 // ms on 64x32^3); only a call without work fields (or DD_SAP_INCR=0) takes the
 // general kernel there, whose layouts read the packed links one real at a time
 // (four sweeps without work fields, unstaged alone -> the layouts below: FP32
