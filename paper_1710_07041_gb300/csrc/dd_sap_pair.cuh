@@ -34,9 +34,9 @@
 // operator field as paired_scale says).
 //
 // Bound and figures (profiles/k_sap_pair_clocks.md). A CTA of FP32 64x32^3 lives
-// 55000 clocks at 4 MR steps: 37000 in the half-steps (three quarters of what the
+// 55400 clocks at 4 MR steps: 37800 in the half-steps (three quarters of what the
 // register ports allow a stream of packed multiply-adds with three distinct
-// operands), 5500 taking in residual and flux, 4700 sending the flux, 1700 on x,
+// operands), 5400 taking in residual and flux, 4800 sending the flux, 1500 on x,
 // the rest staging. Per phase, general kernel (clover blocks in tensor memory,
 // one site pair per two threads) -> this one: 64x32^3 FP32 0.514 -> 0.370 ms; FP16
 // 48x24^3 with 12 right-hand sides 1.62 -> 1.26 ms; 16x8^3 FP32, where it is the
